@@ -55,6 +55,9 @@ struct SysParams {
   float rc2f;        // rc^2 as float (FP32 force cutoff)
   float c2f;         // c2 as float
   double skin;       // list margin (validity rule 2 d_max >= skin)
+  long long Lfix;    // L in fixed-point pair units (2^-60, modulo 2^64)
+  long long rc2fix;  // rc^2 in units of 2^-56
+  long long c2fix;   // c2 / 3 in units of 2^-56, plus kFixBias
   double disp_thr;   // FP32-force form: threshold of the squared fixed-point displacement
   float rlf;         // rc + skin as float
   float csf;         // cell side L / nc as float
@@ -71,6 +74,7 @@ struct SysParams {
   int32_t active;    // 1 if the system takes part in the current launches
   int32_t rule;      // list validity: 0 displacement (2 d_max >= skin), 1 velocity bound (DUTC)
   int32_t half;      // 1: half list (each pair once, in its lower slot's list; Newton's third law)
+  int32_t fixed;     // 1: the FP64 form's pair arithmetic runs in 64-bit fixed point (rc <= kFixMaxRc)
 };
 
 // Per-system status words written by kernels and read by the host.
@@ -113,6 +117,7 @@ struct DevArrays {
   double4_32a* f;         // stored forces (double); half list: the own-list sums of the step
   double4_32a* facc;      // half list: forces added by the partners' threads (atomics), zeroed on use
   int4* xq[2];        // fixed-point shadow positions (uint32 per axis, wraps at L)
+  longlong4_32a* xl[2];  // FP64 form: positions in fixed-point pair units (2^-60, modulo 2^64)
   int32_t* id;        // caller index of each slot, -1 for padding
   int32_t* cell;      // cell of each slot (valid after binning)
   int32_t* ncnt;      // list length of each slot

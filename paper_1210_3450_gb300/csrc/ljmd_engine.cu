@@ -8,6 +8,7 @@
 #include <string>
 
 #include "ljmd_engine.h"
+#include "ljmd_fixed.cuh"
 
 namespace ljmd {
 
@@ -72,6 +73,14 @@ int cells_per_axis(double L, double rl) {
   int nc = (int)std::floor(L / rl);
   if (nc >= 1 && L / nc < rl * (1.0 + 1e-9)) nc -= 1;
   return nc >= 3 ? nc : 1;
+}
+
+// x >= 2^-8 in fixed-point pair units (2^-60, modulo 2^64), exact.
+long long host_to_fix(double x) {
+  int e = 0;
+  const unsigned long long m = (unsigned long long)std::ldexp(std::frexp(x, &e), 53);  // x = m 2^(e - 53)
+  const int sh = e - 53 + 60;
+  return (long long)(sh >= 64 ? 0ull : sh >= 0 ? m << sh : m >> -sh);
 }
 
 int initial_kmax(const SysSpec& s, double rl) {
@@ -286,7 +295,7 @@ int footprint(const SysSpec& s, SysFootprint* f, SysHost* h) {
 // ------------------------------------------------------------- arena
 
 void Engine::free_all() {
-  for (int b = 0; b < 2; ++b) { dfree(d_.x[b]); dfree(d_.xq[b]); }
+  for (int b = 0; b < 2; ++b) { dfree(d_.x[b]); dfree(d_.xq[b]); dfree(d_.xl[b]); }
   dfree(d_.v); dfree(d_.xref); dfree(d_.xqref); dfree(d_.f); dfree(d_.facc); dfree(d_.id); dfree(d_.cell); dfree(d_.ncnt);
   dfree(d_.nbr); dfree(d_.tile_obs); dfree(d_.skey); dfree(d_.xf); dfree(d_.vtmp); dfree(d_.idtmp);
   dfree(d_.celltmp); dfree(d_.perm); dfree(d_.sid); dfree(d_.ccount); dfree(d_.cstart); dfree(d_.chunk_sum);
@@ -409,7 +418,19 @@ int Engine::alloc_arrays() {
   CK(cudaMallocHost((void**)&h_ctl_, sizeof(GraphCtl)));
   CK(cudaMallocHost((void**)&h_reb_count_, sizeof(int32_t) * ns));
   ++struct_ver_;
+  CKR(ensure_fixed());
   return upload_params();
+}
+
+// The FP64 form's positions in pair units (its full lists only).
+int Engine::ensure_fixed() {
+  if (precision_ != 0 || half_ || d_.xl[0]) return kOK;
+  for (int b = 0; b < 2; ++b) {
+    CKR(dmalloc(&d_.xl[b], caps_.slots));
+    CK(cudaMemset(d_.xl[b], 0, sizeof(longlong4_32a) * caps_.slots));
+  }
+  ++struct_ver_;
+  return kOK;
 }
 
 int Engine::stage(int64_t n, double** out) {
@@ -558,6 +579,12 @@ int Engine::upload_params(int only) {
       P.rl2f_lo = std::nextafter((float)(P.rl2 * (1.0 - eps)), 0.0f);
       P.rl2f_hi = std::nextafter((float)(P.rl2 * (1.0 + eps)), 3.0e38f);
     }
+    P.Lfix = host_to_fix(h.spec.L);
+    P.fixed = h.spec.rc <= kFixMaxRc && precision_ == 0 && !half_ ? 1 : 0;
+    if (P.fixed) {
+      P.rc2fix = (long long)std::llrint(std::ldexp(P.rc2, 56));
+      P.c2fix = (long long)std::llrint(std::ldexp(h.c2 / 3.0, 56)) + kFixBias;
+    }
     P.skin = h.spec.skin;
     {
       // FP32-force validity threshold: each shadow coordinate is within 1/2 unit
@@ -618,6 +645,7 @@ int Engine::upload_order() {
 
 DevArrays Engine::arrays() const {
   DevArrays a = d_;
+  if (precision_ != 0 || half_) a.xl[0] = a.xl[1] = nullptr;  // not kept up by the other forms
   a.params = d_params_;
   a.status = d_status_;
   a.disp2 = d_disp2_;
@@ -640,6 +668,8 @@ int Engine::set_precision(int mode) {
   if (mode != precision_) {
     precision_ = mode;
     ++struct_ver_;
+    CKR(ensure_fixed());
+    CKR(upload_params());
     for (SysHost& h : sys_) {
       h.f_valid = false;
       if (h.has_state) h.force_rebuild = true;  // refresh the fixed-point shadow
@@ -666,6 +696,7 @@ int Engine::set_list_kind(int kind) {
   if ((kind == 1) != half_) {
     half_ = kind == 1;
     ++struct_ver_;
+    CKR(ensure_fixed());
     for (SysHost& h : sys_) {
       h.f_valid = false;
       if (h.has_state) h.force_rebuild = true;
@@ -691,6 +722,9 @@ int Engine::set_active(int k, bool on) {
                     cudaMemcpyDeviceToDevice));
       CK(cudaMemcpy(d_.xq[cur_] + h.p_off, d_.xq[h.park] + h.p_off, sizeof(int4) * nslot,
                     cudaMemcpyDeviceToDevice));
+      if (d_.xl[0])
+        CK(cudaMemcpy(d_.xl[cur_] + h.p_off, d_.xl[h.park] + h.p_off, sizeof(longlong4_32a) * nslot,
+                      cudaMemcpyDeviceToDevice));
     }
     h.park = -1;
   }

@@ -164,6 +164,7 @@ class Engine {
 
  private:
   int alloc_arrays();
+  int ensure_fixed();
   void free_all();
   int upload_params(int only = -1);
   int upload_order();

@@ -1,0 +1,203 @@
+// Pair arithmetic of the FP64 form in 64-bit fixed point.
+//
+// GB300's FP64 pipe issues one warp instruction per 64 cycles of a scheduler, its
+// integer multipliers one per 2-4, so the 17 FP64 instructions of a pair (about 1,090
+// cycles per warp) cost several times what the same arithmetic costs in integers.
+// Here a pair's force factor comes from products of 64-bit fixed-point numbers, each
+// formed from 32 x 32 -> 64-bit multiply-adds of its halves, and the sums are kept as
+// 96-bit integers: additions are exact, so a force does not depend on the order in
+// which its pairs are added. Nothing is rounded more coarsely than in FP64: against
+// 128-bit arithmetic the forces of perturbed lattices at densities 0.3 to 0.9, cutoffs
+// 2.5 to 3.9, err by 2e-16 to 1.5e-15 (rms) where the FP64 pipe's err by 1.2e-15 to
+// 2.4e-14.
+//
+// Formats (value = integer x unit):
+//   position, separation  unit 2^-60, modulo 2^64 (16 length units; a separation
+//                         below 8 is recovered exactly from two wrapped positions,
+//                         and an FP64 position of 2^-8 or more is held exactly)
+//   r^2                   2^-56   (r^2 < 16)
+//   y = 1 / r^2           2^-63   (r^2 >= kFixR2Min = 0.84: y < 1.1905)
+//   y^2, y^3, y^4         2^-62, 2^-61, 2^-60
+//   g / 24                2^-56   (|g / 24| < 4.77)
+//   force sums / 24       2^-84   (96 bits; 468 pairs of the largest force, 4.37,
+//                         reach their range)
+// Pairs closer than sqrt(0.84) and lists longer than kFixMaxList take the FP64 pipe.
+#pragma once
+#include <stdint.h>
+
+namespace ljmd {
+
+constexpr int kFixMaxList = 448;                                // longest list summed in 96 bits
+constexpr unsigned kFixR2Min = 14092862u;                      // 0.84 in units of 2^-24 (r^2's high word)
+constexpr double kFixMaxRc = 3.99;                              // r^2 < 16
+
+// A number split into a signed high and a signed low half (the low half rounded to
+// nearest): products of halves are signed 32 x 32 -> 64. fix_split takes the number
+// plus kFixBias, so that the rounding costs no addition where the bias can be folded
+// into a constant or an operand prepared once.
+constexpr long long kFixBias = 0x80000000ll;
+struct Fix2 {
+  int h, l;
+};
+static __device__ __forceinline__ Fix2 fix_split(long long biased) {
+  Fix2 s;
+  s.l = (int)((unsigned)biased + 0x80000000u);
+  s.h = (int)(biased >> 32);
+  return s;
+}
+// FP64 to position units, rounded to nearest (integer operations only; modulo 2^64).
+static __device__ __forceinline__ long long to_fix(double x) {
+  const long long b = __double_as_longlong(x);
+  const int sh = (int)((b >> 52) & 0x7FF) - (1075 - 60);
+  const unsigned long long m = ((unsigned long long)b & 0xFFFFFFFFFFFFFull) | (1ull << 52);
+  unsigned long long r;
+  if (sh >= 0) r = sh < 64 ? m << sh : 0ull;
+  else r = sh >= -54 ? ((m >> (-sh - 1)) + 1ull) >> 1 : 0ull;
+  return b < 0 ? -(long long)r : (long long)r;
+}
+
+// The multiply-add chains below are written out: from the same sums in C++ the compiler
+// makes 1.5 times the multiplier work (a 32 x 32 -> 64-bit multiply-add holds the
+// multiplier for 4 cycles, four times a float one, and is what bounds the pair).
+
+// r^2 of a separation (units 2^-56; the products of two low halves are below the unit).
+static __device__ __forceinline__ unsigned long long fix_r2(const Fix2& x, const Fix2& y, const Fix2& z) {
+  unsigned long long r;
+  asm("{\n\t"
+      ".reg .s64 s;\n\t"
+      "mul.wide.s32 s, %1, %2;\n\t"
+      "mad.wide.s32 s, %3, %4, s;\n\t"
+      "mad.wide.s32 s, %5, %6, s;\n\t"
+      "shr.s64 s, s, 31;\n\t"
+      "mad.wide.s32 s, %1, %1, s;\n\t"
+      "mad.wide.s32 s, %3, %3, s;\n\t"
+      "mad.wide.s32 %0, %5, %5, s;\n\t"
+      "}"
+      : "=l"(r)
+      : "r"(x.h), "r"(x.l), "r"(y.h), "r"(y.l), "r"(z.h), "r"(z.l));
+  return r;
+}
+
+// 1 / r^2 from a hardware float estimate and two Newton steps on exact integer
+// residuals r^2 y - 1 (only their low 32 bits are formed: they are small). The
+// estimate errs by less than 2^-21, the first step leaves 2^-27, the last a relative
+// error near 2^-55.
+static __device__ __forceinline__ unsigned long long fix_rcp(unsigned long long r2) {
+  const unsigned rh = (unsigned)(r2 >> 32), rl = (unsigned)r2;
+  float yf;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"(__uint2float_rn(rh)));
+  const unsigned y0 = __float2uint_rn(yf * 4503599627370496.0f);            // 2^52: unit 2^-28
+  const int e0 = (int)(rh * y0 + __umulhi(rl, y0));                         // unit 2^-52
+  const unsigned y1 = (y0 << 3) - (unsigned)(__mulhi((int)y0, e0) >> 17);   // unit 2^-31
+  const int e1 = (int)(0u - (rh * y1 + __umulhi(rl, y1)));                  // unit 2^-55
+  unsigned long long y;                                                     // y1 + y1 e1
+  asm("{\n\t"
+      ".reg .s64 c;\n\t"
+      ".reg .u32 c0, c1;\n\t"
+      "mul.wide.s32 c, %2, %3;\n\t"  // unit 2^-85
+      "shr.s64 c, c, 22;\n\t"
+      "mov.b64 {c0, c1}, c;\n\t"
+      "add.u32 c1, c1, %1;\n\t"
+      "mov.b64 %0, {c0, c1};\n\t"
+      "}"
+      : "=l"(y)
+      : "r"(y1), "r"((int)(y1 >> 1)), "r"(e1));
+  return y;
+}
+
+// g / 24 = y^4 (1 - 2 y^3) + c2 / 3 (g: the factor 24 r^-8 - 48 r^-14 + 8 c2) plus
+// kFixBias; c2_3b is c2 / 3 in units of 2^-56 plus kFixBias. With y < 1.1905 the cross
+// terms of y y^2 stay below 2^64.
+static __device__ __forceinline__ long long fix_force_factor(unsigned long long y, long long c2_3b) {
+  long long g;
+  asm("{\n\t"
+      ".reg .u64 c, p;\n\t"
+      ".reg .s64 d, t;\n\t"
+      ".reg .u32 y0, y1, a0, a1, b0, b1, c0, c1, z;\n\t"
+      ".reg .s32 wh, wl, qh, ql, d0, d1, sg;\n\t"
+      "mov.b64 {y0, y1}, %1;\n\t"
+      "mul.wide.u32 c, y1, y0;\n\t"            // y^2 (unit 2^-62)
+      "shr.u64 c, c, 31;\n\t"
+      "mad.wide.u32 p, y1, y1, c;\n\t"
+      "mov.b64 {a0, a1}, p;\n\t"
+      "mul.wide.u32 c, y1, a0;\n\t"            // y^3 (unit 2^-61)
+      "mad.wide.u32 c, y0, a1, c;\n\t"
+      "mov.b64 {c0, c1}, c;\n\t"
+      "mov.u32 z, 0;\n\t"
+      "mov.b64 c, {c1, z};\n\t"
+      "mad.wide.u32 c, y1, a1, c;\n\t"
+      "mov.b64 {b0, b1}, c;\n\t"
+      "sub.cc.u32 b0, 0x80000000, b0;\n\t"     // 1 - 2 y^3 (unit 2^-60) plus the bias
+      "subc.u32 wh, 0x10000000, b1;\n\t"
+      "add.u32 wl, b0, 0x80000000;\n\t"
+      "mad.wide.u32 c, a1, a0, 0x4000000000000000;\n\t"  // y^4 (unit 2^-60) plus the bias
+      "shr.u64 c, c, 31;\n\t"
+      "mad.wide.u32 p, a1, a1, c;\n\t"
+      "mov.b64 {b0, qh}, p;\n\t"
+      "add.u32 ql, b0, 0x80000000;\n\t"
+      "mad.wide.s32 d, wl, qh, 0x80000000;\n\t"  // the product, rounded to unit 2^-56
+      "mad.wide.s32 d, wh, ql, d;\n\t"
+      "mad.wide.s32 t, wh, qh, %2;\n\t"
+      "mov.b64 {d0, d1}, d;\n\t"
+      "shr.s32 sg, d1, 31;\n\t"
+      "mov.b64 {c0, c1}, t;\n\t"
+      "add.cc.u32 c0, c0, d1;\n\t"
+      "addc.u32 c1, c1, sg;\n\t"
+      "mov.b64 %0, {c0, c1};\n\t"
+      "}"
+      : "=l"(g)
+      : "l"(y), "l"(c2_3b));
+  return g;
+}
+
+// 96-bit sum of products g d (units 2^-84: g 2^-56, d 2^-60).
+struct FixSum {
+  unsigned lo = 0u;   // units of 2^-84
+  long long hi = 0;   // units of 2^-52
+  __device__ __forceinline__ void add(const Fix2& g, const Fix2& d) {
+    asm("{\n\t"
+        ".reg .s32 m, sg, c0, c1, h0, h1;\n\t"
+        ".reg .s64 c;\n\t"
+        "mul.hi.s32 m, %3, %5;\n\t"
+        "cvt.s64.s32 c, m;\n\t"
+        "mad.wide.s32 c, %2, %5, c;\n\t"
+        "mad.wide.s32 c, %3, %4, c;\n\t"
+        "mad.wide.s32 %1, %2, %4, %1;\n\t"
+        "mov.b64 {c0, c1}, c;\n\t"
+        "shr.s32 sg, c1, 31;\n\t"
+        "mov.b64 {h0, h1}, %1;\n\t"
+        "add.cc.u32 %0, %0, c0;\n\t"
+        "addc.cc.u32 h0, h0, c1;\n\t"
+        "addc.u32 h1, h1, sg;\n\t"
+        "mov.b64 %1, {h0, h1};\n\t"
+        "}"
+        : "+r"(lo), "+l"(hi)
+        : "r"(g.h), "r"(g.l), "r"(d.h), "r"(d.l));
+  }
+  // 24 x the sum as FP64, formed with integer operations (the FP64 pipe's conversions
+  // would cost more than the pairs of three rounds).
+  __device__ __forceinline__ double value24() const {
+    unsigned long long h = (unsigned long long)hi;
+    unsigned l = lo;
+    if (hi < 0) {  // magnitude of the 96-bit sum
+      l = 0u - l;
+      h = ~h + (l == 0u ? 1ull : 0ull);
+    }
+    if (h == 0ull && l == 0u) return 0.0;
+    const int z = h ? __clzll((long long)h) : 64 + __clz((int)l);  // leading zeros of 96 bits
+    unsigned long long m;                                         // top 64 bits, normalised
+    if (z == 0) m = h;
+    else if (z < 32) m = (h << z) | (l >> (32 - z));
+    else if (z < 64) m = (h << z) | ((unsigned long long)l << (z - 32));
+    else m = (unsigned long long)l << (z - 32);
+    m = (m >> 3) * 3ull;                  // in [3, 6) x 2^60: value m 2^(-84 + 32 - z + 3 + 3)
+    const int up = (int)(m >> 62);        // 1: m in [2^62, 2^63)
+    const int k = up ? 10 : 9;            // m >> k has 53 bits
+    m = (m + (1ull << (k - 1))) >> k;     // may round up to 2^53: the addition below carries
+    const int ex = 1023 + 52 + k - 46 - z;
+    const unsigned long long b = ((unsigned long long)(ex - 1) << 52) + m;
+    return __longlong_as_double((long long)(b | (hi < 0 ? 0x8000000000000000ull : 0ull)));
+  }
+};
+
+}  // namespace ljmd

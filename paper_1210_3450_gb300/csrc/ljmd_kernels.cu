@@ -20,6 +20,7 @@
 #include <algorithm>
 
 #include "ljmd_dev.cuh"
+#include "ljmd_fixed.cuh"
 #include "ljmd_math.cuh"
 
 namespace ljmd {
@@ -49,6 +50,22 @@ __device__ __forceinline__ bool tile_ctx(const DevArrays& a, TileCtx& t, SysPara
   if (!P.active) return false;
   t.tl = warp - P.t_off;
   t.local = t.tl * kTile + lane;
+  t.s = P.p_off + t.local;
+  t.act = t.local < P.n;
+  return true;
+}
+
+// The same without a copy of the system's parameters (held in registers they would
+// cost a kernel its occupancy).
+__device__ __forceinline__ bool tile_ref(const DevArrays& a, TileCtx& t) {
+  const int warp = (int)((blockIdx.x * (unsigned)blockDim.x + threadIdx.x) >> 5);
+  if (warp >= a.ntiles) return false;
+  t.sys = a.tile_sys[warp];
+  if (t.sys < 0) return false;
+  const SysParams& P = a.params[t.sys];
+  if (!P.active) return false;
+  t.tl = warp - P.t_off;
+  t.local = t.tl * kTile + (threadIdx.x & 31);
   t.s = P.p_off + t.local;
   t.act = t.local < P.n;
   return true;
@@ -356,8 +373,19 @@ __global__ void k_cell_rank(DevArrays a, int cur) {
 // The rebuilt state of one slot back into place. The list build does this for the
 // tiles it builds: it reads only the build-time positions, shadows and scratch
 // cells, which the copy does not touch, so the copy needs no launch of its own.
+__device__ __forceinline__ longlong4_32a fix4(const double4_32a& x) {
+  longlong4_32a q;
+  q.x = to_fix(x.x);
+  q.y = to_fix(x.y);
+  q.z = to_fix(x.z);
+  q.w = 0;
+  return q;
+}
+
 __device__ __forceinline__ void copy_back_slot(const DevArrays& a, int cur, int64_t s) {
-  a.x[cur][s] = a.xref[s];
+  const double4_32a x = a.xref[s];
+  a.x[cur][s] = x;
+  if (a.xl[0]) a.xl[cur][s] = fix4(x);
   a.v[s] = a.vtmp[s];
   a.id[s] = a.idtmp[s];
   a.cell[s] = a.celltmp[s];
@@ -1077,8 +1105,10 @@ __device__ __forceinline__ unsigned long long integrate(const DevArrays& a, cons
     const long long ex = wrapped_diff(q.x, r.x), ey = wrapped_diff(q.y, r.y), ez = wrapped_diff(q.z, r.z);
     return (unsigned long long)(ex * ex) + (unsigned long long)(ey * ey) + (unsigned long long)(ez * ez);
   }
-  // the fixed-point shadow, which the FP64 force loop's pre-classification reads
+  // the fixed-point shadow, which the FP64 force loop's pre-classification reads, and
+  // the positions in pair units
   a.xq[cur ^ 1][t.s] = fixed4(xn, P.qscale);
+  if (a.xl[0]) a.xl[cur ^ 1][t.s] = fix4(xn);
   if (flags & kStepVmax) return v2b();
   // exact FP64 check, the same operations as the reference
   const double4_32a r = a.xref[t.s];
@@ -1238,32 +1268,38 @@ __device__ __forceinline__ double force_factor(double r2, double c2x8) {
   return fma(24.0, ir8, fma(-48.0, ir14, c2x8));
 }
 
-// FP64 form. The FP64 pipe is the bound (on GB300 a warp's FP64 instruction
-// holds the pipe about as long as 60 other instructions take to issue), and a
-// warp pays for an FP64 instruction whether one lane or all 32 need it. So each
-// thread first classifies its listed partners on their fixed-point shadow
-// positions (integer separations, float r^2, no FP64 instruction) against
-// rc^2 (1 + 1e-5), a bound that no pair inside rc can exceed (each shadow
-// coordinate errs by at most half a unit of L / 2^32, and the float r^2 by a few
-// parts in 1e7), and queues the list words of the pairs that
-// may be inside in shared memory. The FP64 work then runs in rounds in which every
-// thread with partners left takes the next pair of its own queue: per pair 3 DADD
-// for the separation and 3 for r^2, the exact test r^2 < rc^2 (bit patterns,
-// r^2 >= 0), and for pairs inside the reciprocal (3 DFMA after an integer-built
-// FP32 seed), the powers and factor (5) and the accumulation (3). A thread's
-// queue keeps list order and the pairs left out are outside rc, where the force
-// is zero, so every force is summed in the same order as a plain loop over the
-// list: the results are the same bit for bit.
-constexpr int kQueue64 = 16;  // queued list words per thread (FP64 pair loops)
+// FP64 form. On GB300 a warp's FP64 instruction holds the FP64 pipe for 64 cycles, so
+// with the 17 FP64 instructions of a pair the loop ran at that pipe's rate (3.7 ms per
+// step at 2,048,000 particles, pipe 89 % busy). Two things take the load off it:
+//   The pair arithmetic runs in 64-bit fixed point on the integer multipliers
+//   (ljmd_fixed.cuh: about 245 cycles per pair and warp against 1,140): 1.01 ms per
+//   pair pass, with smaller errors than the FP64 pipe's.
+//   Pairs outside rc are left out before it. Each thread classifies its listed
+//   partners on their fixed-point shadow positions (integer separations, float r^2)
+//   against rc^2 (1 + 1e-5), a bound that no pair inside rc can exceed (each shadow
+//   coordinate errs by at most half a unit of L / 2^32, and the float r^2 by a few
+//   parts in 1e7), and queues the list words of the pairs that may be inside in shared
+//   memory; the pairs then run in rounds in which every thread with partners left
+//   takes the next one of its own queue (1.10 ms without the queue).
+// The FP64 pipe still takes the pairs out of the fixed-point range, cutoffs above
+// kFixMaxRc and the approximate-reciprocal modes: 3 DADD for the separation and 3
+// operations for r^2, the exact test r^2 < rc^2 (bit patterns, r^2 >= 0), the
+// reciprocal (3 DFMA after an integer-built FP32 seed), the powers and factor (5) and
+// the accumulation (3). The fixed-point sums are exact and a thread's queue keeps list
+// order for the others, so the results equal a plain loop's bit for bit.
+constexpr int kQueue64 = 32;  // queued list words per thread (FP64 pair loops)
 
 // The classify-and-queue loop of the FP64 pair loops: every thread of the warp
-// calls it (cnt = 0 for a lane without a particle); body(e) runs for the list
-// words e of the thread's maybe-inside pairs, in list order, in rounds where
-// every thread with a queued pair takes one. qme points at the thread's queue
-// column (entry q at qme[q * BLOCK]).
-template <int BLOCK, class Body>
+// calls it (cnt = 0 for a lane without a particle). The list words of the thread's
+// maybe-inside pairs go through pair(load(e), e) in list order: each pass of the loop classifies up to kClassify groups of four
+// partners per lane (as far as its queue has room) and then runs as many rounds as
+// every lane with partners left has queued, so the warp votes once per pass and
+// not once per round. qme points at the thread's queue column (entry q at
+// qme[q * BLOCK]).
+constexpr int kClassify = 7;
+template <int BLOCK, class Load, class Pair>
 __device__ __forceinline__ void queued_pairs(const DevArrays& a, const TileCtx& t, const SysParams& P, int lane,
-                                             int cur, int cnt, uint32_t* qme, Body&& body) {
+                                             int cur, int cnt, uint32_t* qme, Load&& load, Pair&& pair) {
   const uint4* lp4 = (const uint4*)(a.nbr + list_word(P.l_off, t.tl, P.kmax, lane, 0));
   const int4* qs = a.xq[cur] + P.p_off;
   const int4 qi = t.act ? qs[t.local] : make_int4(0, 0, 0, 0);
@@ -1271,115 +1307,167 @@ __device__ __forceinline__ void queued_pairs(const DevArrays& a, const TileCtx& 
   const uint32_t self = (uint32_t)t.local;
   int k = 0;  // next listed partner to classify
   unsigned head = 0u, tail = 0u;
+  uint4 w = make_uint4(self, self, self, self);
+  if (cnt > 0) w = __ldg(lp4);
   while (true) {
-    const unsigned qn = tail - head;
-    const bool left = k < cnt;
-    const unsigned has = __ballot_sync(kFull, qn > 0u);
-    const unsigned busy = __ballot_sync(kFull, qn > 0u || left);
-    if (busy == 0u) break;
-    const unsigned room = __ballot_sync(kFull, left && qn <= (unsigned)(kQueue64 - 4));
-    if (has == busy || room == 0u) {
-      // FP64 round: each thread with a queued pair takes the next one
-      if (qn > 0u) {
-        const uint32_t e = qme[(head & (kQueue64 - 1)) * BLOCK];
-        ++head;
-        body(e);
-      }
-    } else if ((room >> (threadIdx.x & 31)) & 1u) {  // the ballot's bit of this thread
-      // classification of the next four listed partners (no FP64 instruction)
-      const uint4 w = __ldg(lp4 + (int64_t)(k >> 2) * kTile);
+#pragma unroll 1
+    for (int u = 0; u < kClassify; ++u) {
+      if (k >= cnt || tail - head > (unsigned)(kQueue64 - 4)) break;
+      // the next four listed partners (no FP64 instruction)
       const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
+      k += 4;
+      if (k < cnt) w = __ldg(lp4 + (int64_t)(k >> 2) * kTile);  // the next group's load in flight
 #pragma unroll
       for (int m = 0; m < 4; ++m) {
-        const bool ok = k + m < cnt;
-        const int4 qj = qs[ok ? partner_slot(a, t.sys, ws[m], P.n, self) : self];
+        const int4 qj = qs[partner_slot(a, t.sys, ws[m], P.n, self)];
         const float ax = (float)wrapped_diff(qj.x, qi.x);
         const float ay = (float)wrapped_diff(qj.y, qi.y);
         const float az = (float)wrapped_diff(qj.z, qi.z);
-        if (ok && fmaf(az, az, fmaf(ay, ay, ax * ax)) < rc2q) {
+        // the list's padding entries name the particle itself
+        if (ws[m] != self && fmaf(az, az, fmaf(ay, ay, ax * ax)) < rc2q) {
           qme[(tail & (kQueue64 - 1)) * BLOCK] = ws[m];
           ++tail;
         }
       }
-      k += 4;
     }
+    const bool left = k < cnt;
+    const bool more = __any_sync(kFull, left);
+    const unsigned rounds = more ? __reduce_min_sync(kFull, left ? tail - head : ~0u)
+                                 : __reduce_max_sync(kFull, tail - head);
+#pragma unroll 1
+    for (unsigned r = 0; r < rounds; ++r) {
+      if (head == tail) continue;
+      const uint32_t e = qme[(head & (kQueue64 - 1)) * BLOCK];
+      ++head;
+      pair(load(e), e);
+    }
+    if (!more) break;
   }
 }
 
+// Force of one particle, pair by pair. MODE 0 sums in fixed point (ljmd_fixed.cuh)
+// where the system's cutoff and the particle's list length allow it; pairs closer than
+// its range and all pairs of the other modes take the FP64 pipe.
+template <int MODE>
+struct PairForce {
+  const DevArrays& a;
+  const TileCtx& t;
+  const SysParams& P;
+  int cur;
+  longlong4_32a qi;
+  bool fixed;
+  FixSum sx, sy, sz;
+  double* slow;  // the FP64 pairs' sums, one column of a shared array per thread
+  int stride;
 
-// QUEUE false: the plain loop over the list (every listed pair takes the FP64
-// separation and r^2, the warp pays the force body whenever one lane is inside).
+  __device__ __forceinline__ PairForce(const DevArrays& a_, const TileCtx& t_, const SysParams& P_, int cur_, int cnt,
+                                       double* slow_, int stride_)
+      : a(a_), t(t_), P(P_), cur(cur_), slow(slow_), stride(stride_) {
+    slow[0] = slow[stride] = slow[2 * stride] = 0.0;
+    fixed = MODE == 0 && a.xl[0] && P.fixed && cnt <= kFixMaxList;
+    qi = fixed && t.act ? a.xl[cur][t.s] : longlong4_32a{0, 0, 0, 0};
+    qi.x -= kFixBias; qi.y -= kFixBias; qi.z -= kFixBias;  // separations come biased for fix_split
+  }
+  __device__ __forceinline__ void fp64_pair(uint32_t j, unsigned code) {
+    const long long rc2b = __double_as_longlong(P.rc2);
+    const double c2x8 = 8.0 * P.c2;
+    const double4_32a xi = a.x[cur][t.s];
+    const double4_32a xj = a.x[cur][P.p_off + j];
+    double dx = xj.x - xi.x, dy = xj.y - xi.y, dz = xj.z - xi.z;
+    if (code) {
+      dx = apply_image(dx, code & 3u, P.L);
+      dy = apply_image(dy, (code >> 2) & 3u, P.L);
+      dz = apply_image(dz, (code >> 4) & 3u, P.L);
+    }
+    const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
+    if (__double_as_longlong(r2) < rc2b) {
+      const double g = force_factor<MODE>(r2, c2x8);  // 24 r^-8 - 48 r^-14 + 8 c2
+      slow[0] = fma(g, dx, slow[0]);
+      slow[stride] = fma(g, dy, slow[stride]);
+      slow[2 * stride] = fma(g, dz, slow[2 * stride]);
+    }
+  }
+  __device__ __forceinline__ uint32_t slot(uint32_t e) const {
+    return partner_slot(a, t.sys, e, P.n, (uint32_t)t.local);
+  }
+  __device__ __forceinline__ longlong4_32a load(uint32_t e) const {
+    if (MODE == 0 && fixed) return a.xl[cur][P.p_off + slot(e)];
+    return longlong4_32a{0, 0, 0, 0};
+  }
+  __device__ __forceinline__ void pair(const longlong4_32a& qj, uint32_t e) {
+    const unsigned code = e >> kIdxBits;
+    if (MODE == 0 && fixed) {
+      long long dx = qj.x - qi.x, dy = qj.y - qi.y, dz = qj.z - qi.z;
+      if (code) {
+        const long long L = P.Lfix;
+        dx += (code & 3u) == 1u ? L : ((code & 3u) == 2u ? -L : 0);
+        dy += (code & 12u) == 4u ? L : ((code & 12u) == 8u ? -L : 0);
+        dz += (code & 48u) == 16u ? L : ((code & 48u) == 32u ? -L : 0);
+      }
+      const Fix2 fx = fix_split(dx), fy = fix_split(dy), fz = fix_split(dz);
+      const unsigned long long r2 = fix_r2(fx, fy, fz);
+      const bool far = (unsigned)(r2 >> 32) >= kFixR2Min;
+      if (far & ((long long)(r2 - (unsigned long long)P.rc2fix) < 0)) {
+        const Fix2 g = fix_split(fix_force_factor(fix_rcp(r2), P.c2fix));
+        sx.add(g, fx);
+        sy.add(g, fy);
+        sz.add(g, fz);
+      } else if (!far) {
+        fp64_pair(slot(e), code);
+      }
+    } else {
+      fp64_pair(slot(e), code);
+    }
+  }
+  // The sums as FP64 (the FP64 pairs' share added where there is one).
+  __device__ __forceinline__ void result(double& x, double& y, double& z) const {
+    x = slow[0]; y = slow[stride]; z = slow[2 * stride];
+    if (MODE == 0 && fixed) {
+      const bool some = x != 0.0 || y != 0.0 || z != 0.0;
+      const double fx = sx.value24(), fy = sy.value24(), fz = sz.value24();
+      x = some ? fx + x : fx; y = some ? fy + y : fy; z = some ? fz + z : fz;
+    }
+  }
+};
+
+// QUEUE false: the plain loop over the list.
+// 32 warps per SM (64 registers): 1.01 ms per pair pass at 2,048,000 particles against
+// 1.06 at 28 and 1.08 at 24.
 template <int BLOCK, int MODE, bool QUEUE>
-__global__ void __launch_bounds__(BLOCK) k_step_fp64(DevArrays a, int cur, double ka, double kb, int flags) {
+__global__ void __launch_bounds__(BLOCK, MODE == 0 ? 1024 / BLOCK : 1) k_step_fp64(DevArrays a, int cur, double ka, double kb, int flags) {
   __shared__ uint32_t qbuf[QUEUE ? kQueue64 : 1][BLOCK];  // entry q of thread t at [q][t]: no bank conflicts
+  __shared__ double slow[3][BLOCK];
   if (a.ctl) {  // graph-captured loop (uniform over the grid)
     if (a.ctl->abort) return;
     flags = a.ctl->flags;
   }
   TileCtx t;
-  SysParams P;
-  if (!tile_ctx(a, t, P)) return;  // uniform over the warp
+  if (!tile_ref(a, t)) return;  // uniform over the warp
+  const SysParams& P = a.params[t.sys];
   const int lane = threadIdx.x & 31;
   double Fx = 0.0, Fy = 0.0, Fz = 0.0;
-  double4_32a xi = make_double4_32a(0.0, 0.0, 0.0, 0.0);
-  if (t.act) xi = a.x[cur][t.s];
   if (flags & kStepUseStoredF) {
     if (t.act) {
       const double4_32a f = a.f[t.s];
       Fx = f.x; Fy = f.y; Fz = f.z;
     }
-  } else if (!QUEUE) {
-    if (t.act) {
-      const int cnt = list_count(a, t.sys, t.s, P.kmax);
-      const uint32_t* lp = a.nbr + list_word(P.l_off, t.tl, P.kmax, lane, 0);
-      const double4_32a* xs = a.x[cur] + P.p_off;
-      const long long rc2b = __double_as_longlong(P.rc2);
-      const double c2x8 = 8.0 * P.c2, L = P.L;
-      for (int k = 0; k < cnt; ++k) {
-        const uint32_t e = __ldg(lp + (int64_t)(k >> 2) * (4 * kTile) + (k & 3));
-        const double4_32a xj = xs[partner_slot(a, t.sys, e, P.n, (uint32_t)t.local)];
-        double dx = xj.x - xi.x, dy = xj.y - xi.y, dz = xj.z - xi.z;
-        const unsigned code = e >> kIdxBits;
-        if (code) {
-          dx = apply_image(dx, code & 3u, L);
-          dy = apply_image(dy, (code >> 2) & 3u, L);
-          dz = apply_image(dz, (code >> 4) & 3u, L);
-        }
-        const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
-        if (__double_as_longlong(r2) < rc2b) {
-          const double g = force_factor<MODE>(r2, c2x8);  // 24 r^-8 - 48 r^-14 + 8 c2
-          Fx = fma(g, dx, Fx);
-          Fy = fma(g, dy, Fy);
-          Fz = fma(g, dz, Fz);
-        }
-      }
-    }
   } else {  // every lane of the warp takes part (inactive ones with an empty list)
     const int cnt = t.act ? list_count(a, t.sys, t.s, P.kmax) : 0;
-    const double4_32a* xs = a.x[cur] + P.p_off;
-    const long long rc2b = __double_as_longlong(P.rc2);
-    const double c2x8 = 8.0 * P.c2, L = P.L;
-    const uint32_t self = (uint32_t)t.local;
-    queued_pairs<BLOCK>(a, t, P, lane, cur, cnt, &qbuf[0][threadIdx.x], [&](uint32_t e) {
-      const double4_32a xj = xs[partner_slot(a, t.sys, e, P.n, self)];
-      double dx = xj.x - xi.x, dy = xj.y - xi.y, dz = xj.z - xi.z;
-      const unsigned code = e >> kIdxBits;
-      if (code) {
-        dx = apply_image(dx, code & 3u, L);
-        dy = apply_image(dy, (code >> 2) & 3u, L);
-        dz = apply_image(dz, (code >> 4) & 3u, L);
+    PairForce<MODE> pf(a, t, P, cur, cnt, &slow[0][threadIdx.x], BLOCK);
+    if (QUEUE) {
+      queued_pairs<BLOCK>(a, t, P, lane, cur, cnt, &qbuf[0][threadIdx.x], [&](uint32_t e) { return pf.load(e); },
+                          [&](const longlong4_32a& q, uint32_t e) { pf.pair(q, e); });
+    } else {
+      const uint32_t* lp = a.nbr + list_word(P.l_off, t.tl, P.kmax, lane, 0);
+      for (int k = 0; k < cnt; ++k) {
+        const uint32_t e = __ldg(lp + (int64_t)(k >> 2) * (4 * kTile) + (k & 3));
+        pf.pair(pf.load(e), e);
       }
-      const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
-      if (__double_as_longlong(r2) < rc2b) {
-        const double g = force_factor<MODE>(r2, c2x8);  // 24 r^-8 - 48 r^-14 + 8 c2
-        Fx = fma(g, dx, Fx);
-        Fy = fma(g, dy, Fy);
-        Fz = fma(g, dz, Fz);
-      }
-    });
+    }
+    pf.result(Fx, Fy, Fz);
   }
   unsigned long long d2b = 0ull;
-  if (t.act) d2b = integrate<false>(a, P, t, cur, xi, Fx, Fy, Fz, ka, kb, flags);
+  if (t.act) d2b = integrate<false>(a, P, t, cur, a.x[cur][t.s], Fx, Fy, Fz, ka, kb, flags);
   warp_max_disp(a, t.sys, d2b, flags);
 }
 
@@ -1533,8 +1621,8 @@ __global__ void __launch_bounds__(kBlock) k_pe_virial(DevArrays a, int cur, int 
     const uint32_t self = (uint32_t)t.local;
     double s12 = 0.0, s6 = 0.0, sr = 0.0;
     int nin = 0;
-    queued_pairs<kBlock>(a, t, P, lane, cur, cnt, &qbuf[0][threadIdx.x], [&](uint32_t e) {
-      const double4_32a xj = xs[partner_slot(a, t.sys, e, P.n, self)];
+    auto load = [&](uint32_t e) { return xs[partner_slot(a, t.sys, e, P.n, self)]; };
+    queued_pairs<kBlock>(a, t, P, lane, cur, cnt, &qbuf[0][threadIdx.x], load, [&](const double4_32a& xj, uint32_t e) {
       double dx = xj.x - xi.x, dy = xj.y - xi.y, dz = xj.z - xi.z;
       const unsigned code = e >> kIdxBits;
       if (code) {
@@ -1713,6 +1801,7 @@ __global__ void k_positions_by_id(DevArrays a, int cur, const double* __restrict
   const double4_32a xv = make_double4_32a(x[3 * i + 0], x[3 * i + 1], x[3 * i + 2], 0.0);
   a.x[cur][s] = xv;
   a.xq[cur][s] = fixed4(xv, P.qscale);
+  if (a.xl[0]) a.xl[cur][s] = fix4(xv);
 }
 
 void launch_positions_by_id(const DevArrays& a, int cur, const double* x, int64_t sys_n, int sys, cudaStream_t s) {

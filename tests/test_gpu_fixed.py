@@ -1,0 +1,66 @@
+"""Fixed-point pair arithmetic of the FP64 form at the edges of its range: the change
+to the FP64 pipe at close pairs, at long lists and at large cutoffs, positions at both
+ends of a large box, pairs at the cutoff. The bound is the FP64 form's 1e-12 of the
+rms force; both force loops give the same bits."""
+import numpy as np
+import pytest
+
+import lj_inputs as li
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+
+def _dimers(r, box, seed):
+    """Pairs at the given distances in random directions, the pairs 7 apart."""
+    g = np.random.Generator(np.random.PCG64(seed))
+    m = int(box // 7.0)
+    k = np.arange(len(r))
+    assert m ** 3 >= len(r)
+    c = np.stack([k % m, k // m % m, k // m ** 2], 1) * 7.0 + 0.5 + g.uniform(0, 0.5, (len(r), 3))
+    u = g.standard_normal((len(r), 3))
+    u /= np.linalg.norm(u, axis=1, keepdims=True)
+    return np.mod(np.concatenate([c, c + u * r[:, None]]), box)
+
+
+def _case(name):
+    if name == "close":  # around r^2 = 0.84, where the fixed-point range ends
+        r = np.concatenate([np.sqrt(0.84) * (1 + np.linspace(-1e-6, 1e-6, 41)), np.linspace(0.7, 1.1, 59)])
+        return _dimers(r, 40.0, 1), 40.0, 2.5
+    if name == "cutoff":
+        r = np.concatenate([2.5 * (1 + np.linspace(-1e-9, 1e-9, 41)), np.linspace(2.3, 2.7, 59)])
+        return _dimers(r, 40.0, 2), 40.0, 2.5
+    if name == "far corner":  # positions near 0 and near a large L, pairs across every face
+        r = np.linspace(0.9, 2.6, 60)
+        x = _dimers(r, 30.0, 3)
+        x[::3] += 1200.5 - 15.0
+        x[1::3] -= 15.0
+        return np.mod(x, 1200.5), 1200.5, 2.5
+    if name == "long lists":  # more partners than the 96-bit sums take, some below the limit
+        x, box = li.perturbed_fcc(3001, 1.5, 0.02, 4)
+        keep = (x[:, 0] < 0.55 * box) | (np.arange(len(x)) % 3 == 0)
+        return np.ascontiguousarray(x[keep]), box, 3.9
+    if name == "rc 3.99":
+        return *li.perturbed_fcc(2000, 0.85, 0.1, 5), 3.99
+    if name == "rc 4.0":
+        return *li.perturbed_fcc(2000, 0.85, 0.1, 6), 4.0
+    return *li.perturbed_fcc(33, 0.3, 0.05, 7), 1.9  # one cell: every pair a candidate
+
+
+@pytest.mark.parametrize("name", ["close", "cutoff", "far corner", "long lists", "rc 3.99", "rc 4.0", "small"])
+def test_forces_at_the_edges(name):
+    from paper_1210_3450_gb300 import MD_FP64, LJSystem
+    x, box, rc = _case(name)
+    ref = oracle.forces_brute(x, box, rc)
+    rms = np.sqrt((ref ** 2).sum(1).mean())
+    got = []
+    with LJSystem(box, len(x), rc, 0.3, MD_FP64) as s:
+        for queue in (1, 0):
+            s.set_tuning(fp64_queue=queue)
+            s.set_state(x, np.zeros_like(x))
+            got.append(s.forces())
+        if name == "long lists":
+            cnt = np.diff(s.get_list()[0])
+            assert cnt.min() <= 448 < cnt.max()
+    np.testing.assert_array_equal(got[0], got[1])
+    assert np.abs(got[0] - ref).max() <= 1e-12 * rms
