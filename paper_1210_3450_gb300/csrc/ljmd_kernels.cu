@@ -1056,6 +1056,217 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) k_build_list_staged(DevAr
   while (next_rebuild_tile(a, sys, tl)) build_tile_staged(a, cur, sys, tl, sbuf[threadIdx.x >> 5]);
 }
 
+// List build with one candidate per lane, for passes of too few tiles to fill the GPU
+// with one warp each (such a pass waits on one warp's serial sweep of 9 rows, 70 us
+// whatever its size). A block takes `span` consecutive slots (8 or 32: 1 or 4 per
+// warp). The particles of one cell have the same 27 neighbour cells, so for each run of
+// slots in one cell the block copies all candidates into shared memory in row order,
+// shifted to their image, with every load in flight at once (a global load per round of
+// 32 candidates would cost its L2 latency each time); each particle's warp then tests
+// them 32 at a time and appends the accepted lanes by their place in the ballot. That
+// is candidate order, so the lists are the same word for word.
+namespace {
+
+constexpr int kWideBlock = 256;
+constexpr int kWideWarps = kWideBlock / 32;
+constexpr int kWideStage = 1024;  // candidates staged at a time
+
+struct WideShared {
+  float4 cand[kWideStage];
+  uint32_t word[kWideStage];
+  int cell[kTile];
+};
+
+// Slots [s0, s1) of system sys (within one tile, at most 32); called by the whole block
+// with uniform arguments. Returns the longest list of the warp's particles.
+__device__ __forceinline__ int build_span(const DevArrays& a, int cur, int sys, const SysParams* __restrict__ Pp,
+                                          int s0, int s1, WideShared& sh) {
+  const int lane = threadIdx.x & 31, wv = threadIdx.x >> 5;
+  const unsigned below = (1u << lane) - 1u;
+  const int nc = Pp->nc, kmax = Pp->kmax;
+  const int64_t p_off = Pp->p_off;
+  const bool half = Pp->half != 0;
+  const double4_32a* xs = a.xref + p_off;
+  // list words of slot s0; those of slot s0 + p follow at 4 p
+  uint32_t* out = a.nbr + list_word(Pp->l_off, s0 / kTile, kmax, s0 % kTile, 0);
+  int wmax = 0;
+  // appends the lanes with `in` set (candidate j, list word e) to particle p's list of length c
+  auto append = [&](bool in, int p, int j, uint32_t e, int& c) {
+    if (kChecks && in) in = check_ok(a, sys, (unsigned)j < (unsigned)Pp->n && j != s0 + p, kChkListEntry);
+    const unsigned m = __ballot_sync(kFull, in);
+    const int k = c + __popc(m & below);
+    if (in && k < kmax) out[((k >> 2) * kTile + p) * 4 + (k & 3)] = e;
+    c += __popc(m);
+  };
+  auto finish = [&](int p, int c) {  // padding to a whole group of four (ListCtx::pad), length
+    const int k = c + lane;
+    if (k < ((c + 3) & ~3) && k < kmax) out[((k >> 2) * kTile + p) * 4 + (k & 3)] = (uint32_t)(s0 + p);
+    if (lane == 0) a.ncnt[p_off + s0 + p] = c < kmax ? c : kmax;
+    wmax = c > wmax ? c : wmax;
+  };
+  if (nc == 1) {  // every particle is a candidate, at its minimum image (as sweep_all)
+    const int4* q = a.xq[cur] + p_off;
+    const float hi2 = Pp->rl2q_hi;
+    const int n = Pp->n;
+    for (int p = wv; p < s1 - s0; p += kWideWarps) {
+      const int i = s0 + p;
+      const int4 qi = q[i];
+      int c = 0;
+      for (int j0 = 0; j0 < n; j0 += 32) {
+        const int j = j0 + lane;
+        bool in = false;
+        unsigned code = 0u;
+        if (j < n && (half ? j > i : j != i)) {
+          const int4 qj = q[j];
+          const float ax = (float)wrapped_diff(qj.x, qi.x);
+          const float ay = (float)wrapped_diff(qj.y, qi.y);
+          const float az = (float)wrapped_diff(qj.z, qi.z);
+          if (fmaf(az, az, fmaf(ay, ay, ax * ax)) < hi2) {
+            const double4_32a xi = xs[i], xj = xs[j];
+            const unsigned r = exact_inside(xi.x, xi.y, xi.z, xj.x, xj.y, xj.z, 0xffu, Pp->L, Pp->rl2);
+            in = (r & 0x100u) != 0u;
+            code = r & 0xffu;
+          }
+        }
+        append(in, p, j, (uint32_t)j | (code << kIdxBits), c);
+      }
+      finish(p, c);
+    }
+    return wmax;
+  }
+  const float4* __restrict__ xf = a.xf + p_off;
+  const float lo2 = Pp->rl2f_lo, hi2 = Pp->rl2f_hi, Lf = Pp->Lf;
+  if (wv == 0) sh.cell[lane] = s0 + lane < s1 ? a.celltmp[p_off + s0 + lane] : -1;
+  __syncthreads();
+  for (int p0 = 0; p0 < s1 - s0;) {  // runs of slots in one cell (slots are in cell order)
+    const int cell = sh.cell[p0];
+    const int p1 = p0 + __popc(__ballot_sync(kFull, sh.cell[lane] == cell));
+    const int cx = cell % nc, cy = (cell / nc) % nc, cz = cell / (nc * nc);
+    // lane 2 r holds row r's candidate range and image code, lane 2 r + 1 its second
+    // piece where the row wraps in x; `at` is the place of its first candidate
+    int lo = 0, hi = 0;
+    unsigned code = 0u;
+    if (lane < 18) {
+      const int r = lane >> 1;
+      const bool second = lane & 1;
+      int nz = cz + r / 3 - 1, ny = cy + r % 3 - 1;
+      unsigned shz = 0, shy = 0;
+      if (nz < 0) { nz += nc; shz = 2; } else if (nz >= nc) { nz -= nc; shz = 1; }
+      if (ny < 0) { ny += nc; shy = 2; } else if (ny >= nc) { ny -= nc; shy = 1; }
+      const int32_t* cst = a.cstart + Pp->c_off + nc * (ny + nc * nz);
+      code = (shy << 2) | (shz << 4);
+      int c0 = cx - 1, c1 = cx + 2;  // cells [c0, c1)
+      if (cx == 0) {
+        if (second) { c0 = 0; c1 = 2; }
+        else { c0 = nc - 1; c1 = nc; code |= 2u; }  // x image -L
+      } else if (cx == nc - 1) {
+        if (second) { c0 = 0; c1 = 1; code |= 1u; }  // x image +L
+        else { c0 = nc - 2; c1 = nc; }
+      } else if (second) {
+        c0 = c1 = 0;
+      }
+      if (c0 < c1) { lo = cst[c0]; hi = cst[c1]; }
+    }
+    int at = hi - lo;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(kFull, at, o);
+      if (lane >= o) at += y;
+    }
+    const int total = __shfl_sync(kFull, at, 31);
+    at -= hi - lo;
+    int c[4] = {0, 0, 0, 0};  // list lengths of the warp's particles p0 + wv + 8 i
+    for (int base = 0; base < total; base += kWideStage) {
+      for (int l = wv; l < 18; l += kWideWarps) {
+        const int jlo = __shfl_sync(kFull, lo, l), jhi = __shfl_sync(kFull, hi, l);
+        const int f0 = __shfl_sync(kFull, at, l) - base - jlo;
+        const unsigned cd = __shfl_sync(kFull, code, l);
+        // image code 1 adds +L to x_j - x_i, code 2 adds -L: the candidate is shifted in
+        // float (the same bound as shifting the particle, 4 u L and u L for the other)
+        const float sx = (cd & 3u) == 1u ? Lf : ((cd & 3u) == 2u ? -Lf : 0.f);
+        const float sy = (cd & 12u) == 4u ? Lf : ((cd & 12u) == 8u ? -Lf : 0.f);
+        const float sz = (cd & 48u) == 16u ? Lf : ((cd & 48u) == 32u ? -Lf : 0.f);
+#pragma unroll 4
+        for (int j = jlo + lane; j < jhi; j += 32) {
+          const int f = f0 + j;
+          if ((unsigned)f < (unsigned)kWideStage) {
+            const float4 q = xf[j];
+            sh.cand[f] = make_float4(q.x + sx, q.y + sy, q.z + sz, 0.f);
+            sh.word[f] = (uint32_t)j | (cd << kIdxBits);
+          }
+        }
+      }
+      __syncthreads();
+      const int nb = min(kWideStage, total - base);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int p = p0 + wv + kWideWarps * i;
+        if (p >= p1) break;  // uniform over the warp
+        const float4 x = xf[s0 + p];
+        for (int f = lane; f < nb + lane; f += 32) {
+          const bool ok = f < nb;
+          const float4 q = sh.cand[ok ? f : 0];
+          const uint32_t e = sh.word[ok ? f : 0];
+          const int j = (int)(e & kIdxMask);
+          const float dx = q.x - x.x, dy = q.y - x.y, dz = q.z - x.z;
+          const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
+          bool in = ok && r2 < hi2 && (half ? j > s0 + p : j != s0 + p);
+          if (in && !(r2 < lo2)) {  // between the pre-test's thresholds: the exact FP64 test (rare)
+            const double4_32a xi = xs[s0 + p], xj = xs[j];
+            in = (exact_inside(xi.x, xi.y, xi.z, xj.x, xj.y, xj.z, e >> kIdxBits, Pp->L, Pp->rl2) & 0x100u) != 0u;
+          }
+          append(in, p, j, e, c[i]);
+        }
+      }
+      __syncthreads();  // before the next candidates
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int p = p0 + wv + kWideWarps * i;
+      if (p < p1) finish(p, c[i]);
+    }
+    p0 = p1;
+  }
+  return wmax;
+}
+
+__device__ __forceinline__ void build_lists_wide(const DevArrays& a, int cur, int span, WideShared& sh) {
+  const int nreb = reb_systems(a);
+  const int per = kTile / span;  // blocks' pieces per tile
+  const int total = a.reb_pref[nreb] * per;
+  for (int w = blockIdx.x; w < total; w += gridDim.x) {
+    int lo = 0, hi = nreb - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (a.reb_pref[mid] * per <= w) lo = mid;
+      else hi = mid - 1;
+    }
+    const int sys = a.rebuild_ids[lo];
+    const SysParams* __restrict__ Pp = a.params + sys;
+    const int s0 = (w - a.reb_pref[lo] * per) * span;
+    const int s1 = min(s0 + span, Pp->n);
+    if (!Pp->active || s0 >= s1) continue;  // uniform over the block
+    const int me = s0 + (int)threadIdx.x;
+    if (me < s1) copy_back_slot(a, cur, Pp->p_off + me);
+    const int wmax = build_span(a, cur, sys, Pp, s0, s1, sh);
+    if ((threadIdx.x & 31) == 0 && wmax > 0) {
+      atomicMax(&a.status[sys].max_count, wmax);
+      if (wmax > Pp->kmax) {
+        atomicMax(&a.status[sys].overflow, wmax);
+        if (a.ctl) atomicMax(&a.ctl->abort, 1);  // graph-captured loop: stop; the host grows the list
+      }
+    }
+    __syncthreads();  // before the next span's cells
+  }
+}
+
+}  // namespace
+
+__global__ void __launch_bounds__(kWideBlock, 4) k_build_list_wide(DevArrays a, int cur, int span) {
+  __shared__ WideShared sh;
+  build_lists_wide(a, cur, span, sh);
+}
+
 // ------------------------------------- fused force + velocity-Verlet step
 
 namespace {
@@ -2027,9 +2238,24 @@ static void launch_build_list_v(const DevArrays& a, int cur, int block, cudaStre
   }
 }
 
+// The one-candidate-per-lane build takes the passes of arenas up to 1,300 tiles, where it
+// is the faster one (rc 2.5, launch included): 22 against 74 us at 1000 particles, 24
+// against 85 at 4000, 43 against 88 at 16,000, 74 against 95 at 32,000; from there a
+// warp per tile fills the GPU (112 against 103 us at 64,000). Spans of 8 slots make
+// enough blocks of small arenas; larger ones read the candidates of fewer runs (4000
+// particles: 24 us at 8, 41 at 32; 32,000 particles: 94 at 8, 76 at 16, 74 at 32).
+constexpr int kWideMaxTiles = 1300;
+inline int wide_span(int ntiles) { return ntiles <= 152 ? 8 : ntiles <= 304 ? 16 : 32; }
+
 void launch_build_list(const DevArrays& a, int cur, const Tuning& tu, cudaStream_t s) {
   switch (tu.list_variant) {
     case 5:
+      if (a.ntiles <= kWideMaxTiles) {
+        const int span = wide_span(a.ntiles);
+        k_build_list_wide<<<(unsigned)std::max(1, std::min(a.ntiles * (kTile / span), kSMs * 8)), kWideBlock, 0, s>>>(
+            a, cur, span);
+        break;
+      }
       switch (tu.list_block) {
         case 64: k_build_list_staged<64><<<reb_blocks(a, 64, 16), 64, 0, s>>>(a, cur); break;
         case 256: k_build_list_staged<256><<<reb_blocks(a, 256, 4), 256, 0, s>>>(a, cur); break;
