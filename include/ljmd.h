@@ -286,8 +286,10 @@ MD_API int md_probe_fma_rate(int kind, int64_t iters, double* fma_per_s);
  *   MD_TUNE_GRAPH        1: md_step runs its steps in CUDA-graph launches (a loop node of
  *                        two steps, each followed by a device-side list-validity
  *                        decision and a conditional rebuild pass), reading the
- *                        control words once per launch; 0: the host decides after
- *                        every step. Results are identical. Timing (md_set_timing)
+ *                        control words once per launch; small full-list arenas (up to
+ *                        32 systems of at most about 30,000 particles together) run all
+ *                        steps of a call in one cooperative launch instead; 0: the host
+ *                        decides after every step. Results are identical. Timing (md_set_timing)
  *                        uses the host-driven loop.
  *   MD_TUNE_FP64_QUEUE   1: the FP64 force loops classify each listed pair on the
  *                        fixed-point shadow positions first and run the FP64

@@ -100,6 +100,7 @@ enum StepFlags : int {
 // DevArrays when the host drives the loop).
 struct GraphCtl {
   int32_t abort;   // 1: a pair list overflowed, 2: a non-finite value; the remaining steps do nothing
+                   // (3: a grid barrier of the persistent loop gave up)
   int32_t flags;   // StepFlags of the next step
   int32_t nreb;    // systems rebuilding in the current pass
   int32_t done;    // steps taken
@@ -108,6 +109,25 @@ struct GraphCtl {
   int32_t next_tile;  // list build's work counter
   int32_t pad_;
 };
+
+// Arguments of the persistent step loop of small arenas (k_loop).
+struct LoopArgs {
+  int cur;       // position buffer of the first step
+  int nsys;      // system records (at most kLoopMaxSys)
+  int fp32;      // force form
+  int vmax;      // velocity-bound rule
+  int stored;    // 1: the first step takes the stored forces
+  int steady;    // 1: the first step also completes the previous step's kick
+  int finish;    // 1: after the last step, forces (stored) and the closing half kick
+  int stride;    // list words per particle in shared memory
+  int lanes;     // threads per particle
+  int32_t* rebuild_ids;
+  int32_t* reb_pref;
+  int32_t* reb_count;
+  unsigned long long* disp;  // 3 maxima per system, taken in turn (zeroed before the launch)
+  unsigned* bar;             // grid barrier's arrival count (zeroed before the launch)
+};
+constexpr int kLoopMaxSys = 32;
 
 struct DevArrays {
   double4_32a* x[2];      // positions (w unused), ping-pong by step parity
@@ -212,6 +232,11 @@ void launch_build_list(const DevArrays& a, int cur, const Tuning& tu, cudaStream
 void launch_decide(const DevArrays& a, int nsys, int fp32, int vflag, int32_t* rebuild, int32_t* rebuild_ids,
                    int32_t* reb_pref, int32_t* reb_count, cudaGraphConditionalHandle h_if,
                    cudaGraphConditionalHandle h_loop, int last, cudaStream_t s);
+// Persistent step loop of small arenas: threads per particle for the given launch (0: the
+// arena does not fit; kmax: the longest list capacity) and the shared list stride.
+int loop_lanes(int fp32, int ntiles, int kmax, int* stride);
+// One cooperative launch that takes ctl->target steps, rebuilds included (see k_loop).
+cudaError_t launch_loop(const DevArrays& a, const LoopArgs& g, cudaStream_t s);
 // mode 0: FP64 reciprocal; 1..4: approximate reciprocal of Sec. 3.3 (8 bits,
 // 8 bits corrected, 23 bits, 23 bits corrected)
 void launch_step_fp64(const DevArrays& a, int cur, double ka, double kb, int flags, const Tuning& tu,

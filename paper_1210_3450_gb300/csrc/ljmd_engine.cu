@@ -303,7 +303,7 @@ void Engine::free_all() {
   dfree(d_obs_); dfree(d_stage_); dfree(d_pairs_); dfree(d_obs_work_); dfree(d_obs_chunk_);
   hfree(h_status_); hfree(h_disp2_); hfree(h_rebuild_); hfree(h_obs_); hfree(h_obs_work_);
   drop_graphs();
-  dfree(d_ctl_); dfree(d_reb_count_); hfree(h_ctl_); hfree(h_reb_count_);
+  dfree(d_ctl_); dfree(d_loop_); dfree(d_reb_count_); hfree(h_ctl_); hfree(h_reb_count_);
   d_ = DevArrays{};
   stage_n_ = 0;
 }
@@ -413,6 +413,7 @@ int Engine::alloc_arrays() {
   CK(cudaMallocHost((void**)&h_rebuild_, sizeof(int32_t) * (4 * ns + 2)));
   CK(cudaMallocHost((void**)&h_obs_, sizeof(double) * 3 * ns));
   CKR(dmalloc(&d_ctl_, 1));
+  CKR(dmalloc(&d_loop_, 1 + 3 * (int64_t)ns));
   CKR(dmalloc(&d_reb_count_, ns));
   CK(cudaMemset(d_ctl_, 0, sizeof(GraphCtl)));
   CK(cudaMallocHost((void**)&h_ctl_, sizeof(GraphCtl)));
@@ -1088,8 +1089,15 @@ int Engine::run_graph(int64_t nsteps, int first_flags, int64_t* done, cudaStream
   CKR(sync_check(s));
   const GraphCtl r = *h_ctl_;
   *done = r.done;
-  if (r.done & 1) cur_ ^= 1;
   n_launch_ += (half_ ? 3 : 2) * (int64_t)r.done + kRebuildLaunches * (int64_t)r.passes;
+  return after_steps(r.done, s);
+}
+
+// After a launch of several steps (control words, rebuild counts and status words read
+// back): the bookkeeping, errors, and a list that overflowed grown and rebuilt.
+int Engine::after_steps(int64_t done, cudaStream_t s) {
+  const GraphCtl r = *h_ctl_;
+  if (done & 1) cur_ ^= 1;
   n_rebuild_seq_ += r.passes;
   for (int k = 0; k < nsys(); ++k) {
     if (h_reb_count_[k] <= 0) continue;
@@ -1119,6 +1127,69 @@ int Engine::run_graph(int64_t nsteps, int first_flags, int64_t* done, cudaStream
   return kOK;
 }
 
+// Threads per particle of the persistent loop: full lists, at most kLoopMaxSys systems,
+// and for the FP64 form the fixed-point range of every system.
+int Engine::loop_plan() {
+  if (loop_ver_ == struct_ver_) return loop_lanes_;
+  loop_ver_ = struct_ver_;
+  loop_lanes_ = 0;
+  if (half_ || precision_ > 1 || nsys() > kLoopMaxSys) return 0;
+  int kmax = 0;
+  for (const SysHost& h : sys_) {
+    if (!h.used) continue;
+    kmax = std::max(kmax, h.kmax);
+    if (precision_ == 0 && (h.spec.rc > kFixMaxRc || h.kmax > kFixMaxList)) return 0;
+  }
+  if (precision_ == 0 && !d_.xl[0]) return 0;
+  loop_lanes_ = loop_lanes(precision_ == 1, ntiles_, kmax, &loop_stride_);
+  return loop_lanes_;
+}
+
+int Engine::run_loop(int64_t nsteps, bool stored, bool steady, int64_t* done, bool* finished, cudaStream_t s) {
+  *done = 0;
+  *finished = false;
+  GraphCtl c{};
+  c.target = (int32_t)nsteps;
+  *h_ctl_ = c;
+  CK(cudaMemcpyAsync(d_ctl_, h_ctl_, sizeof(GraphCtl), cudaMemcpyHostToDevice, s));
+  CK(cudaMemsetAsync(d_reb_count_, 0, sizeof(int32_t) * nsys(), s));
+  CK(cudaMemsetAsync(d_loop_, 0, sizeof(unsigned long long) * (1 + 3 * (size_t)nsys()), s));
+  DevArrays a = arrays();
+  a.ctl = d_ctl_;
+  LoopArgs g{};
+  g.cur = cur_;
+  g.nsys = nsys();
+  g.fp32 = precision_ == 1 ? 1 : 0;
+  g.vmax = rule_ == 1 ? 1 : 0;
+  g.stored = stored ? 1 : 0;
+  g.steady = steady ? 1 : 0;
+  g.finish = 1;
+  g.stride = loop_stride_;
+  g.lanes = loop_lanes_;
+  g.rebuild_ids = d_rebuild_ + nsys();
+  g.reb_pref = d_rebuild_ + 2 * nsys();
+  g.reb_count = d_reb_count_;
+  g.bar = (unsigned*)d_loop_;
+  g.disp = d_loop_ + 1;
+  const cudaError_t e = launch_loop(a, g, s);
+  if (e != cudaSuccess) {
+    set_error(std::string("persistent step loop: ") + cudaGetErrorString(e));
+    return kErrCuda;
+  }
+  CK(cudaMemcpyAsync(h_ctl_, d_ctl_, sizeof(GraphCtl), cudaMemcpyDeviceToHost, s));
+  CK(cudaMemcpyAsync(h_reb_count_, d_reb_count_, sizeof(int32_t) * nsys(), cudaMemcpyDeviceToHost, s));
+  CK(cudaMemcpyAsync(h_status_, d_status_, sizeof(SysStatus) * nsys(), cudaMemcpyDeviceToHost, s));
+  CKR(sync_check(s));
+  n_launch_ += 1;
+  if (h_ctl_->abort == 3) {
+    set_error("a grid barrier of the step loop gave up");
+    return kErrTimeout;
+  }
+  *done = h_ctl_->done;
+  *finished = h_ctl_->abort == 0;
+  return after_steps(*done, s);
+}
+
 int Engine::step(int64_t nsteps, const std::vector<double>& dt, cudaStream_t s) {
   if (nsteps < 0) { set_error("nsteps < 0"); return kErrArg; }
   if ((int)dt.size() != nsys()) { set_error("one dt per system required"); return kErrArg; }
@@ -1133,7 +1204,15 @@ int Engine::step(int64_t nsteps, const std::vector<double>& dt, cudaStream_t s) 
   CKR(ensure_forces(s));
   CK(cudaMemsetAsync(d_ctl_, 0, sizeof(GraphCtl), s));
   int64_t it = 0;
+  bool finished = false;
   if (graph_ && !timing_) {
+    while (it < nsteps && loop_plan() > 0) {
+      int64_t done = 0;
+      const int rc = run_loop(std::min<int64_t>(nsteps - it, 1 << 30), it == 0, it > 0, &done, &finished, s);
+      it += done;
+      if (rc != kOK) return rc;
+    }
+
     while (nsteps - it >= 2) {
       const int first = (it == 0 ? (kStepUseStoredF | kStepDrift | kStepKickB) : (kStepKickA | kStepKickB | kStepDrift)) |
                         (rule_ == 1 ? kStepVmax : 0);
@@ -1149,8 +1228,10 @@ int Engine::step(int64_t nsteps, const std::vector<double>& dt, cudaStream_t s) 
     cur_ ^= 1;
     CKR(post_drift(s));
   }
-  CKR(launch_step(0.5, 0.0, kStepStoreF, s));
-  CKR(sync_check(s));
+  if (!finished) {  // the closing half kick of the last step
+    CKR(launch_step(0.5, 0.0, kStepStoreF, s));
+    CKR(sync_check(s));
+  }
   for (SysHost& h : sys_) {
     if (!h.active) continue;
     h.f_valid = true;

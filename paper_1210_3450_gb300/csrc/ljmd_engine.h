@@ -186,6 +186,12 @@ class Engine {
   int build_graph(cudaGraph_t g, int parity);
   void drop_graphs();
   int run_graph(int64_t nsteps, int first_flags, int64_t* done, cudaStream_t s);
+  // Persistent step loop of small arenas (tuning key 5 as well): all steps of a call in
+  // one cooperative launch, the closing force evaluation included. loop_plan returns its
+  // threads per particle, 0 where the arena does not take it.
+  int loop_plan();
+  int run_loop(int64_t nsteps, bool stored, bool steady, int64_t* done, bool* finished, cudaStream_t s);
+  int after_steps(int64_t done, cudaStream_t s);
   int sync_check(cudaStream_t s);
   bool any_active() const;  // some system takes part in launches
   int read_checks(cudaStream_t s);  // checked build: MD_ERR_CHECK if a device check failed
@@ -218,6 +224,9 @@ class Engine {
   int64_t gver_[2] = {-1, -1};
   cudaStream_t cap_[2] = {nullptr, nullptr};
   GraphCtl* d_ctl_ = nullptr;
+  unsigned long long* d_loop_ = nullptr;  // persistent loop: barrier word, then 3 maxima per system
+  int loop_lanes_ = 0, loop_stride_ = 0;
+  int64_t loop_ver_ = -1;                 // struct_ver_ the plan was made for
   GraphCtl* h_ctl_ = nullptr;
   int32_t* d_reb_count_ = nullptr;
   int32_t* h_reb_count_ = nullptr;

@@ -105,13 +105,17 @@ __device__ __forceinline__ bool reb_tile(const DevArrays& a, int nreb, int w, Ti
 __device__ __forceinline__ int reb_systems(const DevArrays& a) { return a.ctl ? a.ctl->nreb : a.nreb; }
 
 // Rebuild passes visit only the tiles of the rebuilding systems, each warp
-// striding over them (a grid sized to the GPU, not to the arena).
-template <class F>
+// striding over them (a grid sized to the GPU, not to the arena). kSpread: consecutive
+// tiles go to different blocks (few tiles, spread over the SMs) and not to the warps of
+// one (many tiles, neighbours sharing L1).
+template <bool kSpread, class F>
 __device__ __forceinline__ void for_rebuild_tiles(const DevArrays& a, F&& body) {
   const int nreb = reb_systems(a);
   const int total = a.reb_pref[nreb];
   const int nw = (int)((gridDim.x * blockDim.x) >> 5);
-  for (int w = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); w < total; w += nw) {
+  const int w0 = kSpread ? (int)((threadIdx.x >> 5) * gridDim.x + blockIdx.x)
+                         : (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+  for (int w = w0; w < total; w += nw) {
     TileCtx t;
     SysParams P;
     if (reb_tile(a, nreb, w, t, P)) body(t, P);
@@ -183,8 +187,9 @@ __device__ __forceinline__ int warp_cell_add(int32_t* counts, int c) {
   return base + __popc(same & ((1u << (threadIdx.x & 31)) - 1u));  // this lane's place in the group
 }
 
-__global__ void k_cell_count(DevArrays a, int cur) {
-  for_rebuild_tiles(a, [&](const TileCtx& t, const SysParams& P) {
+template <bool kSpread>
+__device__ __forceinline__ void cell_count_pass(const DevArrays& a, int cur) {
+  for_rebuild_tiles<kSpread>(a, [&](const TileCtx& t, const SysParams& P) {
     // Positions are wrapped into [0, L) only here (at a list build): between
     // builds they move freely so that the periodic images stored in the list
     // stay valid.
@@ -208,6 +213,8 @@ __global__ void k_cell_count(DevArrays a, int cur) {
     }
   });
 }
+
+__global__ void k_cell_count(DevArrays a, int cur) { cell_count_pass<false>(a, cur); }
 
 // Exclusive scan of the cell counts of the rebuilding systems over chunks of
 // kScanChunk cells, so that a large system spreads over many blocks: the count
@@ -239,10 +246,8 @@ __device__ __forceinline__ int block_sum(int v, int* ws) {
   return t;
 }
 
-__global__ void __launch_bounds__(kScanBlock) k_cell_starts(DevArrays a, int nreb) {
-  if (a.ctl) nreb = a.ctl->nreb;
-  if (nreb <= 0) return;
-  __shared__ int ws[kScanBlock / 32];
+// ws holds kScanBlock / 32 ints.
+__device__ __forceinline__ void cell_starts_pass(const DevArrays& a, int nreb, int* ws) {
   const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
   const int total = a.chunk_pref[nreb];
   for (int w = blockIdx.x; w < total; w += gridDim.x) {
@@ -297,13 +302,21 @@ __global__ void __launch_bounds__(kScanBlock) k_cell_starts(DevArrays a, int nre
   }
 }
 
+__global__ void __launch_bounds__(kScanBlock) k_cell_starts(DevArrays a, int nreb) {
+  if (a.ctl) nreb = a.ctl->nreb;
+  if (nreb <= 0) return;
+  __shared__ int ws[kScanBlock / 32];
+  cell_starts_pass(a, nreb, ws);
+}
+
 // Scatter into cell order (arbitrary within a cell). Beside the old slot, the
 // scattered position receives the particle's sort key (x, then caller index) and
 // cell, so that the ranking below reads them contiguously (the caller index goes
 // to sid, the cell to the cell scratch).
 
-__global__ void k_scatter(DevArrays a, int cur) {
-  for_rebuild_tiles(a, [&](const TileCtx& t, const SysParams& P) {
+template <bool kSpread>
+__device__ __forceinline__ void scatter_pass(const DevArrays& a, int cur) {
+  for_rebuild_tiles<kSpread>(a, [&](const TileCtx& t, const SysParams& P) {
     if (P.nc == 1) {  // uniform over the warp
       if (t.act) a.perm[t.s] = t.local;
       return;
@@ -322,6 +335,8 @@ __global__ void k_scatter(DevArrays a, int cur) {
   });
 }
 
+__global__ void k_scatter(DevArrays a, int cur) { scatter_pass<false>(a, cur); }
+
 // Order the particles of each cell by x, ties by caller index (deterministic), and
 // gather each into its slot. A row of neighbouring cells along x is then sorted by
 // x as a whole, which lets the list build restrict each row to the window
@@ -333,8 +348,9 @@ __global__ void k_scatter(DevArrays a, int cur) {
 // slot (copy_back_slot). Every slot of a cell holds that cell in the scratch in
 // both orders, so the ranking's reads of it need no barrier. The first member of
 // each cell resets the cell's fill counter.
-__global__ void k_cell_rank(DevArrays a, int cur) {
-  for_rebuild_tiles(a, [&](const TileCtx& t, const SysParams& P) {
+template <bool kSpread>
+__device__ __forceinline__ void cell_rank_pass(const DevArrays& a, int cur) {
+  for_rebuild_tiles<kSpread>(a, [&](const TileCtx& t, const SysParams& P) {
     if (!t.act) return;
     const int p = t.local;           // position in the scattered order
     const int i = a.perm[t.s];       // the particle's slot before the rebuild
@@ -347,11 +363,15 @@ __global__ void k_cell_rank(DevArrays a, int cur) {
       if (p == lo) a.ccount[P.c_off + c] = 0;  // ready for the next binning
       const long long ki = key[p];
       const int32_t idi = idk[p];
-      int rank = 0;
+      int rank = 0, same = 0;
+#pragma unroll 4
       for (int q = lo; q < hi; ++q) {
         const long long kj = key[q];
-        rank += (kj < ki || (kj == ki && idk[q] < idi)) ? 1 : 0;
+        rank += kj < ki ? 1 : 0;
+        same += kj == ki ? 1 : 0;
       }
+      if (same > 1)  // equal keys (rare): by caller index
+        for (int q = lo; q < hi; ++q) rank += key[q] == ki && idk[q] < idi ? 1 : 0;
       if (!check_ok(a, t.sys, lo + rank < hi, kChkRank)) return;
       dst = lo + rank;
     }
@@ -369,6 +389,8 @@ __global__ void k_cell_rank(DevArrays a, int cur) {
     a.celltmp[d] = a.cell[old];
   });
 }
+
+__global__ void k_cell_rank(DevArrays a, int cur) { cell_rank_pass<false>(a, cur); }
 
 // The rebuilt state of one slot back into place. The list build does this for the
 // tiles it builds: it reads only the build-time positions, shadows and scratch
@@ -1075,11 +1097,13 @@ struct WideShared {
   float4 cand[kWideStage];
   uint32_t word[kWideStage];
   int cell[kTile];
+  int at[32], lo[32];    // pieces of the rows: place of the first candidate, its slot,
+  unsigned code[32];     // image code
 };
 
 // Slots [s0, s1) of system sys (within one tile, at most 32); called by the whole block
 // with uniform arguments. Returns the longest list of the warp's particles.
-__device__ __forceinline__ int build_span(const DevArrays& a, int cur, int sys, const SysParams* __restrict__ Pp,
+__device__ __forceinline__ int build_span(const DevArrays& a, int cur, int sys, const SysParams* Pp,
                                           int s0, int s1, WideShared& sh) {
   const int lane = threadIdx.x & 31, wv = threadIdx.x >> 5;
   const unsigned below = (1u << lane) - 1u;
@@ -1106,11 +1130,13 @@ __device__ __forceinline__ int build_span(const DevArrays& a, int cur, int sys, 
   };
   if (nc == 1) {  // every particle is a candidate, at its minimum image (as sweep_all)
     const int4* q = a.xq[cur] + p_off;
-    const float hi2 = Pp->rl2q_hi;
+    const float4* xf1 = a.xf + p_off;
+    const float hi2 = Pp->rl2q_hi, lo2q = Pp->rl2q_lo, hl = 0.5f * Pp->Lf;
     const int n = Pp->n;
     for (int p = wv; p < s1 - s0; p += kWideWarps) {
       const int i = s0 + p;
       const int4 qi = q[i];
+      const float4 fi = xf1[i];
       int c = 0;
       for (int j0 = 0; j0 < n; j0 += 32) {
         const int j = j0 + lane;
@@ -1121,11 +1147,21 @@ __device__ __forceinline__ int build_span(const DevArrays& a, int cur, int sys, 
           const float ax = (float)wrapped_diff(qj.x, qi.x);
           const float ay = (float)wrapped_diff(qj.y, qi.y);
           const float az = (float)wrapped_diff(qj.z, qi.z);
-          if (fmaf(az, az, fmaf(ay, ay, ax * ax)) < hi2) {
-            const double4_32a xi = xs[i], xj = xs[j];
-            const unsigned r = exact_inside(xi.x, xi.y, xi.z, xj.x, xj.y, xj.z, 0xffu, Pp->L, Pp->rl2);
-            in = (r & 0x100u) != 0u;
-            code = r & 0xffu;
+          const float r2 = fmaf(az, az, fmaf(ay, ay, ax * ax));
+          if (r2 < hi2) {
+            // images of the axes from the float separation, unless one is near L / 2
+            const float4 fj = xf1[j];
+            const float dx = fj.x - fi.x, dy = fj.y - fi.y, dz = fj.z - fi.z;
+            const float close = fminf(fabsf(fabsf(dx) - hl), fminf(fabsf(fabsf(dy) - hl), fabsf(fabsf(dz) - hl)));
+            code = (dx > hl ? 2u : (dx < -hl ? 1u : 0u)) | (dy > hl ? 8u : (dy < -hl ? 4u : 0u)) |
+                   (dz > hl ? 32u : (dz < -hl ? 16u : 0u));
+            in = true;
+            if (!(r2 < lo2q) || close < 1e-4f * hl) {  // the exact FP64 test
+              const double4_32a xi = xs[i], xj = xs[j];
+              const unsigned r = exact_inside(xi.x, xi.y, xi.z, xj.x, xj.y, xj.z, 0xffu, Pp->L, Pp->rl2);
+              in = (r & 0x100u) != 0u;
+              code = r & 0xffu;
+            }
           }
         }
         append(in, p, j, (uint32_t)j | (code << kIdxBits), c);
@@ -1134,7 +1170,7 @@ __device__ __forceinline__ int build_span(const DevArrays& a, int cur, int sys, 
     }
     return wmax;
   }
-  const float4* __restrict__ xf = a.xf + p_off;
+  const float4* xf = a.xf + p_off;
   const float lo2 = Pp->rl2f_lo, hi2 = Pp->rl2f_hi, Lf = Pp->Lf;
   if (wv == 0) sh.cell[lane] = s0 + lane < s1 ? a.celltmp[p_off + s0 + lane] : -1;
   __syncthreads();
@@ -1174,49 +1210,85 @@ __device__ __forceinline__ int build_span(const DevArrays& a, int cur, int sys, 
       if (lane >= o) at += y;
     }
     const int total = __shfl_sync(kFull, at, 31);
-    at -= hi - lo;
-    int c[4] = {0, 0, 0, 0};  // list lengths of the warp's particles p0 + wv + 8 i
+    // pieces without candidates share the next one's place: the bisection finds the last
+    // piece that starts at or before a candidate, which holds it
+    if (wv == 0) {
+      sh.at[lane] = lane < 18 ? at - (hi - lo) : 0x7fffffff;
+      sh.lo[lane] = lo;
+      sh.code[lane] = code;
+    }
+    __syncthreads();
+    // the warp's particles p0 + wv + 8 i and their list lengths
+    const int np = min(4, max(0, (p1 - p0 - wv + kWideWarps - 1) / kWideWarps));
+    int c[4] = {0, 0, 0, 0};
+    float px[4], py[4], pz[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float4 x = xf[s0 + min(p0 + wv + kWideWarps * i, p1 - 1)];
+      px[i] = x.x;
+      py[i] = x.y;
+      pz[i] = x.z;
+    }
     for (int base = 0; base < total; base += kWideStage) {
-      for (int l = wv; l < 18; l += kWideWarps) {
-        const int jlo = __shfl_sync(kFull, lo, l), jhi = __shfl_sync(kFull, hi, l);
-        const int f0 = __shfl_sync(kFull, at, l) - base - jlo;
-        const unsigned cd = __shfl_sync(kFull, code, l);
-        // image code 1 adds +L to x_j - x_i, code 2 adds -L: the candidate is shifted in
-        // float (the same bound as shifting the particle, 4 u L and u L for the other)
-        const float sx = (cd & 3u) == 1u ? Lf : ((cd & 3u) == 2u ? -Lf : 0.f);
-        const float sy = (cd & 12u) == 4u ? Lf : ((cd & 12u) == 8u ? -Lf : 0.f);
-        const float sz = (cd & 48u) == 16u ? Lf : ((cd & 48u) == 32u ? -Lf : 0.f);
-#pragma unroll 4
-        for (int j = jlo + lane; j < jhi; j += 32) {
-          const int f = f0 + j;
-          if ((unsigned)f < (unsigned)kWideStage) {
-            const float4 q = xf[j];
-            sh.cand[f] = make_float4(q.x + sx, q.y + sy, q.z + sz, 0.f);
-            sh.word[f] = (uint32_t)j | (cd << kIdxBits);
-          }
+      // thread t copies candidates t, t + 256, ...; a candidate's piece by bisection
+#pragma unroll
+      for (int u = 0; u < kWideStage / kWideBlock; ++u) {
+        const int t = u * kWideBlock + (int)threadIdx.x, f = base + t;
+        if (f < total) {
+          int l = 0;
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1)
+            if (sh.at[l + o] <= f) l += o;
+          const int j = sh.lo[l] + f - sh.at[l];
+          const unsigned cd = sh.code[l];
+          // image code 1 adds +L to x_j - x_i, code 2 adds -L: the candidate is shifted in
+          // float (the same bound as shifting the particle, 4 u L and u L for the other)
+          const float sx = (cd & 3u) == 1u ? Lf : ((cd & 3u) == 2u ? -Lf : 0.f);
+          const float sy = (cd & 12u) == 4u ? Lf : ((cd & 12u) == 8u ? -Lf : 0.f);
+          const float sz = (cd & 48u) == 16u ? Lf : ((cd & 48u) == 32u ? -Lf : 0.f);
+          const float4 q = xf[j];
+          sh.cand[t] = make_float4(q.x + sx, q.y + sy, q.z + sz, 0.f);
+          sh.word[t] = (uint32_t)j | (cd << kIdxBits);
         }
       }
+      const int nr = min(kWideStage, total - base), nb = (nr + 31) & ~31;
+      if (wv == kWideWarps - 1 && nr + lane < nb) {
+        sh.cand[nr + lane] = make_float4(1e18f, 0.f, 0.f, 0.f);
+        sh.word[nr + lane] = 0u;
+      }
       __syncthreads();
-      const int nb = min(kWideStage, total - base);
+      // rounds of 32 candidates (the last one filled up with candidates far away)
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
+        if (i >= np) break;  // uniform over the warp
         const int p = p0 + wv + kWideWarps * i;
-        if (p >= p1) break;  // uniform over the warp
-        const float4 x = xf[s0 + p];
-        for (int f = lane; f < nb + lane; f += 32) {
-          const bool ok = f < nb;
-          const float4 q = sh.cand[ok ? f : 0];
-          const uint32_t e = sh.word[ok ? f : 0];
-          const int j = (int)(e & kIdxMask);
-          const float dx = q.x - x.x, dy = q.y - x.y, dz = q.z - x.z;
+        const uint32_t self = (uint32_t)(s0 + p);
+        const int cut = half ? s0 + p : -1;  // half list: only candidates above the particle's slot
+        uint32_t* op = out + 4 * p;
+        int cnt = c[i];
+#pragma unroll 2
+        for (int f = lane; f < nb; f += 32) {  // nb + the filling: uniform over the warp
+          const float4 q = sh.cand[f];
+          const uint32_t e = sh.word[f];
+          const float dx = q.x - px[i], dy = q.y - py[i], dz = q.z - pz[i];
           const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-          bool in = ok && r2 < hi2 && (half ? j > s0 + p : j != s0 + p);
-          if (in && !(r2 < lo2)) {  // between the pre-test's thresholds: the exact FP64 test (rare)
-            const double4_32a xi = xs[s0 + p], xj = xs[j];
-            in = (exact_inside(xi.x, xi.y, xi.z, xj.x, xj.y, xj.z, e >> kIdxBits, Pp->L, Pp->rl2) & 0x100u) != 0u;
+          bool in = r2 < hi2 && e != self && (int)(e & kIdxMask) > cut;
+          if (__any_sync(kFull, in && !(r2 < lo2))) {  // between the pre-test's thresholds: the exact FP64 test (rare)
+            if (in && !(r2 < lo2)) {
+              const int j = (int)(e & kIdxMask);
+              const double4_32a xi = xs[s0 + p], xj = xs[j];
+              in = (exact_inside(xi.x, xi.y, xi.z, xj.x, xj.y, xj.z, e >> kIdxBits, Pp->L, Pp->rl2) & 0x100u) != 0u;
+            }
+            __syncwarp();
           }
-          append(in, p, j, e, c[i]);
+          if (kChecks && in)
+            in = check_ok(a, sys, (e & kIdxMask) < (uint32_t)Pp->n && (e & kIdxMask) != self, kChkListEntry);
+          const unsigned m = __ballot_sync(kFull, in);
+          const int k = cnt + __popc(m & below);
+          if (in && k < kmax) op[k + (k >> 2) * (4 * kTile - 4)] = e;
+          cnt += __popc(m);
         }
+        c[i] = cnt;
       }
       __syncthreads();  // before the next candidates
     }
@@ -1242,13 +1314,13 @@ __device__ __forceinline__ void build_lists_wide(const DevArrays& a, int cur, in
       else hi = mid - 1;
     }
     const int sys = a.rebuild_ids[lo];
-    const SysParams* __restrict__ Pp = a.params + sys;
+    const SysParams* Pp = a.params + sys;
     const int s0 = (w - a.reb_pref[lo] * per) * span;
     const int s1 = min(s0 + span, Pp->n);
     if (!Pp->active || s0 >= s1) continue;  // uniform over the block
-    const int me = s0 + (int)threadIdx.x;
-    if (me < s1) copy_back_slot(a, cur, Pp->p_off + me);
     const int wmax = build_span(a, cur, sys, Pp, s0, s1, sh);
+    const int me = s0 + (int)threadIdx.x;  // (not before: its loads would delay the candidates')
+    if (me < s1) copy_back_slot(a, cur, Pp->p_off + me);
     if ((threadIdx.x & 31) == 0 && wmax > 0) {
       atomicMax(&a.status[sys].max_count, wmax);
       if (wmax > Pp->kmax) {
@@ -1338,23 +1410,29 @@ __device__ __forceinline__ void warp_max_disp(const DevArrays& a, int sys, unsig
   if ((threadIdx.x & 31) == 0 && d2b) atomicMax(&a.disp2[sys], d2b);
 }
 
-// FP32 pair force from an exact fixed-point separation; returns 0 for invalid
-// slots, for r >= rc and for r = 0 (a list's padding entries name the particle
-// itself) without branching (g (24 r^-8 - 48 r^-14 + 8 c2)).
-__device__ __forceinline__ void pair_fp32(const int4& qi, const int4& qj, bool valid, float qu, float rc2,
-                                          float c2x8, float& fx, float& fy, float& fz) {
-  const float dx = (float)wrapped_diff(qj.x, qi.x) * qu;
-  const float dy = (float)wrapped_diff(qj.y, qi.y) * qu;
-  const float dz = (float)wrapped_diff(qj.z, qi.z) * qu;
+// FP32 pair force factor (24 r^-8 - 48 r^-14 + 8 c2) and separation from an exact
+// fixed-point separation; the factor is 0 for r >= rc and for r = 0 (a list's padding
+// entries name the particle itself), without branching.
+__device__ __forceinline__ float pair_factor_fp32(const int4& qi, const int4& qj, float qu, float rc2, float c2x8,
+                                                  float& dx, float& dy, float& dz) {
+  dx = (float)wrapped_diff(qj.x, qi.x) * qu;
+  dy = (float)wrapped_diff(qj.y, qi.y) * qu;
+  dz = (float)wrapped_diff(qj.z, qi.z) * qu;
   const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-  const bool in = valid && r2 < rc2 && r2 > 0.0f;
+  const bool in = r2 < rc2 && r2 > 0.0f;
   const float r2s = in ? r2 : 1.0f;
   float ir2;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(ir2) : "f"(r2s));
   ir2 = ir2 * fmaf(-r2s, ir2, 2.0f);  // one Newton step
   const float ir6 = ir2 * ir2 * ir2;
-  float g = fmaf(ir2 * ir6, fmaf(-48.0f, ir6, 24.0f), c2x8);
-  g = in ? g : 0.0f;
+  const float g = fmaf(ir2 * ir6, fmaf(-48.0f, ir6, 24.0f), c2x8);
+  return in ? g : 0.0f;
+}
+
+__device__ __forceinline__ void pair_fp32(const int4& qi, const int4& qj, float qu, float rc2, float c2x8, float& fx,
+                                          float& fy, float& fz) {
+  float dx, dy, dz;
+  const float g = pair_factor_fp32(qi, qj, qu, rc2, c2x8, dx, dy, dz);
   fx = fmaf(g, dx, fx);
   fy = fmaf(g, dy, fy);
   fz = fmaf(g, dz, fz);
@@ -1433,7 +1511,7 @@ __global__ void __launch_bounds__(BLOCK) k_step_fp32(DevArrays a, int cur, doubl
         q[4 * u + 3] = ld_shadow(qs + partner_slot(a, t.sys, e[u].w, P.n, self), HINT);
       }
 #pragma unroll
-      for (int m = 0; m < 4 * GROUPS; ++m) pair_fp32(qi, q[m], true, qu, rc2, c2x8, fx, fy, fz);
+      for (int m = 0; m < 4 * GROUPS; ++m) pair_fp32(qi, q[m], qu, rc2, c2x8, fx, fy, fz);
 #pragma unroll
       for (int u = 0; u < GROUPS; ++u) e[u] = en[u];
     }
@@ -1759,7 +1837,7 @@ __global__ void __launch_bounds__(BLOCK) k_force_half_fp32(DevArrays a, int cur,
     const uint32_t j = partner_slot(a, t.sys, __ldg(lp + (int64_t)(k >> 2) * (4 * kTile) + (k & 3)), P.n,
                                     (uint32_t)t.local);
     float px = 0.f, py = 0.f, pz = 0.f;
-    pair_fp32(qi, qs[j], true, qu, rc2, c2x8, px, py, pz);
+    pair_fp32(qi, qs[j], qu, rc2, c2x8, px, py, pz);
     fx += px;
     fy += py;
     fz += pz;
@@ -1989,6 +2067,489 @@ __global__ void __launch_bounds__(256) k_obs_final(const int32_t* __restrict__ w
     out3[3 * sys + 0] = sh[0][0];
     out3[3 * sys + 1] = sh[1][0];
     out3[3 * sys + 2] = sh[2][0];
+  }
+}
+
+// ------------------------------------ persistent step loop of small arenas
+
+// A step of a few thousand particles is a chain of latencies: in separate launches
+// (step, decision, conditional rebuild node, and five kernels per rebuild) it took 28 to
+// 33 us at 1000 to 32,000 particles with FP32 forces and 70 to 77 with FP64 ones, of which
+// the pair arithmetic is about 1 to 8. Here one cooperative launch takes all steps of a
+// call: 6.8, 9.9, 17 and 24 us at 1000, 4000, 16,000 and 32,000 particles (FP32 forces,
+// rebuilds included), 7.8, 11.5 and 26 us at 1000, 4000 and 16,000 (FP64). Without its
+// rebuilds a step of 4000 particles takes 5.0 us: forces 2.2, update 0.9, barrier 1.5,
+// decision 0.4; a rebuild 40 us. Several threads share a particle, whose
+// position, velocity and list stay in registers and shared memory between rebuilds; a
+// step reads the partners' shadows, writes the own one, and ends at a grid barrier,
+// after which every block takes the list-validity decision for itself from the
+// maxima. A rebuild runs the same passes as the separate kernels between barriers.
+//
+// Results are those of the other loops bit for bit: FP32 pair forces are formed by all
+// threads of the particle, exchanged through shared memory and added by one thread
+// per axis in list order; FP64 forces are exact integer sums (ljmd_fixed.cuh), and pairs
+// out of their range are added in list order.
+namespace {
+
+constexpr int kLoopBlock = 256;
+constexpr int kLoopWarps = kLoopBlock / 32;
+constexpr int kBarrierPolls = 1 << 21;  // about a second, then the launch gives up
+
+__host__ __device__ constexpr int loop_chunk(int T) { return T >= 32 ? 3 : 4; }  // pairs per thread between exchanges
+// FP32 exchange buffer of one particle (words; the 4 extra ones keep the particles of a
+// warp on different banks)
+__host__ __device__ constexpr int loop_ex(int T) { return loop_chunk(T) * T * 4 + 4; }
+__host__ __device__ constexpr size_t loop_union_bytes(int T) {
+  return sizeof(WideShared) > (size_t)loop_ex(T) * 4 * (kLoopBlock / T) ? sizeof(WideShared)
+                                                                       : (size_t)loop_ex(T) * 4 * (kLoopBlock / T);
+}
+
+// List words in shared memory: the FP32 form needs the partner's slot only (an arena of
+// the loop has fewer than 2^16).
+template <bool kFP32> struct LoopWord { using type = uint32_t; };
+template <> struct LoopWord<true> { using type = uint16_t; };
+
+struct LoopShared {
+  unsigned long long d2[kLoopWarps];
+  int sys[kLoopWarps];
+  double margin[kLoopMaxSys];
+  int need[kLoopMaxSys];
+  int ws[kScanBlock / 32];
+  int flag;  // barrier: 0 gave up
+};
+
+// Every block of the (cooperative) launch arrives before any passes. False if the wait
+// ran out; `target` counts this block's barriers in arrivals.
+__device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned& target, LoopShared& sh, GraphCtl* ctl) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    target += gridDim.x;
+    __threadfence();  // the block's writes (ordered before it by the barrier above)
+    atomicAdd(bar, 1u);
+    int polls = 0;
+    unsigned v;
+    do {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+    } while ((int)(v - target) < 0 && ++polls < kBarrierPolls);
+    sh.flag = polls < kBarrierPolls;
+    if (polls >= kBarrierPolls) atomicMax(&ctl->abort, 3);
+  }
+  __syncthreads();
+  return sh.flag != 0;
+}
+
+// Work lists of a rebuild pass (k_decide's, for at most 32 systems), by one warp.
+__device__ __forceinline__ void loop_worklists(const DevArrays& a, const LoopArgs& g, const int* need) {
+  const int lane = threadIdx.x & 31;
+  const int k = lane < g.nsys ? a.sys_order[lane] : -1;
+  const bool n = k >= 0 && need[k];
+  const unsigned m = __ballot_sync(kFull, n);
+  const int r = __popc(m & ((1u << lane) - 1u));
+  int tiles = 0, chunks = 0;
+  if (n) {
+    const SysParams& P = a.params[k];
+    tiles = P.ntiles;
+    chunks = scan_chunks((int64_t)P.nc * P.nc * P.nc);
+  }
+  int ti = tiles, ci = chunks;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(kFull, ti, o), z = __shfl_up_sync(kFull, ci, o);
+    if (lane >= o) { ti += y; ci += z; }
+  }
+  if (n) {
+    g.rebuild_ids[r] = k;
+    g.reb_pref[r] = ti - tiles;
+    a.chunk_pref[r] = ci - chunks;
+    g.reb_count[k] += 1;
+    const_cast<int32_t*>(a.rebuild)[k] = 1;
+    a.status[k].overflow = 0;
+    a.status[k].max_count = 0;
+  } else if (k >= 0) {
+    const_cast<int32_t*>(a.rebuild)[k] = 0;
+  }
+  const int call = __shfl_sync(kFull, ci, 31);
+  for (int q = lane; q < call * kChunkCopies; q += 32) a.chunk_sum[q] = 0;
+  if (lane == 31) {
+    const int nreb = __popc(m);
+    g.reb_pref[nreb] = ti;
+    a.chunk_pref[nreb] = ci;
+    a.ctl->nreb = nreb;
+    a.ctl->passes += 1;
+  }
+}
+
+// Separation pair in the FP64 form's fixed-point units; adds to the sums, returns true
+// if the pair is closer than the fixed-point range (the FP64 pipe takes it).
+__device__ __forceinline__ bool loop_fixed_pair(const SysParams& P, const longlong4_32a& qi, const longlong4_32a& qj,
+                                                unsigned code, long long rc2, long long c2, FixSum& sx, FixSum& sy,
+                                                FixSum& sz) {
+  long long dx = qj.x - qi.x, dy = qj.y - qi.y, dz = qj.z - qi.z;
+  if (code) {
+    const long long L = P.Lfix;
+    dx += (code & 3u) == 1u ? L : ((code & 3u) == 2u ? -L : 0);
+    dy += (code & 12u) == 4u ? L : ((code & 12u) == 8u ? -L : 0);
+    dz += (code & 48u) == 16u ? L : ((code & 48u) == 32u ? -L : 0);
+  }
+  const Fix2 fx = fix_split(dx), fy = fix_split(dy), fz = fix_split(dz);
+  const unsigned long long r2 = fix_r2(fx, fy, fz);
+  const bool far = (unsigned)(r2 >> 32) >= kFixR2Min;
+  if (far & ((long long)(r2 - (unsigned long long)rc2) < 0)) {
+    const Fix2 g = fix_split(fix_force_factor(fix_rcp(r2), c2));
+    sx.add(g, fx);
+    sy.add(g, fy);
+    sz.add(g, fz);
+  }
+  return !far;
+}
+
+}  // namespace
+
+template <bool kFP32, int T>
+__global__ void __launch_bounds__(kLoopBlock, T == 4 ? (kFP32 ? 4 : 3) : (kFP32 ? 3 : 2)) k_loop(DevArrays a, LoopArgs g) {
+  extern __shared__ __align__(32) unsigned char smem[];
+  __shared__ LoopShared sh;
+  constexpr int CH = loop_chunk(T);
+  float* ex_all = (float*)smem;
+  WideShared& wide = *(WideShared*)smem;
+  using Word = typename LoopWord<kFP32>::type;
+  Word* lists = (Word*)(smem + loop_union_bytes(T));
+
+  const int lane = threadIdx.x & 31, wv = threadIdx.x >> 5;
+  const int sub = lane & (T - 1);                    // place among the particle's threads
+  const int part = threadIdx.x / T;                  // particle of the block
+  const int64_t slot = ((int64_t)blockIdx.x * kLoopBlock + threadIdx.x) / T;
+  const int tile = (int)(slot / kTile);
+  const int sys = tile < a.ntiles ? a.tile_sys[tile] : -1;  // uniform over the warp
+  const SysParams& P = a.params[sys < 0 ? 0 : sys];
+  const bool on = sys >= 0 && P.active;
+  const int local = on ? (int)(slot - P.p_off) : 0;
+  const bool act = on && local < P.n;
+  const bool comp = act && sub < 3;  // this thread integrates axis `sub`
+  const int64_t p_off = on ? P.p_off : 0;
+  Word* list = lists + (size_t)part * g.stride;
+  float* ex = ex_all + (size_t)part * loop_ex(T);
+  const float qu = P.qunit, rc2f = P.rc2f, c2x8 = 8.0f * P.c2f;
+  const long long rc2x = P.rc2fix, c2x = P.c2fix;
+  const double dt = P.dt, h = P.hdt, qscale = P.qscale;
+
+  int cur = g.cur;
+  int niter = 0;                  // chunks of the warp's longest list
+  double x = 0.0, v = 0.0, refd = 0.0;
+  int q = 0, refq = 0;            // own shadow and its build-time value (FP32 form)
+  long long ql = 0;               // own position in pair units (FP64 form)
+  const int c = sub < 3 ? sub : 0;
+
+  // The particle's state and list, after a rebuild or at the start. Lists are padded
+  // with the particle itself to whole chunks.
+  auto load_state = [&]() {
+    int cnt = 0;
+    if (act) {
+      cnt = list_count(a, sys, slot, P.kmax);
+      if (sub < 3) {
+        x = ((const double*)&a.x[cur][slot])[c];
+        v = ((const double*)&a.v[slot])[c];
+        if (kFP32) {
+          q = ((const int*)&a.xq[cur][slot])[c];
+          refq = ((const int*)&a.xqref[slot])[c];
+        } else {
+          ql = ((const long long*)&a.xl[cur][slot])[c];
+          refd = ((const double*)&a.xref[slot])[c];
+        }
+      }
+    }
+    const int most = __reduce_max_sync(kFull, cnt);
+    niter = (most + CH * T - 1) / (CH * T);
+    const uint32_t* lp = a.nbr + (on ? list_word(P.l_off, local / kTile, P.kmax, local % kTile, 0) : 0);
+    for (int k = sub; k < niter * CH * T; k += T) {
+      uint32_t e = (uint32_t)local;
+      if (k < cnt) {
+        e = lp[(int64_t)(k >> 2) * (4 * kTile) + (k & 3)];
+        const uint32_t j = partner_slot(a, sys, e, P.n, (uint32_t)local);
+        e = kFP32 ? j : (e & ~kIdxMask) | j;
+      }
+      list[k] = (Word)e;
+    }
+    __syncwarp();
+  };
+
+  // Force on the particle (axis c) at the positions of buffer cur.
+  auto force = [&]() -> double {
+    if constexpr (kFP32) {
+      const int4* qs = a.xq[cur] + p_off;
+      int4 qi;
+      qi.x = __shfl_sync(kFull, q, 0, T);
+      qi.y = __shfl_sync(kFull, q, 1, T);
+      qi.z = __shfl_sync(kFull, q, 2, T);
+      float f = 0.f;
+      for (int it = 0; it < niter; ++it) {
+        int4 qj[CH];
+#pragma unroll
+        for (int u = 0; u < CH; ++u) qj[u] = qs[list[(it * CH + u) * T + sub]];
+#pragma unroll
+        for (int u = 0; u < CH; ++u) {
+          float4 d;
+          d.w = pair_factor_fp32(qi, qj[u], qu, rc2f, c2x8, d.x, d.y, d.z);
+          *(float4*)(ex + (u * T + sub) * 4) = d;
+        }
+        __syncwarp();
+        if (sub < 3) {
+#pragma unroll 8
+          for (int m = 0; m < CH * T; ++m) f = fmaf(ex[4 * m + 3], ex[4 * m + c], f);
+        }
+        __syncwarp();
+      }
+      return f2d_bits(f);
+    } else {
+      const longlong4_32a* qs = a.xl[cur] + p_off;
+      longlong4_32a qi;
+      qi.x = __shfl_sync(kFull, ql, 0, T) - kFixBias;
+      qi.y = __shfl_sync(kFull, ql, 1, T) - kFixBias;
+      qi.z = __shfl_sync(kFull, ql, 2, T) - kFixBias;
+      FixSum sx, sy, sz;
+      int slow = 0, k0 = 0x7fffffff, k1 = 0x7fffffff;  // this thread's pairs for the FP64 pipe
+#pragma unroll 1
+      for (int it = 0; it < niter; ++it) {
+        longlong4_32a qj[CH];
+        uint32_t e[CH];
+#pragma unroll
+        for (int u = 0; u < CH; ++u) {
+          e[u] = list[(it * CH + u) * T + sub];
+          qj[u] = qs[e[u] & kIdxMask];
+        }
+#pragma unroll
+        for (int u = 0; u < CH; ++u) {
+          if (e[u] == (uint32_t)local) continue;  // padding
+          if (loop_fixed_pair(P, qi, qj[u], e[u] >> kIdxBits, rc2x, c2x, sx, sy, sz)) {
+            if (slow == 0) k0 = (it * CH + u) * T + sub;
+            else if (slow == 1) k1 = (it * CH + u) * T + sub;
+            ++slow;
+          }
+        }
+      }
+#pragma unroll
+      for (int o = T / 2; o > 0; o >>= 1) {
+        FixSum* s3[3] = {&sx, &sy, &sz};
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+          const unsigned l = __shfl_xor_sync(kFull, s3[m]->lo, o);
+          const long long hh = __shfl_xor_sync(kFull, s3[m]->hi, o);
+          const unsigned t = s3[m]->lo + l;
+          s3[m]->hi += hh + (t < l ? 1 : 0);
+          s3[m]->lo = t;
+        }
+      }
+      double F = (c == 0 ? sx : c == 1 ? sy : sz).value24();
+      if (__any_sync(kFull, slow > 0)) {
+        // the FP64 pipe's pairs, in list order: the particle's threads take the lowest
+        // entry left among them each time (a thread with more than two goes through
+        // its whole list)
+        const long long rc2b = __double_as_longlong(P.rc2);
+        const double c8 = 8.0 * P.c2, L = P.L;
+        double S0 = 0.0, S1 = 0.0, S2 = 0.0;
+        const bool many = slow > 2;
+        int next = many ? sub : k0;
+        const int end = niter * CH * T;
+        while (true) {
+          if (many && next < end) {  // the next of this thread's entries that the fixed-point range leaves out
+            for (; next < end; next += T) {
+              const uint32_t e = list[next];
+              if (e == (uint32_t)local) continue;
+              FixSum t0, t1, t2;
+              if (loop_fixed_pair(P, qi, qs[e & kIdxMask], e >> kIdxBits, rc2x, c2x, t0, t1, t2)) break;
+            }
+          }
+          int low = next < end ? next : 0x7fffffff;
+#pragma unroll
+          for (int o = T / 2; o > 0; o >>= 1) low = min(low, __shfl_xor_sync(kFull, low, o));
+          if (!__any_sync(kFull, low != 0x7fffffff)) break;
+          if (low != 0x7fffffff) {
+            const uint32_t e = list[low];
+            const double4_32a xi = a.x[cur][slot], xj = a.x[cur][p_off + (e & kIdxMask)];
+            double dx = xj.x - xi.x, dy = xj.y - xi.y, dz = xj.z - xi.z;
+            const unsigned code = e >> kIdxBits;
+            if (code) {
+              dx = apply_image(dx, code & 3u, L);
+              dy = apply_image(dy, (code >> 2) & 3u, L);
+              dz = apply_image(dz, (code >> 4) & 3u, L);
+            }
+            const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
+            if (__double_as_longlong(r2) < rc2b) {
+              const double gg = force_factor<0>(r2, c8);
+              S0 = fma(gg, dx, S0);
+              S1 = fma(gg, dy, S1);
+              S2 = fma(gg, dz, S2);
+            }
+            if (next == low) next = many ? next + T : (next == k0 ? k1 : 0x7fffffff);
+          }
+          __syncwarp();
+        }
+        const double S = c == 0 ? S0 : c == 1 ? S1 : S2;
+        if (S0 != 0.0 || S1 != 0.0 || S2 != 0.0) F += S;
+      }
+      return F;
+    }
+  };
+
+  for (int k = threadIdx.x; k < g.nsys; k += kLoopBlock) sh.margin[k] = a.margin[k];
+  load_state();
+  const int target_steps = a.ctl->target;
+  unsigned arrivals = 0;
+  int done = 0, abort = 0;
+  bool alive = true;
+  // the decision's constants of system threadIdx.x
+  bool dactive = false;
+  double dthr = 0.0, ddt = 0.0;
+  if ((int)threadIdx.x < g.nsys) {
+    const SysParams& Q = a.params[threadIdx.x];
+    dactive = Q.active != 0;
+    dthr = kFP32 ? Q.disp_thr : Q.skin;
+    ddt = Q.dt;
+  }
+  __syncthreads();
+
+  while (done < target_steps) {
+    unsigned long long d2 = 0ull;
+    // block 0 clears the maximum of the next step: its last readers passed a barrier
+    if (blockIdx.x == 0 && (int)threadIdx.x < g.nsys) g.disp[((done + 1) % 3) * g.nsys + threadIdx.x] = 0ull;
+    if (on) {
+      const bool first = done == 0;
+      double F;
+      if (first && g.stored) F = comp ? ((const double*)&a.f[slot])[c] : 0.0;
+      else F = force();
+      bool fine = true;
+      long long s0 = 0;         // squared displacement of the axis (exact integer) ...
+      double sd = 0.0;          // ... or its FP64 square, or the squared velocity
+      if (comp) {
+        if (!first || g.steady) v = fma(h, F, v);
+        v = fma(h, F, v);
+        const double xn = fma(dt, v, x);
+        x = xn;
+        fine = finite_bits(xn) && finite_bits(v);
+        ((double*)&a.x[cur ^ 1][slot])[c] = xn;
+        if (kFP32) {
+          q = to_fixed(xn, qscale);
+          ((int*)&a.xq[cur ^ 1][slot])[c] = q;
+          const long long e = wrapped_diff(q, refq);
+          s0 = e * e;
+        } else {
+          ql = to_fix(xn);
+          ((long long*)&a.xl[cur ^ 1][slot])[c] = ql;
+          if (!g.vmax) {
+            const double e = __dsub_rn(xn, refd);
+            sd = __dmul_rn(e, e);
+          }
+        }
+        if (g.vmax) sd = __dmul_rn(v, v);
+      }
+      const unsigned bad = __ballot_sync(kFull, !fine);
+      if (kFP32 && !g.vmax) {
+        unsigned long long t = (unsigned long long)s0;
+        t += (unsigned long long)__shfl_down_sync(kFull, s0, 1, T);
+        t += (unsigned long long)__shfl_down_sync(kFull, s0, 2, T);
+        d2 = t;  // valid at sub == 0
+      } else {
+        const double y = __shfl_down_sync(kFull, sd, 1, T), z = __shfl_down_sync(kFull, sd, 2, T);
+        d2 = (unsigned long long)__double_as_longlong(__dadd_rn(__dadd_rn(sd, y), z));
+      }
+      if (sub != 0 || !act) d2 = 0ull;
+      if (bad) {
+        if (lane == 0) a.status[sys].nonfinite = 1;
+        d2 = ~0ull;
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long y = __shfl_xor_sync(kFull, d2, o);
+        d2 = y > d2 ? y : d2;
+      }
+    }
+    // one atomic per block and system (on one word they complete one after the other)
+    if (lane == 0) {
+      sh.d2[wv] = d2;
+      sh.sys[wv] = on ? sys : -1;
+    }
+    __syncthreads();
+    if (wv == 0) {
+      const int k = sh.sys[lane & (kLoopWarps - 1)];
+      unsigned long long m = sh.d2[lane & (kLoopWarps - 1)];
+      if (__all_sync(kFull, k == sh.sys[0])) {
+#pragma unroll
+        for (int o = kLoopWarps / 2; o > 0; o >>= 1) {
+          const unsigned long long y = __shfl_xor_sync(kFull, m, o);
+          m = y > m ? y : m;
+        }
+        if (lane == 0 && k >= 0 && m) atomicMax(&g.disp[(done % 3) * g.nsys + k], m);
+      } else if (lane < kLoopWarps && k >= 0 && m) {
+        atomicMax(&g.disp[(done % 3) * g.nsys + k], m);
+      }
+    }
+    if (!grid_barrier(g.bar, arrivals, sh, a.ctl)) { alive = false; break; }
+    // the list-validity decision (k_decide's)
+    bool need = false, stop = false;
+    if ((int)threadIdx.x < g.nsys) {
+      const int k = threadIdx.x;
+      if (dactive) {
+        const unsigned long long m2 = __ldcg(&g.disp[(done % 3) * g.nsys + k]);
+        stop = m2 == ~0ull;
+        if (g.vmax) {
+          const double m = __dsub_rn(sh.margin[k], __dmul_rn(__dmul_rn(2.0, __dsqrt_rn(__longlong_as_double((long long)m2))), ddt));
+          sh.margin[k] = m;
+          need = !(m > 0.0);
+        } else if (kFP32) {
+          need = __ull2double_rn(m2) >= dthr;
+        } else {
+          need = !(2.0 * __dsqrt_rn(__longlong_as_double((long long)m2)) < dthr);
+        }
+      }
+      sh.need[k] = need ? 1 : 0;
+    }
+    cur ^= 1;
+    ++done;
+    if (__syncthreads_or(stop)) { abort = 2; break; }
+    if (!__syncthreads_or(need)) continue;
+    // rebuild pass
+    const bool mine = on && sh.need[sys];
+    if (mine && comp) {
+      ((double*)&a.x[cur][slot])[c] = x;
+      ((double*)&a.v[slot])[c] = v;
+    }
+    if (blockIdx.x == 0 && wv == 0) loop_worklists(a, g, sh.need);
+    if (!(alive = grid_barrier(g.bar, arrivals, sh, a.ctl))) break;
+    cell_count_pass<true>(a, cur);
+    if (!(alive = grid_barrier(g.bar, arrivals, sh, a.ctl))) break;
+    cell_starts_pass(a, a.ctl->nreb, sh.ws);
+    if (!(alive = grid_barrier(g.bar, arrivals, sh, a.ctl))) break;
+    scatter_pass<true>(a, cur);
+    if (!(alive = grid_barrier(g.bar, arrivals, sh, a.ctl))) break;
+    cell_rank_pass<true>(a, cur);
+    if (!(alive = grid_barrier(g.bar, arrivals, sh, a.ctl))) break;
+    build_lists_wide(a, cur, T == 32 ? 8 : T == 16 ? 16 : 32, wide);
+    if (!(alive = grid_barrier(g.bar, arrivals, sh, a.ctl))) break;
+    if ((int)threadIdx.x < g.nsys && sh.need[threadIdx.x]) sh.margin[threadIdx.x] = a.margin[threadIdx.x];
+    if (mine) load_state();
+    abort = *(volatile int*)&a.ctl->abort;
+    __syncthreads();
+    if (abort) break;  // a list overflowed: the host grows it (uniform over the grid)
+  }
+
+  double F = 0.0;
+  const bool close = alive && abort == 0 && g.finish;
+  if (close && on) {
+    F = force();
+    if (comp) v = fma(h, F, v);
+  }
+  if (comp) {
+    ((double*)&a.x[cur][slot])[c] = x;
+    ((double*)&a.v[slot])[c] = v;
+    if (!kFP32) ((int*)&a.xq[cur][slot])[c] = to_fixed(x, qscale);
+    if (close) ((double*)&a.f[slot])[c] = F;
+  }
+  if (blockIdx.x == 0) {
+    if ((int)threadIdx.x < g.nsys) a.margin[threadIdx.x] = sh.margin[threadIdx.x];
+    if (threadIdx.x == 0) {
+      a.ctl->done = done;
+      if (abort) atomicMax(&a.ctl->abort, abort);
+    }
   }
 }
 
@@ -2347,6 +2908,70 @@ void launch_step_fp32(const DevArrays& a, int cur, double ka, double kb, int fla
 #undef LJMD_STEP32B
 #undef LJMD_STEP32
 }
+namespace {
+template <bool kFP32, int T>
+cudaError_t loop_setup(int kmax, int* stride, size_t* bytes, int* blocks_per_sm) {
+  const int unit = loop_chunk(T) * T;
+  int st = (kmax + unit - 1) / unit * unit;  // whole chunks, the particles of a warp on different banks
+  st += (T - st % 32 + 32) % 32;
+  *stride = st;
+  *bytes = loop_union_bytes(T) + sizeof(typename LoopWord<kFP32>::type) * (size_t)st * (kLoopBlock / T);
+  cudaError_t e = cudaFuncSetAttribute(k_loop<kFP32, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*bytes);
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_loop<kFP32, T>, kLoopBlock, *bytes);
+  return e;
+}
+template <bool kFP32>
+cudaError_t loop_setup(int T, int kmax, int* stride, size_t* bytes, int* bps) {
+  switch (T) {
+    case 32: return loop_setup<kFP32, 32>(kmax, stride, bytes, bps);
+    case 16: return loop_setup<kFP32, 16>(kmax, stride, bytes, bps);
+    case 8: return loop_setup<kFP32, 8>(kmax, stride, bytes, bps);
+    default: return loop_setup<kFP32, 4>(kmax, stride, bytes, bps);
+  }
+}
+template <bool kFP32>
+const void* loop_kernel(int T) {
+  return T == 32 ? (const void*)k_loop<kFP32, 32> : T == 16 ? (const void*)k_loop<kFP32, 16>
+         : T == 8 ? (const void*)k_loop<kFP32, 8> : (const void*)k_loop<kFP32, 4>;
+}
+unsigned loop_blocks(int ntiles, int T) { return (unsigned)(((int64_t)ntiles * kTile * T + kLoopBlock - 1) / kLoopBlock); }
+}  // namespace
+
+// The most threads per particle whose blocks are all resident at once: 32 and 16 up to
+// two blocks per SM (2,432 and 4,864 particles), 8 and 4 up to what fits (three or four
+// blocks of the FP32 form, 38,912 particles; three of the FP64 form, 29,184).
+int loop_lanes(int fp32, int ntiles, int kmax, int* stride) {
+  int dev = 0, sms = 0;
+  if (ntiles <= 0 || (int64_t)ntiles * kTile > 65535 /* LoopWord */ || cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  for (int T : {32, 16, 8, 4}) {
+    size_t bytes = 0;
+    int bps = 0;
+    const cudaError_t e = fp32 ? loop_setup<true>(T, kmax, stride, &bytes, &bps) : loop_setup<false>(T, kmax, stride, &bytes, &bps);
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      continue;
+    }
+    if (T >= 16) bps = std::min(bps, 2);
+    if (loop_blocks(ntiles, T) <= (unsigned)(sms * bps)) return T;
+  }
+  return 0;
+}
+
+cudaError_t launch_loop(const DevArrays& a, const LoopArgs& g, cudaStream_t s) {
+  DevArrays ac = a;
+  LoopArgs gc = g;
+  void* args[] = {&ac, &gc};
+  const void* fn = g.fp32 ? loop_kernel<true>(g.lanes) : loop_kernel<false>(g.lanes);
+  const size_t word = g.fp32 ? sizeof(LoopWord<true>::type) : sizeof(LoopWord<false>::type);
+  const size_t bytes = loop_union_bytes(g.lanes) + word * (size_t)g.stride * (kLoopBlock / g.lanes);
+  return cudaLaunchCooperativeKernel(fn, dim3(loop_blocks(a.ntiles, g.lanes)), dim3(kLoopBlock), args, bytes, s);
+}
+
 void launch_pe_virial(const DevArrays& a, int cur, int with_pairs, const int32_t* select, cudaStream_t s) {
   k_pe_virial<<<tile_blocks(a), kBlock, 0, s>>>(a, cur, with_pairs, select);
 }
