@@ -23,7 +23,10 @@
 //                         reach their range)
 // Pairs closer than sqrt(0.84) and lists longer than kFixMaxList take the FP64 pipe.
 #pragma once
+#include <cuda_runtime.h>
 #include <stdint.h>
+
+#include <cmath>
 
 namespace ljmd {
 
@@ -150,6 +153,70 @@ static __device__ __forceinline__ long long fix_force_factor(unsigned long long 
   return g;
 }
 
+// y^3 (units 2^-61) and the square of a fraction a < 2^31.4 / 2^32 of its range (units
+// 2^-2u of the high words: y^3 in 2^-61 gives y^6 in 2^-58).
+static __device__ __forceinline__ unsigned long long fix_y3(unsigned long long y) {
+  unsigned long long r;
+  asm("{\n\t"
+      ".reg .u64 c, p;\n\t"
+      ".reg .u32 y0, y1, a0, a1, c0, c1, z;\n\t"
+      "mov.b64 {y0, y1}, %1;\n\t"
+      "mul.wide.u32 c, y1, y0;\n\t"
+      "shr.u64 c, c, 31;\n\t"
+      "mad.wide.u32 p, y1, y1, c;\n\t"
+      "mov.b64 {a0, a1}, p;\n\t"
+      "mul.wide.u32 c, y1, a0;\n\t"
+      "mad.wide.u32 c, y0, a1, c;\n\t"
+      "mov.b64 {c0, c1}, c;\n\t"
+      "mov.u32 z, 0;\n\t"
+      "mov.b64 c, {c1, z};\n\t"
+      "mad.wide.u32 %0, y1, a1, c;\n\t"
+      "}"
+      : "=l"(r)
+      : "l"(y));
+  return r;
+}
+static __device__ __forceinline__ unsigned long long fix_sqr(unsigned long long a) {
+  unsigned long long r;
+  asm("{\n\t"
+      ".reg .u64 c;\n\t"
+      ".reg .u32 a0, a1;\n\t"
+      "mov.b64 {a0, a1}, %1;\n\t"
+      "mul.wide.u32 c, a1, a0;\n\t"
+      "shr.u64 c, c, 31;\n\t"
+      "mad.wide.u32 %0, a1, a1, c;\n\t"
+      "}"
+      : "=l"(r)
+      : "l"(a));
+  return r;
+}
+
+// Exact sum of 64-bit non-negative terms in 128 bits.
+struct FixAcc {
+  unsigned long long lo = 0ull, hi = 0ull;
+  __device__ __forceinline__ void add(unsigned long long v) {
+    lo += v;
+    hi += lo < v ? 1ull : 0ull;
+  }
+  // Adds the sum of the lane o away (all 32 lanes of the warp call it).
+  __device__ __forceinline__ void join(int o) {
+    const unsigned long long l = __shfl_xor_sync(0xffffffffu, lo, o), h = __shfl_xor_sync(0xffffffffu, hi, o);
+    lo += l;
+    hi += h + (lo < l ? 1ull : 0ull);
+  }
+  // The sum x 2^-unit as FP64 (rounded to nearest, halves up; unit at most 900), by
+  // integer operations.
+  __device__ __forceinline__ double value(int unit) const {
+    if ((lo | hi) == 0ull) return 0.0;
+    const int z = hi ? __clzll((long long)hi) : 64 + __clzll((long long)lo);
+    // the top 64 bits, normalised: sum = m 2^(64 - z)
+    const unsigned long long m = z == 0 ? hi : z < 64 ? (hi << z) | (lo >> (64 - z)) : lo << (z - 64);
+    const unsigned long long r = (m >> 11) + ((m >> 10) & 1ull);  // 53 bits; may round up to 2^53
+    const int ex = 1023 + 52 + 11 + 64 - z - unit;
+    return __longlong_as_double((long long)(((unsigned long long)(ex - 1) << 52) + r));
+  }
+};
+
 // 96-bit sum of products g d (units 2^-84: g 2^-56, d 2^-60).
 struct FixSum {
   unsigned lo = 0u;   // units of 2^-84
@@ -173,6 +240,14 @@ struct FixSum {
         "}"
         : "+r"(lo), "+l"(hi)
         : "r"(g.h), "r"(g.l), "r"(d.h), "r"(d.l));
+  }
+  // Adds the sum of the lane o away (all 32 lanes of the warp call it).
+  __device__ __forceinline__ void join(int o) {
+    const unsigned l = __shfl_xor_sync(0xffffffffu, lo, o);
+    const long long h = __shfl_xor_sync(0xffffffffu, hi, o);
+    const unsigned t = lo + l;
+    hi += h + (t < l ? 1 : 0);
+    lo = t;
   }
   // 24 x the sum as FP64, formed with integer operations (the FP64 pipe's conversions
   // would cost more than the pairs of three rounds).
@@ -199,5 +274,53 @@ struct FixSum {
     return __longlong_as_double((long long)(b | (hi < 0 ? 0x8000000000000000ull : 0ull)));
   }
 };
+
+// Separation qj - qi plus the periodic image `code` (two bits per axis: 1 adds L, 2
+// subtracts it), split; qi comes minus kFixBias.
+static __device__ __forceinline__ void fix_separation(const longlong4_32a& qi, const longlong4_32a& qj, unsigned code,
+                                                      long long L, Fix2& fx, Fix2& fy, Fix2& fz) {
+  long long dx = qj.x - qi.x, dy = qj.y - qi.y, dz = qj.z - qi.z;
+  if (code) {
+    dx += (code & 3u) == 1u ? L : ((code & 3u) == 2u ? -L : 0);
+    dy += (code & 12u) == 4u ? L : ((code & 12u) == 8u ? -L : 0);
+    dz += (code & 48u) == 16u ? L : ((code & 48u) == 32u ? -L : 0);
+  }
+  fx = fix_split(dx);
+  fy = fix_split(dy);
+  fz = fix_split(dz);
+}
+static __device__ __forceinline__ unsigned long long fix_separation2(const longlong4_32a& qi, const longlong4_32a& qj,
+                                                                     unsigned code, long long L) {
+  Fix2 fx, fy, fz;
+  fix_separation(qi, qj, code, L, fx, fy, fz);
+  return fix_r2(fx, fy, fz);
+}
+
+// One pair: where r < rc, its force is added to the sums (qi, code, L as above; rc2 in
+// units of 2^-56, c2_3b as for fix_force_factor). Returns true, with
+// nothing added, for a pair closer than the range (the FP64 pipe takes it).
+static __device__ __forceinline__ bool fix_pair(const longlong4_32a& qi, const longlong4_32a& qj, unsigned code,
+                                                long long L, long long rc2, long long c2_3b, FixSum& sx, FixSum& sy,
+                                                FixSum& sz) {
+  Fix2 fx, fy, fz;
+  fix_separation(qi, qj, code, L, fx, fy, fz);
+  const unsigned long long r2 = fix_r2(fx, fy, fz);
+  const bool far = (unsigned)(r2 >> 32) >= kFixR2Min;
+  if (far & ((long long)(r2 - (unsigned long long)rc2) < 0)) {
+    const Fix2 g = fix_split(fix_force_factor(fix_rcp(r2), c2_3b));
+    sx.add(g, fx);
+    sy.add(g, fy);
+    sz.add(g, fz);
+  }
+  return !far;
+}
+
+// x >= 2^-8 in position units (host; exact).
+static inline long long fix_host(double x) {
+  int e = 0;
+  const unsigned long long m = (unsigned long long)std::ldexp(std::frexp(x, &e), 53);  // x = m 2^(e - 53)
+  const int sh = e - 53 + 60;
+  return (long long)(sh >= 64 ? 0ull : sh >= 0 ? m << sh : m >> -sh);
+}
 
 }  // namespace ljmd
