@@ -74,7 +74,7 @@ struct SysParams {
   int32_t active;    // 1 if the system takes part in the current launches
   int32_t rule;      // list validity: 0 displacement (2 d_max >= skin), 1 velocity bound (DUTC)
   int32_t half;      // 1: half list (each pair once, in its lower slot's list; Newton's third law)
-  int32_t fixed;     // 1: the FP64 form's pair arithmetic runs in 64-bit fixed point (rc <= kFixMaxRc)
+  int32_t fixed;     // 1: the cutoff is in the range of the 64-bit fixed-point pair arithmetic (rc <= kFixMaxRc)
 };
 
 // Per-system status words written by kernels and read by the host.

@@ -75,14 +75,6 @@ int cells_per_axis(double L, double rl) {
   return nc >= 3 ? nc : 1;
 }
 
-// x >= 2^-8 in fixed-point pair units (2^-60, modulo 2^64), exact.
-long long host_to_fix(double x) {
-  int e = 0;
-  const unsigned long long m = (unsigned long long)std::ldexp(std::frexp(x, &e), 53);  // x = m 2^(e - 53)
-  const int sh = e - 53 + 60;
-  return (long long)(sh >= 64 ? 0ull : sh >= 0 ? m << sh : m >> -sh);
-}
-
 int initial_kmax(const SysSpec& s, double rl) {
   const double rho = (double)s.n / (s.L * s.L * s.L);
   const double expect = 4.0 / 3.0 * M_PI * rl * rl * rl * rho;
@@ -580,8 +572,8 @@ int Engine::upload_params(int only) {
       P.rl2f_lo = std::nextafter((float)(P.rl2 * (1.0 - eps)), 0.0f);
       P.rl2f_hi = std::nextafter((float)(P.rl2 * (1.0 + eps)), 3.0e38f);
     }
-    P.Lfix = host_to_fix(h.spec.L);
-    P.fixed = h.spec.rc <= kFixMaxRc && precision_ == 0 && !half_ ? 1 : 0;
+    P.Lfix = fix_host(h.spec.L);
+    P.fixed = h.spec.rc <= kFixMaxRc ? 1 : 0;
     if (P.fixed) {
       P.rc2fix = (long long)std::llrint(std::ldexp(P.rc2, 56));
       P.c2fix = (long long)std::llrint(std::ldexp(h.c2 / 3.0, 56)) + kFixBias;

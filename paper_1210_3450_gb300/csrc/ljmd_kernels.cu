@@ -133,8 +133,10 @@ __global__ void k_from_caller(DevArrays a, int cur, const double* __restrict__ x
   if (l >= (int64_t)P.ntiles * kTile) return;
   const int64_t s = P.p_off + l;
   if (l < P.n) {
-    a.x[cur][s] = make_double4_32a(wrap_full(x[3 * l + 0], P.L), wrap_full(x[3 * l + 1], P.L),
-                               wrap_full(x[3 * l + 2], P.L), 0.0);
+    // (wrap_fast: the FP64 divisions of the full wrap only for positions outside the box;
+    // 29 against 7 us for 262,143 particles)
+    a.x[cur][s] = make_double4_32a(wrap_fast(x[3 * l + 0], P.L), wrap_fast(x[3 * l + 1], P.L),
+                               wrap_fast(x[3 * l + 2], P.L), 0.0);
     a.v[s] = make_double4_32a(v[3 * l + 0], v[3 * l + 1], v[3 * l + 2], 0.0);
     a.id[s] = (int32_t)l;
   } else {
@@ -1585,8 +1587,9 @@ constexpr int kQueue64 = 32;  // queued list words per thread (FP64 pair loops)
 // every lane with partners left has queued, so the warp votes once per pass and
 // not once per round. qme points at the thread's queue column (entry q at
 // qme[q * BLOCK]).
+// kUpper: only partners in higher slots (each pair of a full list once).
 constexpr int kClassify = 7;
-template <int BLOCK, class Load, class Pair>
+template <int BLOCK, bool kUpper, class Load, class Pair>
 __device__ __forceinline__ void queued_pairs(const DevArrays& a, const TileCtx& t, const SysParams& P, int lane,
                                              int cur, int cnt, uint32_t* qme, Load&& load, Pair&& pair) {
   const uint4* lp4 = (const uint4*)(a.nbr + list_word(P.l_off, t.tl, P.kmax, lane, 0));
@@ -1608,12 +1611,14 @@ __device__ __forceinline__ void queued_pairs(const DevArrays& a, const TileCtx& 
       if (k < cnt) w = __ldg(lp4 + (int64_t)(k >> 2) * kTile);  // the next group's load in flight
 #pragma unroll
       for (int m = 0; m < 4; ++m) {
-        const int4 qj = qs[partner_slot(a, t.sys, ws[m], P.n, self)];
+        const uint32_t j = partner_slot(a, t.sys, ws[m], P.n, self);
+        if (kUpper && j <= self) continue;
+        const int4 qj = qs[j];
         const float ax = (float)wrapped_diff(qj.x, qi.x);
         const float ay = (float)wrapped_diff(qj.y, qi.y);
         const float az = (float)wrapped_diff(qj.z, qi.z);
         // the list's padding entries name the particle itself
-        if (ws[m] != self && fmaf(az, az, fmaf(ay, ay, ax * ax)) < rc2q) {
+        if ((kUpper || ws[m] != self) && fmaf(az, az, fmaf(ay, ay, ax * ax)) < rc2q) {
           qme[(tail & (kQueue64 - 1)) * BLOCK] = ws[m];
           ++tail;
         }
@@ -1686,24 +1691,7 @@ struct PairForce {
   __device__ __forceinline__ void pair(const longlong4_32a& qj, uint32_t e) {
     const unsigned code = e >> kIdxBits;
     if (MODE == 0 && fixed) {
-      long long dx = qj.x - qi.x, dy = qj.y - qi.y, dz = qj.z - qi.z;
-      if (code) {
-        const long long L = P.Lfix;
-        dx += (code & 3u) == 1u ? L : ((code & 3u) == 2u ? -L : 0);
-        dy += (code & 12u) == 4u ? L : ((code & 12u) == 8u ? -L : 0);
-        dz += (code & 48u) == 16u ? L : ((code & 48u) == 32u ? -L : 0);
-      }
-      const Fix2 fx = fix_split(dx), fy = fix_split(dy), fz = fix_split(dz);
-      const unsigned long long r2 = fix_r2(fx, fy, fz);
-      const bool far = (unsigned)(r2 >> 32) >= kFixR2Min;
-      if (far & ((long long)(r2 - (unsigned long long)P.rc2fix) < 0)) {
-        const Fix2 g = fix_split(fix_force_factor(fix_rcp(r2), P.c2fix));
-        sx.add(g, fx);
-        sy.add(g, fy);
-        sz.add(g, fz);
-      } else if (!far) {
-        fp64_pair(slot(e), code);
-      }
+      if (fix_pair(qi, qj, code, P.Lfix, P.rc2fix, P.c2fix, sx, sy, sz)) fp64_pair(slot(e), code);
     } else {
       fp64_pair(slot(e), code);
     }
@@ -1744,7 +1732,7 @@ __global__ void __launch_bounds__(BLOCK, MODE == 0 ? 1024 / BLOCK : 1) k_step_fp
     const int cnt = t.act ? list_count(a, t.sys, t.s, P.kmax) : 0;
     PairForce<MODE> pf(a, t, P, cur, cnt, &slow[0][threadIdx.x], BLOCK);
     if (QUEUE) {
-      queued_pairs<BLOCK>(a, t, P, lane, cur, cnt, &qbuf[0][threadIdx.x], [&](uint32_t e) { return pf.load(e); },
+      queued_pairs<BLOCK, false>(a, t, P, lane, cur, cnt, &qbuf[0][threadIdx.x], [&](uint32_t e) { return pf.load(e); },
                           [&](const longlong4_32a& q, uint32_t e) { pf.pair(q, e); });
     } else {
       const uint32_t* lp = a.nbr + list_word(P.l_off, t.tl, P.kmax, lane, 0);
@@ -1880,84 +1868,127 @@ __global__ void __launch_bounds__(kBlock) k_integrate_half(DevArrays a, int cur,
 
 // ------------------------------------------------- observables (FP64 sums)
 
-// Per particle: 1/2 sum_j V(r) and 1/2 sum_j -r V'(r) over listed partners with
-// r < rc (the full list counts each pair twice; a half list once, without the
-// 1/2), and 1/2 |v|^2; each tile sums its 32 values in a fixed shuffle order into
-// tile_obs[3 t ...]. With V(r) = 4 (r^-12 - r^-6) + 4 c2 r^2 + 4 c0 (Eq. 1) and
-// -r V'(r) = 48 r^-12 - 24 r^-6 - 8 c2 r^2, the pair loop only sums r^-12, r^-6
-// and r^2 and counts the pairs inside rc. Like the FP64 force loop it classifies
-// the listed pairs on the fixed-point shadows first and runs the FP64 arithmetic
-// (6 operations for the separation and r^2, 9 for a pair inside rc; the periodic
-// image added only where the list word names one, the cutoff tested on bit
-// patterns, r^2 >= 0) in full-warp rounds from per-thread queues; the sums keep
-// list order, so the results equal a plain loop's bit for bit.
+// Potential energy and virial of the pairs with r < rc, and 1/2 |v|^2: each tile sums its
+// particles' shares into tile_obs[3 t ...]. With V(r) = 4 (r^-12 - r^-6) + 4 c2 r^2 + 4 c0
+// (Eq. 1) and -r V'(r) = 48 r^-12 - 24 r^-6 - 8 c2 r^2, the pair loop only sums r^-12, r^-6
+// and r^2 and counts the pairs inside rc. A full list holds each pair twice: the
+// particle in its lower slot takes it. Like the FP64 force loop it classifies the
+// listed pairs on the fixed-point shadows and runs the others from per-thread queues, in
+// fixed point (ljmd_fixed.cuh; sums exact, over the tile as well) where the cutoff
+// allows it, else and for close pairs on the FP64 pipe. With all pairs on that pipe and
+// each taken twice the kernel ran at its rate: 455 us at 262,143 particles.
+// xl: positions in pair units.
 __global__ void __launch_bounds__(kBlock) k_pe_virial(DevArrays a, int cur, int with_pairs,
-                                                      const int32_t* __restrict__ select) {
+                                                      const int32_t* __restrict__ select, const longlong4_32a* xl) {
   __shared__ uint32_t qbuf[kQueue64][kBlock];
   TileCtx t;
-  SysParams P;
-  if (!tile_ctx(a, t, P)) return;           // uniform over the warp
+  if (!tile_ref(a, t)) return;              // uniform over the warp
   if (select && !select[t.sys]) return;     // uniform over the warp
+  const SysParams& P = a.params[t.sys];
   const int lane = threadIdx.x & 31;
   double pe = 0.0, w = 0.0, ke = 0.0;
   if (with_pairs) {  // every lane takes part (inactive ones with an empty list)
-    const double4_32a xi = t.act ? a.x[cur][t.s] : make_double4_32a(0.0, 0.0, 0.0, 0.0);
     const double4_32a* xs = a.x[cur] + P.p_off;
+    const longlong4_32a* ls = xl + P.p_off;
     const int cnt = t.act ? list_count(a, t.sys, t.s, P.kmax) : 0;
-    const long long rc2b = __double_as_longlong(P.rc2);
-    const long long tinyb = __double_as_longlong(1e-30);
-    const double L = P.L;
     const uint32_t self = (uint32_t)t.local;
-    double s12 = 0.0, s6 = 0.0, sr = 0.0;
+    const bool fixed = P.fixed != 0;  // uniform over the warp
+    longlong4_32a qi = fixed && t.act ? ls[t.local] : longlong4_32a{0, 0, 0, 0};
+    qi.x -= kFixBias; qi.y -= kFixBias; qi.z -= kFixBias;
+    FixAcc a12, a6, ar;
+    double s12 = 0.0, s6 = 0.0, sr = 0.0;  // the FP64 pipe's pairs
     int nin = 0;
-    auto load = [&](uint32_t e) { return xs[partner_slot(a, t.sys, e, P.n, self)]; };
-    queued_pairs<kBlock>(a, t, P, lane, cur, cnt, &qbuf[0][threadIdx.x], load, [&](const double4_32a& xj, uint32_t e) {
+    bool slow = false;
+    auto fp64_pair = [&](uint32_t j, unsigned code) {
+      const double4_32a xi = xs[t.local], xj = xs[j];
       double dx = xj.x - xi.x, dy = xj.y - xi.y, dz = xj.z - xi.z;
-      const unsigned code = e >> kIdxBits;
       if (code) {
-        dx = apply_image(dx, code & 3u, L);
-        dy = apply_image(dy, (code >> 2) & 3u, L);
-        dz = apply_image(dz, (code >> 4) & 3u, L);
+        dx = apply_image(dx, code & 3u, P.L);
+        dy = apply_image(dy, (code >> 2) & 3u, P.L);
+        dz = apply_image(dz, (code >> 4) & 3u, P.L);
       }
       const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
       const long long r2b = __double_as_longlong(r2);
-      if (r2b < rc2b) {
+      if (r2b < __double_as_longlong(P.rc2)) {
         // reciprocal within rounding in 3 DFMA (see rcp_f64); IEEE division only for
         // (near-)coincident pairs, outside rcp_f64's range
-        const double ir2 = r2b > tinyb ? rcp_f64(r2) : 1.0 / r2;
+        const double ir2 = r2b > __double_as_longlong(1e-30) ? rcp_f64(r2) : 1.0 / r2;
         const double ir6 = ir2 * ir2 * ir2;
         s12 = fma(ir6, ir6, s12);
         s6 += ir6;
         sr += r2;
         ++nin;
+        slow = true;
+      }
+    };
+    auto load = [&](uint32_t e) {
+      if (fixed) return ls[partner_slot(a, t.sys, e, P.n, self)];
+      return longlong4_32a{0, 0, 0, 0};
+    };
+    queued_pairs<kBlock, true>(a, t, P, lane, cur, cnt, &qbuf[0][threadIdx.x], load, [&](const longlong4_32a& qj, uint32_t e) {
+      const unsigned code = e >> kIdxBits;
+      if (fixed) {
+        const unsigned long long r2 = fix_separation2(qi, qj, code, P.Lfix);
+        const bool far = (unsigned)(r2 >> 32) >= kFixR2Min;
+        if (far & ((long long)(r2 - (unsigned long long)P.rc2fix) < 0)) {
+          const unsigned long long y3 = fix_y3(fix_rcp(r2));
+          a12.add(fix_sqr(y3));
+          a6.add(y3);
+          ar.add(r2);
+          ++nin;
+        } else if (!far) {
+          fp64_pair(partner_slot(a, t.sys, e, P.n, self), code);
+        }
+      } else {
+        fp64_pair(partner_slot(a, t.sys, e, P.n, self), code);
       }
     });
-    if (t.act) {
-      const double c2 = P.c2;
-      pe = 4.0 * (s12 - s6) + 4.0 * fma(c2, sr, P.c0 * (double)nin);
-      w = 48.0 * s12 - 24.0 * s6 - 8.0 * c2 * sr;
-      if (!P.half) {  // the full list counts each pair twice
-        pe *= 0.5;
-        w *= 0.5;
-      }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      a12.join(o);
+      a6.join(o);
+      ar.join(o);
     }
+    nin = __reduce_add_sync(kFull, nin);
+    if (__any_sync(kFull, slow)) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        s12 += __shfl_xor_sync(kFull, s12, o);
+        s6 += __shfl_xor_sync(kFull, s6, o);
+        sr += __shfl_xor_sync(kFull, sr, o);
+      }
+      s12 += a12.value(58);
+      s6 += a6.value(61);
+      sr += ar.value(56);
+    } else {
+      s12 = a12.value(58);
+      s6 = a6.value(61);
+      sr = ar.value(56);
+    }
+    const double c2 = P.c2;
+    pe = 4.0 * (s12 - s6) + 4.0 * fma(c2, sr, P.c0 * (double)nin);
+    w = 48.0 * s12 - 24.0 * s6 - 8.0 * c2 * sr;
   }
   if (t.act) {
     const double4_32a v = a.v[t.s];
     ke = 0.5 * (v.x * v.x + v.y * v.y + v.z * v.z);
   }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    pe += __shfl_xor_sync(kFull, pe, o);
-    w += __shfl_xor_sync(kFull, w, o);
-    ke += __shfl_xor_sync(kFull, ke, o);
-  }
+  for (int o = 16; o > 0; o >>= 1) ke += __shfl_xor_sync(kFull, ke, o);
   if (lane == 0) {
     const int64_t g = (int64_t)(P.t_off + t.tl) * 3;
     a.tile_obs[g + 0] = pe;
     a.tile_obs[g + 1] = w;
     a.tile_obs[g + 2] = ke;
   }
+}
+
+// Positions in pair units into scratch (the rebuild's gathered velocities, free between
+// rebuilds), for forms that do not keep them up: cheaper than converting each partner.
+__global__ void __launch_bounds__(kBlock) k_fix_positions(DevArrays a, int cur, const int32_t* __restrict__ select) {
+  TileCtx t;
+  if (!tile_ref(a, t) || !t.act || (select && !select[t.sys])) return;
+  reinterpret_cast<longlong4_32a*>(a.vtmp)[t.s] = fix4(a.x[cur][t.s]);
 }
 
 // Counts of listed pairs and of listed pairs with r < rc (FP64 test), per system.
@@ -2179,30 +2210,6 @@ __device__ __forceinline__ void loop_worklists(const DevArrays& a, const LoopArg
   }
 }
 
-// Separation pair in the FP64 form's fixed-point units; adds to the sums, returns true
-// if the pair is closer than the fixed-point range (the FP64 pipe takes it).
-__device__ __forceinline__ bool loop_fixed_pair(const SysParams& P, const longlong4_32a& qi, const longlong4_32a& qj,
-                                                unsigned code, long long rc2, long long c2, FixSum& sx, FixSum& sy,
-                                                FixSum& sz) {
-  long long dx = qj.x - qi.x, dy = qj.y - qi.y, dz = qj.z - qi.z;
-  if (code) {
-    const long long L = P.Lfix;
-    dx += (code & 3u) == 1u ? L : ((code & 3u) == 2u ? -L : 0);
-    dy += (code & 12u) == 4u ? L : ((code & 12u) == 8u ? -L : 0);
-    dz += (code & 48u) == 16u ? L : ((code & 48u) == 32u ? -L : 0);
-  }
-  const Fix2 fx = fix_split(dx), fy = fix_split(dy), fz = fix_split(dz);
-  const unsigned long long r2 = fix_r2(fx, fy, fz);
-  const bool far = (unsigned)(r2 >> 32) >= kFixR2Min;
-  if (far & ((long long)(r2 - (unsigned long long)rc2) < 0)) {
-    const Fix2 g = fix_split(fix_force_factor(fix_rcp(r2), c2));
-    sx.add(g, fx);
-    sy.add(g, fy);
-    sz.add(g, fz);
-  }
-  return !far;
-}
-
 }  // namespace
 
 template <bool kFP32, int T>
@@ -2320,7 +2327,7 @@ __global__ void __launch_bounds__(kLoopBlock, T == 4 ? (kFP32 ? 4 : 3) : (kFP32 
 #pragma unroll
         for (int u = 0; u < CH; ++u) {
           if (e[u] == (uint32_t)local) continue;  // padding
-          if (loop_fixed_pair(P, qi, qj[u], e[u] >> kIdxBits, rc2x, c2x, sx, sy, sz)) {
+          if (fix_pair(qi, qj[u], e[u] >> kIdxBits, P.Lfix, rc2x, c2x, sx, sy, sz)) {
             if (slow == 0) k0 = (it * CH + u) * T + sub;
             else if (slow == 1) k1 = (it * CH + u) * T + sub;
             ++slow;
@@ -2329,15 +2336,9 @@ __global__ void __launch_bounds__(kLoopBlock, T == 4 ? (kFP32 ? 4 : 3) : (kFP32 
       }
 #pragma unroll
       for (int o = T / 2; o > 0; o >>= 1) {
-        FixSum* s3[3] = {&sx, &sy, &sz};
-#pragma unroll
-        for (int m = 0; m < 3; ++m) {
-          const unsigned l = __shfl_xor_sync(kFull, s3[m]->lo, o);
-          const long long hh = __shfl_xor_sync(kFull, s3[m]->hi, o);
-          const unsigned t = s3[m]->lo + l;
-          s3[m]->hi += hh + (t < l ? 1 : 0);
-          s3[m]->lo = t;
-        }
+        sx.join(o);
+        sy.join(o);
+        sz.join(o);
       }
       double F = (c == 0 ? sx : c == 1 ? sy : sz).value24();
       if (__any_sync(kFull, slow > 0)) {
@@ -2356,7 +2357,7 @@ __global__ void __launch_bounds__(kLoopBlock, T == 4 ? (kFP32 ? 4 : 3) : (kFP32 
               const uint32_t e = list[next];
               if (e == (uint32_t)local) continue;
               FixSum t0, t1, t2;
-              if (loop_fixed_pair(P, qi, qs[e & kIdxMask], e >> kIdxBits, rc2x, c2x, t0, t1, t2)) break;
+              if (fix_pair(qi, qs[e & kIdxMask], e >> kIdxBits, P.Lfix, rc2x, c2x, t0, t1, t2)) break;
             }
           }
           int low = next < end ? next : 0x7fffffff;
@@ -2973,7 +2974,9 @@ cudaError_t launch_loop(const DevArrays& a, const LoopArgs& g, cudaStream_t s) {
 }
 
 void launch_pe_virial(const DevArrays& a, int cur, int with_pairs, const int32_t* select, cudaStream_t s) {
-  k_pe_virial<<<tile_blocks(a), kBlock, 0, s>>>(a, cur, with_pairs, select);
+  const longlong4_32a* xl = a.xl[0] ? a.xl[cur] : reinterpret_cast<const longlong4_32a*>(a.vtmp);
+  if (with_pairs && !a.xl[0]) k_fix_positions<<<tile_blocks(a), kBlock, 0, s>>>(a, cur, select);
+  k_pe_virial<<<tile_blocks(a), kBlock, 0, s>>>(a, cur, with_pairs, select, xl);
 }
 
 // v *= factor for every particle of the systems with scale[sys] != 1.

@@ -64,3 +64,29 @@ def test_forces_at_the_edges(name):
             assert cnt.min() <= 448 < cnt.max()
     np.testing.assert_array_equal(got[0], got[1])
     assert np.abs(got[0] - ref).max() <= 1e-12 * rms
+
+
+@pytest.mark.parametrize("precision", [0, 1], ids=["fp64", "fp32"])
+@pytest.mark.parametrize("half", [False, True], ids=["full", "half"])
+@pytest.mark.parametrize("name", ["close", "cutoff", "far corner", "long lists", "rc 4.0", "small"])
+def test_energy_and_virial_at_the_edges(name, half, precision):
+    """Potential energy and virial (each pair once, fixed-point sums) within 1e-12 of the
+    oracle's, relative to the sum of the pairs' magnitudes."""
+    from paper_1210_3450_gb300 import LJSystem
+    from paper_1210_3450_gb300.ljmd import MD_LIST_HALF
+    x, box, rc = _case(name)
+    v = li.maxwell_boltzmann(len(x), 1.0, 3)
+    d = x[:, None, :] - x[None, :, :]
+    d -= box * np.round(d / box)
+    r2 = (d ** 2).sum(2)[np.triu_indices(len(x), 1)]
+    r2 = r2[r2 < rc * rc]
+    scale = (4 * r2 ** -6 + 4 * r2 ** -3).sum(), (48 * r2 ** -6 + 24 * r2 ** -3).sum()
+    ref = oracle.observables(x, v, box, rc)
+    with LJSystem(box, len(x), rc, 0.3, precision) as s:
+        if half:
+            s.set_pair_list(MD_LIST_HALF)
+        s.set_state(x, v)
+        got = s.observables()
+    assert abs(got["pe"] - ref["pe"]) <= 1e-12 * scale[0]
+    assert abs(got["virial"] - ref["virial"]) <= 1e-12 * scale[1]
+    assert abs(got["ke"] - ref["ke"]) <= 1e-12 * ref["ke"]
