@@ -110,6 +110,12 @@ struct GraphCtl {
   int32_t pad_;
 };
 
+// Nose-Hoover thermostat of one system (device-resident during md_step_nvt).
+struct Thermo {
+  double dt, gT, Q;    // time step, 3 (N - 1) T, thermostat mass
+  double zeta, eta;    // thermostat velocity and position
+};
+
 // Arguments of the persistent step loop of small arenas (k_loop).
 struct LoopArgs {
   int cur;       // position buffer of the first step
@@ -126,6 +132,13 @@ struct LoopArgs {
   int32_t* reb_count;
   unsigned long long* disp;  // 3 maxima per system, taken in turn (zeroed before the launch)
   unsigned* bar;             // grid barrier's arrival count (zeroed before the launch)
+  // Nose-Hoover steps (thermo != NULL): the launch starts with a thermostat half step if
+  // `open` is set, then takes `halves_end` half steps after its last step (two after each
+  // other one); ke: 3 x 4 limbs of the kinetic-energy sums per system, taken in turn
+  // (zeroed before the launch)
+  Thermo* thermo;
+  unsigned long long* ke;
+  int open, halves_end;
 };
 constexpr int kLoopMaxSys = 32;
 
@@ -249,6 +262,10 @@ void launch_step_fp32(const DevArrays& a, int cur, double ka, double kb, int fla
 // select: per-system flags (NULL = every active system)
 void launch_pe_virial(const DevArrays& a, int cur, int with_pairs, const int32_t* select, cudaStream_t s);
 void launch_scale_v(const DevArrays& a, const double* scale, cudaStream_t s);
+// `halves` thermostat half steps of every active system: kinetic energies (4 limbs per
+// system in ke, zero before and after), factors into scale, velocities scaled.
+void launch_thermostat(const DevArrays& a, int nsys, Thermo* thermo, int halves, unsigned long long* ke, double* scale,
+                       cudaStream_t s);
 void launch_pair_stats(const DevArrays& a, int cur, unsigned long long* out2, cudaStream_t s);
 // Per-system (PE, W, KE) sums into out3[3 sys] for the nsel systems listed in work
 // (ids, then the prefix of their 256-tile chunk counts; nchunks in total); chunk3

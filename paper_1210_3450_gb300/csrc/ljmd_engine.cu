@@ -287,7 +287,8 @@ int footprint(const SysSpec& s, SysFootprint* f, SysHost* h) {
 // ------------------------------------------------------------- arena
 
 void Engine::free_all() {
-  for (int b = 0; b < 2; ++b) { dfree(d_.x[b]); dfree(d_.xq[b]); dfree(d_.xl[b]); }
+  for (int b = 0; b < 2; ++b) { dfree(d_.x[b]); dfree(d_.xq[b]); }
+  dfree(d_.xl[0]);
   dfree(d_.v); dfree(d_.xref); dfree(d_.xqref); dfree(d_.f); dfree(d_.facc); dfree(d_.id); dfree(d_.cell); dfree(d_.ncnt);
   dfree(d_.nbr); dfree(d_.tile_obs); dfree(d_.skey); dfree(d_.xf); dfree(d_.vtmp); dfree(d_.idtmp);
   dfree(d_.celltmp); dfree(d_.perm); dfree(d_.sid); dfree(d_.ccount); dfree(d_.cstart); dfree(d_.chunk_sum);
@@ -405,7 +406,9 @@ int Engine::alloc_arrays() {
   CK(cudaMallocHost((void**)&h_rebuild_, sizeof(int32_t) * (4 * ns + 2)));
   CK(cudaMallocHost((void**)&h_obs_, sizeof(double) * 3 * ns));
   CKR(dmalloc(&d_ctl_, 1));
-  CKR(dmalloc(&d_loop_, 1 + 3 * (int64_t)ns));
+  // barrier word, maxima and energy limbs; behind them the thermostats
+  CKR(dmalloc(&d_loop_, 1 + 15 * (int64_t)ns + (int64_t)ns * (int64_t)(sizeof(Thermo) / sizeof(unsigned long long))));
+  d_thermo_ = (Thermo*)(d_loop_ + 1 + 15 * (size_t)ns);
   CKR(dmalloc(&d_reb_count_, ns));
   CK(cudaMemset(d_ctl_, 0, sizeof(GraphCtl)));
   CK(cudaMallocHost((void**)&h_ctl_, sizeof(GraphCtl)));
@@ -418,10 +421,8 @@ int Engine::alloc_arrays() {
 // The FP64 form's positions in pair units (its full lists only).
 int Engine::ensure_fixed() {
   if (precision_ != 0 || half_ || d_.xl[0]) return kOK;
-  for (int b = 0; b < 2; ++b) {
-    CKR(dmalloc(&d_.xl[b], caps_.slots));
-    CK(cudaMemset(d_.xl[b], 0, sizeof(longlong4_32a) * caps_.slots));
-  }
+  CKR(dmalloc(&d_.xl[0], 2 * caps_.slots));  // (every slot is written by a rebuild before it is read)
+  d_.xl[1] = d_.xl[0] + caps_.slots;
   ++struct_ver_;
   return kOK;
 }
@@ -1137,7 +1138,8 @@ int Engine::loop_plan() {
   return loop_lanes_;
 }
 
-int Engine::run_loop(int64_t nsteps, bool stored, bool steady, int64_t* done, bool* finished, cudaStream_t s) {
+int Engine::run_loop(int64_t nsteps, bool stored, bool steady, int64_t* done, bool* finished, cudaStream_t s,
+                     bool nvt, bool open, int halves_end) {
   *done = 0;
   *finished = false;
   GraphCtl c{};
@@ -1145,7 +1147,7 @@ int Engine::run_loop(int64_t nsteps, bool stored, bool steady, int64_t* done, bo
   *h_ctl_ = c;
   CK(cudaMemcpyAsync(d_ctl_, h_ctl_, sizeof(GraphCtl), cudaMemcpyHostToDevice, s));
   CK(cudaMemsetAsync(d_reb_count_, 0, sizeof(int32_t) * nsys(), s));
-  CK(cudaMemsetAsync(d_loop_, 0, sizeof(unsigned long long) * (1 + 3 * (size_t)nsys()), s));
+  CK(cudaMemsetAsync(d_loop_, 0, sizeof(unsigned long long) * (1 + 15 * (size_t)nsys()), s));
   DevArrays a = arrays();
   a.ctl = d_ctl_;
   LoopArgs g{};
@@ -1163,6 +1165,13 @@ int Engine::run_loop(int64_t nsteps, bool stored, bool steady, int64_t* done, bo
   g.reb_count = d_reb_count_;
   g.bar = (unsigned*)d_loop_;
   g.disp = d_loop_ + 1;
+  if (nvt) {
+    g.thermo = d_thermo_;
+    g.ke = d_loop_ + 1 + 3 * (size_t)nsys();
+    g.open = open ? 1 : 0;
+    g.halves_end = halves_end;
+    g.finish = 0;
+  }
   const cudaError_t e = launch_loop(a, g, s);
   if (e != cudaSuccess) {
     set_error(std::string("persistent step loop: ") + cudaGetErrorString(e));
@@ -1322,36 +1331,58 @@ int Engine::step_nvt(int64_t nsteps, const std::vector<double>& dt, const std::v
     }
   }
   if (nsteps == 0 || !any_active()) return kOK;
-  std::vector<double> o3((size_t)(3 * ns)), fac((size_t)ns, 1.0);
-  // `halves` consecutive thermostat half steps from one kinetic-energy reduction:
-  // each is zeta += dt/4 G, eta += dt/2 zeta, v *= exp(-dt/2 zeta), zeta += dt/4 G'
-  // with G = (2 KE - g T) / Q, g = 3 (N - 1); a uniform scale multiplies KE by its
-  // square, so the next G needs no new reduction. One velocity scaling at the end.
-  auto thermostat = [&](int halves) -> int {
-    CKR(observables(o3.data(), s, false));
-    for (int k = 0; k < ns; ++k) {
-      fac[(size_t)k] = 1.0;
-      if (!sys_[k].active) continue;
-      const double g = 3.0 * (double)(sys_[k].spec.n - 1);
-      double ke = o3[(size_t)(3 * k + 2)];
-      for (int h = 0; h < halves; ++h) {
-        zeta[k] += 0.25 * dt[k] * (2.0 * ke - g * T[k]) / Q[k];
-        eta[k] += 0.5 * dt[k] * zeta[k];
-        const double sc = std::exp(-0.5 * dt[k] * zeta[k]);
-        fac[(size_t)k] *= sc;
-        ke = ke * sc * sc;
-        zeta[k] += 0.25 * dt[k] * (2.0 * ke - g * T[k]) / Q[k];
-      }
-    }
-    return scale_velocities(fac, s);
-  };
+  // The thermostats run on the device (launch_thermostat, or inside the persistent loop):
+  // kinetic energy, thermostat update and scaling need no word from the host.
+  std::vector<Thermo> th((size_t)ns);
+  for (int k = 0; k < ns; ++k) {
+    th[(size_t)k] = Thermo{dt[k], 3.0 * (double)(sys_[k].spec.n - 1) * T[k], Q[k], zeta[k], eta[k]};
+    if (sys_[k].active) sys_[k].dt = dt[k];
+  }
+  CKR(upload_params());
   CKR(ensure_lists(s));
-  if (nsteps == 0) return kOK;
-  CKR(thermostat(1));
-  for (int64_t it = 0; it < nsteps; ++it) {
+  CKR(ensure_forces(s));
+  CK(cudaMemcpyAsync(d_thermo_, th.data(), sizeof(Thermo) * (size_t)ns, cudaMemcpyHostToDevice, s));
+  unsigned long long* ke = d_loop_ + 1 + 3 * (size_t)ns;
+  CK(cudaMemsetAsync(ke, 0, sizeof(unsigned long long) * 4 * (size_t)ns, s));
+  auto thermostat = [&](int halves) -> int {
+    launch_thermostat(arrays(), ns, d_thermo_, halves, ke, d_obs_, s);
+    CKL();
+    n_launch_ += 3;
+    return kOK;
+  };
+  int64_t it = 0;
+  bool opened = false;
+  while (it < nsteps && graph_ && !timing_ && loop_plan() > 0) {
+    int64_t done = 0;
+    bool finished = false;
+    const int rc = run_loop(std::min<int64_t>(nsteps - it, 1 << 30), true, false, &done, &finished, s, true, !opened,
+                            it + std::min<int64_t>(nsteps - it, 1 << 30) < nsteps ? 2 : 1);
+    opened = true;
+    it += done;
+    if (rc != kOK) return rc;
+    for (SysHost& h : sys_)
+      if (h.active) h.steps += done, h.f_valid = finished;
+    if (!finished) {  // a list overflowed after the last drift: the rest of that step
+      CKR(launch_step(0.5, 0.0, kStepStoreF, s));
+      for (SysHost& h : sys_)
+        if (h.active) h.f_valid = true;
+      CK(cudaMemsetAsync(ke, 0, sizeof(unsigned long long) * 4 * (size_t)ns, s));
+      CKR(thermostat(it < nsteps ? 2 : 1));
+    }
+  }
+  if (it < nsteps && !opened) CKR(thermostat(1));
+  for (; it < nsteps; ++it) {
     CKR(step(1, dt, s));
     // the end of this step and the start of the next are consecutive half steps
+    CK(cudaMemsetAsync(ke, 0, sizeof(unsigned long long) * 4 * (size_t)ns, s));
     CKR(thermostat(it + 1 < nsteps ? 2 : 1));
+  }
+  CK(cudaMemcpyAsync(th.data(), d_thermo_, sizeof(Thermo) * (size_t)ns, cudaMemcpyDeviceToHost, s));
+  CKR(sync_check(s));
+  for (int k = 0; k < ns; ++k) {
+    if (!sys_[k].active) continue;
+    zeta[k] = th[(size_t)k].zeta;
+    eta[k] = th[(size_t)k].eta;
   }
   return kOK;
 }

@@ -190,7 +190,9 @@ class Engine {
   // one cooperative launch, the closing force evaluation included. loop_plan returns its
   // threads per particle, 0 where the arena does not take it.
   int loop_plan();
-  int run_loop(int64_t nsteps, bool stored, bool steady, int64_t* done, bool* finished, cudaStream_t s);
+  // nvt: Nose-Hoover steps (d_thermo_), with an opening half step if `open` is set.
+  int run_loop(int64_t nsteps, bool stored, bool steady, int64_t* done, bool* finished, cudaStream_t s,
+               bool nvt = false, bool open = false, int halves_end = 1);
   int after_steps(int64_t done, cudaStream_t s);
   int sync_check(cudaStream_t s);
   bool any_active() const;  // some system takes part in launches
@@ -224,7 +226,8 @@ class Engine {
   int64_t gver_[2] = {-1, -1};
   cudaStream_t cap_[2] = {nullptr, nullptr};
   GraphCtl* d_ctl_ = nullptr;
-  unsigned long long* d_loop_ = nullptr;  // persistent loop: barrier word, then 3 maxima per system
+  unsigned long long* d_loop_ = nullptr;  // persistent loop: barrier word, 3 maxima and 12 energy limbs per system
+  Thermo* d_thermo_ = nullptr;            // thermostats (nsys) of md_step_nvt
   int loop_lanes_ = 0, loop_stride_ = 0;
   int64_t loop_ver_ = -1;                 // struct_ver_ the plan was made for
   GraphCtl* h_ctl_ = nullptr;

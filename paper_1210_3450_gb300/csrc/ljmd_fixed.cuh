@@ -194,6 +194,20 @@ static __device__ __forceinline__ unsigned long long fix_sqr(unsigned long long 
 // Exact sum of 64-bit non-negative terms in 128 bits.
 struct FixAcc {
   unsigned long long lo = 0ull, hi = 0ull;
+  // Adds an FP64 number >= 0 in units of 2^-64 (bits below the unit are dropped;
+  // 2^63 and more, and what is not finite, count as 2^62).
+  __device__ __forceinline__ void add_fp64(double v) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    const int sh = (int)((b >> 52) & 0x7FF) - (1075 - 64);
+    const unsigned long long m = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);
+    unsigned long long l, h;
+    if (sh > 74) { l = 0ull; h = 1ull << 62; }
+    else if (sh >= 64) { l = 0ull; h = m << (sh - 64); }
+    else if (sh > 0) { l = m << sh; h = m >> (64 - sh); }
+    else { l = sh > -64 ? m >> -sh : 0ull; h = 0ull; }
+    lo += l;
+    hi += h + (lo < l ? 1ull : 0ull);
+  }
   __device__ __forceinline__ void add(unsigned long long v) {
     lo += v;
     hi += lo < v ? 1ull : 0ull;

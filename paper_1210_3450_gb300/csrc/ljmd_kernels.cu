@@ -2101,6 +2101,100 @@ __global__ void __launch_bounds__(256) k_obs_final(const int32_t* __restrict__ w
   }
 }
 
+// ------------------------------------------ Nose-Hoover thermostat (Sec. 4.1)
+
+// The kinetic energy of the thermostat is an exact sum of the squared velocity components
+// (FP64 squares in units of 2^-64, added as integers in four 32-bit limbs), so every way
+// of running the steps, alone or in a batch, gives the same bits whatever the order.
+namespace {
+
+__device__ __forceinline__ void add_limbs(unsigned long long* ke, const FixAcc& s) {
+  if (s.lo & 0xffffffffull) atomicAdd(ke + 0, s.lo & 0xffffffffull);
+  if (s.lo >> 32) atomicAdd(ke + 1, s.lo >> 32);
+  if (s.hi & 0xffffffffull) atomicAdd(ke + 2, s.hi & 0xffffffffull);
+  if (s.hi >> 32) atomicAdd(ke + 3, s.hi >> 32);
+}
+// Kinetic energy from the limbs.
+__device__ __forceinline__ double limbs_ke(unsigned long long a, unsigned long long b, unsigned long long c,
+                                           unsigned long long d) {
+  b += a >> 32;
+  c += b >> 32;
+  d += c >> 32;
+  FixAcc s;
+  s.lo = (b << 32) | (a & 0xffffffffull);
+  s.hi = (d << 32) | (c & 0xffffffffull);
+  return s.value(65);  // half the sum of the squares
+}
+
+// `halves` consecutive thermostat half steps from one kinetic energy: each is
+// zeta += dt/4 G, eta += dt/2 zeta, v *= exp(-dt/2 zeta), zeta += dt/4 G' with
+// G = (2 KE - g T) / Q; a uniform scale multiplies KE by its square, so the next G needs
+// no new sum. Returns the factor of the velocities. (Explicit roundings: the same bits
+// wherever it is inlined.)
+__device__ __forceinline__ double thermo_halves(Thermo& t, double ke, int halves) {
+  double fac = 1.0;
+  const double q = __dmul_rn(0.25, t.dt), e = __dmul_rn(0.5, t.dt);
+  for (int h = 0; h < halves; ++h) {
+    t.zeta = __dadd_rn(t.zeta, __ddiv_rn(__dmul_rn(q, __dsub_rn(__dmul_rn(2.0, ke), t.gT)), t.Q));
+    t.eta = __dadd_rn(t.eta, __dmul_rn(e, t.zeta));
+    const double sc = exp(-__dmul_rn(e, t.zeta));
+    fac = __dmul_rn(fac, sc);
+    ke = __dmul_rn(__dmul_rn(ke, sc), sc);
+    t.zeta = __dadd_rn(t.zeta, __ddiv_rn(__dmul_rn(q, __dsub_rn(__dmul_rn(2.0, ke), t.gT)), t.Q));
+  }
+  return fac;
+}
+
+}  // namespace
+
+__global__ void __launch_bounds__(256) k_ke_limbs(DevArrays a, unsigned long long* ke) {
+  const int lane = threadIdx.x & 31;
+  const int nw = (int)((gridDim.x * blockDim.x) >> 5);
+  FixAcc s;
+  int last = -1;
+  auto flush = [&]() {
+    if (last < 0) return;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s.join(o);
+    if (lane == 0) add_limbs(ke + 4 * last, s);
+    s = FixAcc();
+  };
+  // each warp a run of consecutive tiles (few changes of system)
+  const int per = (a.ntiles + nw - 1) / nw;
+  const int w0 = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * per, w1 = min(w0 + per, a.ntiles);
+  for (int w = w0; w < w1; ++w) {
+    const int sys = a.tile_sys[w];
+    if (sys < 0) continue;
+    const SysParams& P = a.params[sys];
+    if (!P.active) continue;
+    if (sys != last) {
+      flush();
+      last = sys;
+    }
+    const int local = (w - P.t_off) * kTile + lane;
+    if (local < P.n) {
+      const double4_32a v = a.v[P.p_off + local];
+      s.add_fp64(__dmul_rn(v.x, v.x));
+      s.add_fp64(__dmul_rn(v.y, v.y));
+      s.add_fp64(__dmul_rn(v.z, v.z));
+    }
+  }
+  flush();
+}
+
+__global__ void k_thermostat(DevArrays a, int nsys, Thermo* thermo, int halves, unsigned long long* ke, double* scale) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= nsys) return;
+  double f = 1.0;
+  if (a.params[k].active) {
+    Thermo t = thermo[k];
+    f = thermo_halves(t, limbs_ke(ke[4 * k], ke[4 * k + 1], ke[4 * k + 2], ke[4 * k + 3]), halves);
+    thermo[k] = t;
+  }
+  scale[k] = f;
+  for (int m = 0; m < 4; ++m) ke[4 * k + m] = 0ull;
+}
+
 // ------------------------------------ persistent step loop of small arenas
 
 // A step of a few thousand particles is a chain of latencies: in separate launches
@@ -2144,6 +2238,8 @@ struct LoopShared {
   unsigned long long d2[kLoopWarps];
   int sys[kLoopWarps];
   double margin[kLoopMaxSys];
+  double scale[kLoopMaxSys];
+  FixAcc ke[kLoopWarps];
   int need[kLoopMaxSys];
   int ws[kScanBlock / 32];
   int flag;  // barrier: 0 gave up
@@ -2212,7 +2308,7 @@ __device__ __forceinline__ void loop_worklists(const DevArrays& a, const LoopArg
 
 }  // namespace
 
-template <bool kFP32, int T>
+template <bool kFP32, int T, bool kNvt>
 __global__ void __launch_bounds__(kLoopBlock, T == 4 ? (kFP32 ? 4 : 3) : (kFP32 ? 3 : 2)) k_loop(DevArrays a, LoopArgs g) {
   extern __shared__ __align__(32) unsigned char smem[];
   __shared__ LoopShared sh;
@@ -2401,28 +2497,74 @@ __global__ void __launch_bounds__(kLoopBlock, T == 4 ? (kFP32 ? 4 : 3) : (kFP32 
   // the decision's constants of system threadIdx.x
   bool dactive = false;
   double dthr = 0.0, ddt = 0.0;
+  Thermo thermo{};  // system threadIdx.x's thermostat (every block keeps the same)
   if ((int)threadIdx.x < g.nsys) {
     const SysParams& Q = a.params[threadIdx.x];
     dactive = Q.active != 0;
     dthr = kFP32 ? Q.disp_thr : Q.skin;
     ddt = Q.dt;
+    if (kNvt) thermo = g.thermo[threadIdx.x];
   }
   __syncthreads();
 
-  while (done < target_steps) {
+  // `halves` thermostat half steps at the current velocities; `turn` counts the calls.
+  // False if the barrier gave up.
+  int turn = 0;
+  [[maybe_unused]] auto thermostat = [&](int halves) -> bool {
+    if (blockIdx.x == 0 && (int)threadIdx.x < 4 * g.nsys)  // the next turn's sums: their last readers passed a barrier
+      g.ke[((turn + 1) % 3) * 4 * g.nsys + threadIdx.x] = 0ull;
+    FixAcc s;
+    if (comp) s.add_fp64(__dmul_rn(v, v));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s.join(o);
+    if (lane == 0) {
+      sh.ke[wv] = s;
+      sh.sys[wv] = on ? sys : -1;
+    }
+    __syncthreads();
+    if (wv == 0) {
+      const int k = sh.sys[lane & (kLoopWarps - 1)];
+      FixAcc m = sh.ke[lane & (kLoopWarps - 1)];
+      unsigned long long* ke = g.ke + (turn % 3) * 4 * g.nsys;
+      if (__all_sync(kFull, k == sh.sys[0])) {
+#pragma unroll
+        for (int o = kLoopWarps / 2; o > 0; o >>= 1) m.join(o);
+        if (lane == 0 && k >= 0) add_limbs(ke + 4 * k, m);
+      } else if (lane < kLoopWarps && k >= 0) {
+        add_limbs(ke + 4 * k, m);
+      }
+    }
+    if (!grid_barrier(g.bar, arrivals, sh, a.ctl)) return false;
+    if (dactive) {
+      const unsigned long long* ke = g.ke + ((turn % 3) * g.nsys + threadIdx.x) * 4;
+      sh.scale[threadIdx.x] = thermo_halves(thermo, limbs_ke(__ldcg(ke), __ldcg(ke + 1), __ldcg(ke + 2), __ldcg(ke + 3)), halves);
+    }
+    ++turn;
+    __syncthreads();
+    if (comp && sh.scale[sys] != 1.0) v *= sh.scale[sys];
+    return true;
+  };
+  double fnow = 0.0;  // Nose-Hoover steps: the force at the current positions
+  if (kNvt) {
+    if (comp) fnow = ((const double*)&a.f[slot])[c];
+    if (g.open) alive = thermostat(1);
+  }
+
+  while (alive && done < target_steps) {
     unsigned long long d2 = 0ull;
     // block 0 clears the maximum of the next step: its last readers passed a barrier
     if (blockIdx.x == 0 && (int)threadIdx.x < g.nsys) g.disp[((done + 1) % 3) * g.nsys + threadIdx.x] = 0ull;
     if (on) {
       const bool first = done == 0;
       double F;
-      if (first && g.stored) F = comp ? ((const double*)&a.f[slot])[c] : 0.0;
+      if (kNvt) F = fnow;
+      else if (first && g.stored) F = comp ? ((const double*)&a.f[slot])[c] : 0.0;
       else F = force();
       bool fine = true;
       long long s0 = 0;         // squared displacement of the axis (exact integer) ...
       double sd = 0.0;          // ... or its FP64 square, or the squared velocity
       if (comp) {
-        if (!first || g.steady) v = fma(h, F, v);
+        if (!kNvt && (!first || g.steady)) v = fma(h, F, v);
         v = fma(h, F, v);
         const double xn = fma(dt, v, x);
         x = xn;
@@ -2507,34 +2649,41 @@ __global__ void __launch_bounds__(kLoopBlock, T == 4 ? (kFP32 ? 4 : 3) : (kFP32 
     cur ^= 1;
     ++done;
     if (__syncthreads_or(stop)) { abort = 2; break; }
-    if (!__syncthreads_or(need)) continue;
-    // rebuild pass
-    const bool mine = on && sh.need[sys];
-    if (mine && comp) {
-      ((double*)&a.x[cur][slot])[c] = x;
-      ((double*)&a.v[slot])[c] = v;
+    if (__syncthreads_or(need)) {  // rebuild pass
+      const bool mine = on && sh.need[sys];
+      if (mine && comp) {
+        ((double*)&a.x[cur][slot])[c] = x;
+        ((double*)&a.v[slot])[c] = v;
+      }
+      if (blockIdx.x == 0 && wv == 0) loop_worklists(a, g, sh.need);
+      if (!(alive = grid_barrier(g.bar, arrivals, sh, a.ctl))) break;
+      cell_count_pass<true>(a, cur);
+      if (!(alive = grid_barrier(g.bar, arrivals, sh, a.ctl))) break;
+      cell_starts_pass(a, a.ctl->nreb, sh.ws);
+      if (!(alive = grid_barrier(g.bar, arrivals, sh, a.ctl))) break;
+      scatter_pass<true>(a, cur);
+      if (!(alive = grid_barrier(g.bar, arrivals, sh, a.ctl))) break;
+      cell_rank_pass<true>(a, cur);
+      if (!(alive = grid_barrier(g.bar, arrivals, sh, a.ctl))) break;
+      build_lists_wide(a, cur, T == 32 ? 8 : T == 16 ? 16 : 32, wide);
+      if (!(alive = grid_barrier(g.bar, arrivals, sh, a.ctl))) break;
+      if ((int)threadIdx.x < g.nsys && sh.need[threadIdx.x]) sh.margin[threadIdx.x] = a.margin[threadIdx.x];
+      if (mine) load_state();
+      abort = *(volatile int*)&a.ctl->abort;
+      __syncthreads();
+      if (abort) break;  // a list overflowed: the host grows it (uniform over the grid)
     }
-    if (blockIdx.x == 0 && wv == 0) loop_worklists(a, g, sh.need);
-    if (!(alive = grid_barrier(g.bar, arrivals, sh, a.ctl))) break;
-    cell_count_pass<true>(a, cur);
-    if (!(alive = grid_barrier(g.bar, arrivals, sh, a.ctl))) break;
-    cell_starts_pass(a, a.ctl->nreb, sh.ws);
-    if (!(alive = grid_barrier(g.bar, arrivals, sh, a.ctl))) break;
-    scatter_pass<true>(a, cur);
-    if (!(alive = grid_barrier(g.bar, arrivals, sh, a.ctl))) break;
-    cell_rank_pass<true>(a, cur);
-    if (!(alive = grid_barrier(g.bar, arrivals, sh, a.ctl))) break;
-    build_lists_wide(a, cur, T == 32 ? 8 : T == 16 ? 16 : 32, wide);
-    if (!(alive = grid_barrier(g.bar, arrivals, sh, a.ctl))) break;
-    if ((int)threadIdx.x < g.nsys && sh.need[threadIdx.x]) sh.margin[threadIdx.x] = a.margin[threadIdx.x];
-    if (mine) load_state();
-    abort = *(volatile int*)&a.ctl->abort;
-    __syncthreads();
-    if (abort) break;  // a list overflowed: the host grows it (uniform over the grid)
+    if constexpr (kNvt) {  // the step's closing half kick and the thermostat half steps
+      if (on) {
+        fnow = force();
+        if (comp) v = fma(h, fnow, v);
+      }
+      if (!(alive = thermostat(done < target_steps ? 2 : g.halves_end))) break;
+    }
   }
 
   double F = 0.0;
-  const bool close = alive && abort == 0 && g.finish;
+  const bool close = !kNvt && alive && abort == 0 && g.finish;
   if (close && on) {
     F = force();
     if (comp) v = fma(h, F, v);
@@ -2543,10 +2692,13 @@ __global__ void __launch_bounds__(kLoopBlock, T == 4 ? (kFP32 ? 4 : 3) : (kFP32 
     ((double*)&a.x[cur][slot])[c] = x;
     ((double*)&a.v[slot])[c] = v;
     if (!kFP32) ((int*)&a.xq[cur][slot])[c] = to_fixed(x, qscale);
-    if (close) ((double*)&a.f[slot])[c] = F;
+    if (close || kNvt) ((double*)&a.f[slot])[c] = kNvt ? fnow : F;
   }
   if (blockIdx.x == 0) {
-    if ((int)threadIdx.x < g.nsys) a.margin[threadIdx.x] = sh.margin[threadIdx.x];
+    if ((int)threadIdx.x < g.nsys) {
+      a.margin[threadIdx.x] = sh.margin[threadIdx.x];
+      if (kNvt) g.thermo[threadIdx.x] = thermo;
+    }
     if (threadIdx.x == 0) {
       a.ctl->done = done;
       if (abort) atomicMax(&a.ctl->abort, abort);
@@ -2910,6 +3062,13 @@ void launch_step_fp32(const DevArrays& a, int cur, double ka, double kb, int fla
 #undef LJMD_STEP32
 }
 namespace {
+template <bool kFP32, int T, bool kNvt>
+cudaError_t loop_setup_k(size_t bytes, int* blocks_per_sm) {
+  cudaError_t e = cudaFuncSetAttribute(k_loop<kFP32, T, kNvt>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_loop<kFP32, T, kNvt>, kLoopBlock, bytes);
+  return e;
+}
 template <bool kFP32, int T>
 cudaError_t loop_setup(int kmax, int* stride, size_t* bytes, int* blocks_per_sm) {
   const int unit = loop_chunk(T) * T;
@@ -2917,9 +3076,11 @@ cudaError_t loop_setup(int kmax, int* stride, size_t* bytes, int* blocks_per_sm)
   st += (T - st % 32 + 32) % 32;
   *stride = st;
   *bytes = loop_union_bytes(T) + sizeof(typename LoopWord<kFP32>::type) * (size_t)st * (kLoopBlock / T);
-  cudaError_t e = cudaFuncSetAttribute(k_loop<kFP32, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*bytes);
-  if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_loop<kFP32, T>, kLoopBlock, *bytes);
+  // both kinds of steps take the plan
+  int plain = 0, nvt = 0;
+  cudaError_t e = loop_setup_k<kFP32, T, false>(*bytes, &plain);
+  if (e == cudaSuccess) e = loop_setup_k<kFP32, T, true>(*bytes, &nvt);
+  *blocks_per_sm = std::min(plain, nvt);
   return e;
 }
 template <bool kFP32>
@@ -2931,10 +3092,10 @@ cudaError_t loop_setup(int T, int kmax, int* stride, size_t* bytes, int* bps) {
     default: return loop_setup<kFP32, 4>(kmax, stride, bytes, bps);
   }
 }
-template <bool kFP32>
+template <bool kFP32, bool kNvt>
 const void* loop_kernel(int T) {
-  return T == 32 ? (const void*)k_loop<kFP32, 32> : T == 16 ? (const void*)k_loop<kFP32, 16>
-         : T == 8 ? (const void*)k_loop<kFP32, 8> : (const void*)k_loop<kFP32, 4>;
+  return T == 32 ? (const void*)k_loop<kFP32, 32, kNvt> : T == 16 ? (const void*)k_loop<kFP32, 16, kNvt>
+         : T == 8 ? (const void*)k_loop<kFP32, 8, kNvt> : (const void*)k_loop<kFP32, 4, kNvt>;
 }
 unsigned loop_blocks(int ntiles, int T) { return (unsigned)(((int64_t)ntiles * kTile * T + kLoopBlock - 1) / kLoopBlock); }
 }  // namespace
@@ -2967,7 +3128,8 @@ cudaError_t launch_loop(const DevArrays& a, const LoopArgs& g, cudaStream_t s) {
   DevArrays ac = a;
   LoopArgs gc = g;
   void* args[] = {&ac, &gc};
-  const void* fn = g.fp32 ? loop_kernel<true>(g.lanes) : loop_kernel<false>(g.lanes);
+  const void* fn = g.thermo ? (g.fp32 ? loop_kernel<true, true>(g.lanes) : loop_kernel<false, true>(g.lanes))
+                            : (g.fp32 ? loop_kernel<true, false>(g.lanes) : loop_kernel<false, false>(g.lanes));
   const size_t word = g.fp32 ? sizeof(LoopWord<true>::type) : sizeof(LoopWord<false>::type);
   const size_t bytes = loop_union_bytes(g.lanes) + word * (size_t)g.stride * (kLoopBlock / g.lanes);
   return cudaLaunchCooperativeKernel(fn, dim3(loop_blocks(a.ntiles, g.lanes)), dim3(kLoopBlock), args, bytes, s);
@@ -2996,6 +3158,15 @@ __global__ void k_scale_v(DevArrays a, const double* __restrict__ scale) {
 void launch_scale_v(const DevArrays& a, const double* scale, cudaStream_t s) {
   k_scale_v<<<tile_blocks(a), kBlock, 0, s>>>(a, scale);
 }
+void launch_thermostat(const DevArrays& a, int nsys, Thermo* thermo, int halves, unsigned long long* ke, double* scale,
+                       cudaStream_t s) {
+  // at most four blocks per SM, so that few warps meet on a system's sums
+  const unsigned g = (unsigned)std::max(1, std::min((a.ntiles + 7) / 8, kSMs * 4));
+  k_ke_limbs<<<g, 256, 0, s>>>(a, ke);
+  k_thermostat<<<(unsigned)((nsys + 127) / 128), 128, 0, s>>>(a, nsys, thermo, halves, ke, scale);
+  launch_scale_v(a, scale, s);
+}
+
 void launch_pair_stats(const DevArrays& a, int cur, unsigned long long* out2, cudaStream_t s) {
   k_pair_stats<<<tile_blocks(a), kBlock, 0, s>>>(a, cur, out2);
 }

@@ -67,3 +67,22 @@ def test_batch_with_a_paused_system(ljmd, precision):
         for a, c in zip(p[:3], q[:3]):
             np.testing.assert_array_equal(a, c)
         assert p[3] == q[3]
+
+
+@pytest.mark.parametrize("precision", [0, 1], ids=["fp64", "fp32"])
+@pytest.mark.parametrize("n,rho,rc", [(500, 0.85, 2.5), (2433, 0.7, 3.0), (9729, 0.6, 2.5)])
+def test_nvt_equals_host_loop(ljmd, n, rho, rc, precision):
+    x, box = li.perturbed_fcc(n, rho, 0.1, n)
+    v = li.maxwell_boltzmann(n, 1.3, n + 1)
+    out = []
+    for graph in (0, 1):
+        with ljmd.LJSystem(box, n, rc, 0.3, precision) as s:
+            s.set_tuning(graph=graph)
+            s.set_state(x, v)
+            z, e = s.step_nvt(24, 0.005, 0.9, 3.0 * n * 0.05)
+            z, e = s.step_nvt(1, 0.005, 0.9, 3.0 * n * 0.05, z, e)
+            s.step(3, 0.005)
+            out.append((*s.get_state(), s.forces(), np.array([z, e]), s.stats()))
+    for p, q in zip(out[0][:4], out[1][:4]):
+        np.testing.assert_array_equal(p, q)
+    assert out[0][4] == out[1][4]
