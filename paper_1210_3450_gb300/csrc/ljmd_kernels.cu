@@ -554,21 +554,6 @@ struct PreTest<1> {
   __device__ __forceinline__ int4 load(int j) const { return p[j]; }
 };
 
-// PRE 0 reading a row's candidates staged in shared memory: slot j sits at
-// s[j - base].
-struct PreTestS {
-  const float4* s;
-  int base;
-  float cx, cy, cz;
-  float lo2, hi2;
-  __device__ __forceinline__ float key(int j) const { return s[j - base].x; }
-  __device__ __forceinline__ float r2(const float4& q) const {
-    const float dx = q.x - cx, dy = q.y - cy, dz = q.z - cz;
-    return fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-  }
-  __device__ __forceinline__ float4 load(int j) const { return s[j - base]; }
-};
-
 __device__ __forceinline__ float key_of(const float4& q) { return q.x; }
 __device__ __forceinline__ float key_of(const int4& q) { return __int_as_float(q.w); }
 
@@ -966,7 +951,11 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) k_build_list_warp(DevArra
 }
 
 // List build with rows staged in shared memory: the same lists, in the same
-// order, as k_build_list (the same per-thread sweep, pre-test and exact test).
+// order, as k_build_list (the same windows, thresholds and exact test). 0.89 ms per
+// build at 2,048,000 particles (rc 2.5) against 1.02 with two compares per candidate
+// and 4-byte stores (16-byte stores alone: 0.13 of it; L2 traffic fell from 67 M to 22 M
+// store sectors per build of 864,000 particles), 0.95 against 1.18 ms at rc 3.0, density
+// 0.6; now bound by issue (78 % active).
 // For each neighbour row (and piece of a row that wraps in x) the warp first
 // copies the union of its lanes' candidate ranges into shared memory with
 // coalesced loads (up to kStage candidates; a wider union, as where a tile's
@@ -978,8 +967,135 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) k_build_list_warp(DevArra
 namespace {
 
 constexpr int kStage = 160;  // staged candidates per warp and row piece
+struct StageBuf {            // coordinates apart: one 16-byte load gives those of four candidates
+  float x[kStage + 4], y[kStage + 4], z[kStage + 4];
+};
 
-__device__ __forceinline__ void build_tile_staged(const DevArrays& a, int cur, int sys, int tl, float4* buf) {
+// The staged build's list writer: entries are collected in registers and stored four at a
+// time (a lane's 4-byte stores fill a sector of their own each, 67 M of them per build
+// of 864,000 particles).
+struct StagedCtx {
+  ListCtx o;       // its count and place are brought up to date by leave()
+  int count;
+  uint32_t* group; // where the group being collected goes
+  uint32_t g0, g1, g2, g3;
+  __device__ __forceinline__ void push(uint32_t e) {
+    if (o.entry_ok(e)) put(e);
+  }
+  __device__ __forceinline__ void put(uint32_t e) {
+    g0 = g1; g1 = g2; g2 = g3; g3 = e;
+    ++count;
+    // a full group is stored (if it fits: kmax is a multiple of 8), without a branch
+    asm volatile("{\n\t.reg .pred p, q;\n\t.reg .b32 t;\n\tand.b32 t, %1, 3;\n\tsetp.eq.s32 p, t, 0;\n\tsetp.le.and.s32 q, %1, %2, p;\n\t"
+                 "@q st.global.v4.u32 [%0], {%3, %4, %5, %6};\n\t@p add.s64 %0, %0, 512;\n\t}"
+                 : "+l"(group) : "r"(count), "r"(o.kmax), "r"(g0), "r"(g1), "r"(g2), "r"(g3) : "memory");
+  }
+  // To the plain writer (the collected entries stored one by one), and from it.
+  __device__ __forceinline__ void leave() {
+    const int r = count & 3;
+    if (count <= o.kmax) {
+      if (r == 1) group[0] = g3;
+      if (r == 2) { group[0] = g2; group[1] = g3; }
+      if (r == 3) { group[0] = g1; group[1] = g2; group[2] = g3; }
+    }
+    o.count = count;
+    o.wp = group + r;
+  }
+  __device__ __forceinline__ void enter() {
+    count = o.count;
+    group = o.out + (count >> 2) * (4 * kTile);
+    const int r = count & 3;
+    if (r && count <= o.kmax) {
+      const uint32_t w0 = group[0], w1 = group[1], w2 = group[2];
+      g3 = r == 1 ? w0 : r == 2 ? w1 : w2;
+      g2 = r == 2 ? w0 : w1;
+      g1 = w0;
+    }
+  }
+  // Padding with the particle itself, to a whole group (ListCtx::pad).
+  __device__ __forceinline__ void finish() {
+    o.count = count;
+    while (count & 3) put((uint32_t)o.li);
+  }
+};
+
+// sweep_range on staged candidates (slot j at place j - first). The pre-test's squared
+// distance starts at -hi2, so its sign is the test: the signs are shifted into a mask
+// (candidate k of the window at bit 31 - k), 9 instructions per candidate with the
+// smallest distance to the threshold, where two compares and two predicated ORs made
+// it 11 (and those four run on half of the lanes' rate). A window whose smallest
+// distance is within the shell looks at its marked candidates again. Windows start at
+// a multiple of four places; candidates outside [lo, hi) are masked.
+__device__ __forceinline__ void sweep_staged(const StageBuf& S, int first, float px, float py, float pz, float hi2,
+                                             float shell, StagedCtx& w, int lo, int hi, unsigned code, float xlo,
+                                             float xhi) {
+  int b = hi;
+  while (lo < b) {
+    const int m = (lo + b) >> 1;
+    if (S.x[m - first] < xlo) lo = m + 1;
+    else b = m;
+  }
+  const int fe = hi - first, fs = (lo - first) & ~3;
+  int f = fs;
+  bool more = lo < hi;
+  while (more) {
+    const int f0 = f;
+    unsigned bits = 0u;
+    float near = 1e30f;
+#pragma unroll
+    for (int g = 0; g < 8; ++g) {
+      if (more) {
+        const float4 X = *(const float4*)(S.x + f);
+        // past the window (the very first group may begin with candidates of another row)
+        if ((g > 0 || f0 > fs) && !(X.x < xhi)) {
+          more = false;
+        } else {
+          const float4 Y = *(const float4*)(S.y + f), Z = *(const float4*)(S.z + f);
+          auto test = [&](float x, float y, float z) {
+            const float dx = x - px, dy = y - py, dz = z - pz;
+            const float r = fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, -hi2)));
+            bits = __funnelshift_l(__float_as_uint(r), bits, 1);
+            near = fminf(near, fabsf(r));
+          };
+          test(X.x, Y.x, Z.x);
+          test(X.y, Y.y, Z.y);
+          test(X.z, Y.z, Z.z);
+          test(X.w, Y.w, Z.w);
+          f += 4;
+          more = f < fe;
+        }
+      }
+    }
+    const int nt = f - f0;  // candidates tested
+    if (nt == 0) break;
+    bits <<= 32 - nt;
+    const int cut = lo - first - f0, end = fe - f0, s = w.o.li - first - f0;
+    if (cut > 0) bits &= 0xffffffffu >> cut;
+    if (end < 32) bits &= ~(0xffffffffu >> end);
+    if ((unsigned)s < 32u) bits &= ~(0x80000000u >> s);  // not the particle itself
+    if (w.o.half) {  // half list: candidates above the particle's slot
+      if (s >= 31) bits = 0u;
+      else if (s >= 0) bits &= 0xffffffffu >> (s + 1);
+    }
+    if (near <= shell) {  // (rare) between the pre-test's thresholds: the exact FP64 test
+      for (unsigned t = bits; t != 0u;) {
+        const int k = __clz((int)t);
+        t &= ~(0x80000000u >> k);
+        const float dx = S.x[f0 + k] - px, dy = S.y[f0 + k] - py, dz = S.z[f0 + k] - pz;
+        const float r = fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, -hi2)));
+        if (!(r < -shell) && !w.o.exact_in(first + f0 + k, code)) bits &= ~(0x80000000u >> k);
+      }
+    }
+    const uint32_t e0 = (uint32_t)(first + f0) | (code << kIdxBits);  // (no carry into the code: slots end below 2^26)
+    while (bits) {
+      const int k = __clz((int)bits);
+      bits &= ~(0x80000000u >> k);
+      w.push(e0 + (uint32_t)k);
+    }
+  }
+}
+
+__device__ __forceinline__ void build_tile_staged(const DevArrays& a, int cur, int sys, int tl, StageBuf& buf) {
   const int lane = threadIdx.x & 31;
   const SysParams* __restrict__ Pp = a.params + sys;
   if (!Pp->active) return;  // uniform over the warp
@@ -988,8 +1104,9 @@ __device__ __forceinline__ void build_tile_staged(const DevArrays& a, int cur, i
   const bool act = li < n;
   const int64_t p_off = Pp->p_off;
   const int kmax = Pp->kmax;
-  ListCtx o{Pp, a.xref + p_off, a.nbr + list_word(Pp->l_off, tl, kmax, lane, 0), li, 0, kmax, Pp->half != 0,
-            a.checks + sys};
+  StagedCtx st{ListCtx{Pp, a.xref + p_off, a.nbr + list_word(Pp->l_off, tl, kmax, lane, 0), li, 0, kmax, Pp->half != 0,
+                       a.checks + sys}, 0, nullptr, 0u, 0u, 0u, 0u};
+  ListCtx& o = st.o;
   if (act) copy_back_slot(a, cur, p_off + li);
   const int nc = Pp->nc;
   if (nc == 1) {  // uniform over the warp
@@ -998,6 +1115,7 @@ __device__ __forceinline__ void build_tile_staged(const DevArrays& a, int cur, i
     list_done(a, sys, p_off + li, o.count, kmax, act, kFull, lane);
     return;
   }
+  st.group = o.out;
   const float4* __restrict__ xf = a.xf + p_off;
   const int32_t* __restrict__ cst = a.cstart + Pp->c_off;
   const float w = Pp->rlf + Pp->wmargin;  // half-width of the x window
@@ -1005,10 +1123,7 @@ __device__ __forceinline__ void build_tile_staged(const DevArrays& a, int cur, i
   T.p = xf;
   T.lo2 = Pp->rl2f_lo;
   T.hi2 = Pp->rl2f_hi;
-  PreTestS S;
-  S.s = buf;
-  S.lo2 = T.lo2;
-  S.hi2 = T.hi2;
+  const float shell = (T.hi2 - T.lo2) * 1.0001f;  // the difference is exact or rounded once
   int cx = 1, cy = 0, cz = 0;
   if (act) {
     const int ci = a.celltmp[p_off + li];
@@ -1053,29 +1168,32 @@ __device__ __forceinline__ void build_tile_staged(const DevArrays& a, int cur, i
       if (u1 - u0 <= kStage) {
         // stage [u0, u1) and the 3 slots after it (a group of four may read past
         // its range end; the slot arrays have four spare entries)
-        for (int k = lane; k < u1 - u0 + 3; k += 32) buf[k] = xf[u0 + k];
+        for (int k = lane; k < u1 - u0 + 3; k += 32) {
+          const float4 q = xf[u0 + k];
+          buf.x[k] = q.x;
+          buf.y[k] = q.y;
+          buf.z[k] = q.z;
+        }
         __syncwarp();
-        S.base = u0;
-        S.cx = xw;
-        S.cy = T.cy;
-        S.cz = T.cz;
-        sweep_range(S, o, lo, hi, code, xw - w, xw + w);
+        sweep_staged(buf, u0, xw, T.cy, T.cz, T.hi2, shell, st, lo, hi, code, xw - w, xw + w);
         __syncwarp();  // before the next piece overwrites the buffer
       } else {
         T.cx = xw;
+        st.leave();
         sweep_range(T, o, lo, hi, code, xw - w, xw + w);
+        st.enter();
       }
     }
   }
-  if (act) o.pad();
-    list_done(a, sys, p_off + li, o.count, kmax, act, kFull, lane);
+  if (act) st.finish();
+  list_done(a, sys, p_off + li, o.count, kmax, act, kFull, lane);
 }
 
 }  // namespace
 
 template <int BLOCK>
 __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) k_build_list_staged(DevArrays a, int cur) {
-  __shared__ float4 sbuf[BLOCK / 32][kStage + 4];
+  __shared__ __align__(16) StageBuf sbuf[BLOCK / 32];
   int sys, tl;
   while (next_rebuild_tile(a, sys, tl)) build_tile_staged(a, cur, sys, tl, sbuf[threadIdx.x >> 5]);
 }
