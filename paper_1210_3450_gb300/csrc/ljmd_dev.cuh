@@ -122,6 +122,7 @@ struct LoopArgs {
   int nsys;      // system records (at most kLoopMaxSys)
   int fp32;      // force form
   int vmax;      // velocity-bound rule
+  unsigned rebuild0;  // bit k: system k's list is built before the first step
   int stored;    // 1: the first step takes the stored forces
   int steady;    // 1: the first step also completes the previous step's kick
   int finish;    // 1: after the last step, forces (stored) and the closing half kick
@@ -272,6 +273,7 @@ void launch_pair_stats(const DevArrays& a, int cur, unsigned long long* out2, cu
 // holds 3 doubles per chunk.
 void launch_reduce_obs(const DevArrays& a, const int32_t* work, int nsel, int nchunks, double* chunk3, double* out3,
                        cudaStream_t s);
+void launch_state_to_caller(const DevArrays& a, int cur, double* x, double* v, int64_t sys_n, int sys, cudaStream_t s);
 void launch_to_caller(const DevArrays& a, int cur, int which, double* out, int64_t sys_n,
                       int sys, int64_t ntiles_sys, cudaStream_t s);
 void launch_positions_by_id(const DevArrays& a, int cur, const double* x, int64_t sys_n, int sys, cudaStream_t s);

@@ -741,8 +741,7 @@ int Engine::get_state_dev(int k, double* x, double* v, cudaStream_t s) {
   if (!valid_id(k)) { set_error("no such system"); return kErrArg; }
   SysHost& h = sys_[k];
   if (!h.has_state) { set_error("no state set"); return kErrState; }
-  if (x) launch_to_caller(arrays(), cur_of(k), 0, x, h.spec.n, k, h.ntiles, s);
-  if (v) launch_to_caller(arrays(), cur_of(k), 1, v, h.spec.n, k, h.ntiles, s);
+  launch_state_to_caller(arrays(), cur_of(k), x, v, h.spec.n, k, s);
   CKL();
   return kOK;
 }
@@ -864,14 +863,23 @@ int Engine::rebuild(std::vector<int> which, cudaStream_t s) {
   return kErrOverflow;
 }
 
+int Engine::have_states() const {
+  for (const SysHost& h : sys_)
+    if (h.active && !h.has_state) { set_error("no state set"); return kErrState; }
+  return kOK;
+}
+
+bool Engine::forces_valid() const {
+  for (const SysHost& h : sys_)
+    if (h.active && !h.f_valid) return false;
+  return true;
+}
+
 int Engine::ensure_lists(cudaStream_t s) {
+  CKR(have_states());
   std::vector<int> which;
-  for (int k = 0; k < nsys(); ++k) {
-    const SysHost& h = sys_[k];
-    if (!h.active) continue;
-    if (!h.has_state) { set_error("no state set"); return kErrState; }
-    if (h.force_rebuild) which.push_back(k);
-  }
+  for (int k = 0; k < nsys(); ++k)
+    if (sys_[k].active && sys_[k].force_rebuild) which.push_back(k);
   return rebuild(which, s);
 }
 
@@ -908,10 +916,7 @@ int Engine::pair_stats(int k, int64_t* listed, int64_t* inside, cudaStream_t s) 
 }
 
 int Engine::ensure_forces(cudaStream_t s) {
-  bool need = false;
-  for (const SysHost& h : sys_)
-    if (h.active && !h.f_valid) need = true;
-  if (!need) return kOK;
+  if (forces_valid()) return kOK;
   CKR(launch_step(0.0, 0.0, kStepStoreF, s));
   for (SysHost& h : sys_)
     if (h.active) h.f_valid = true;
@@ -1155,7 +1160,9 @@ int Engine::run_loop(int64_t nsteps, bool stored, bool steady, int64_t* done, bo
   g.nsys = nsys();
   g.fp32 = precision_ == 1 ? 1 : 0;
   g.vmax = rule_ == 1 ? 1 : 0;
-  g.stored = stored ? 1 : 0;
+  for (int k = 0; k < nsys(); ++k)
+    if (sys_[k].active && sys_[k].force_rebuild) g.rebuild0 |= 1u << k;
+  g.stored = stored && g.rebuild0 == 0u && forces_valid() ? 1 : 0;
   g.steady = steady ? 1 : 0;
   g.finish = 1;
   g.stride = loop_stride_;
@@ -1201,19 +1208,23 @@ int Engine::step(int64_t nsteps, const std::vector<double>& dt, cudaStream_t s) 
   }
   if (nsteps == 0 || !any_active()) return kOK;  // an empty or fully paused arena: nothing to do
   CKR(upload_params());
-  CKR(ensure_lists(s));
-  CKR(ensure_forces(s));
-  CK(cudaMemsetAsync(d_ctl_, 0, sizeof(GraphCtl), s));
   int64_t it = 0;
   bool finished = false;
-  if (graph_ && !timing_) {
+  if (graph_ && !timing_ && loop_plan() > 0) {
+    CKR(have_states());  // (the launch builds the lists and evaluates the forces that are due)
     while (it < nsteps && loop_plan() > 0) {
       int64_t done = 0;
       const int rc = run_loop(std::min<int64_t>(nsteps - it, 1 << 30), it == 0, it > 0, &done, &finished, s);
       it += done;
       if (rc != kOK) return rc;
     }
-
+  }
+  if (!finished) {
+    CKR(ensure_lists(s));
+    if (it == 0) CKR(ensure_forces(s));
+    CK(cudaMemsetAsync(d_ctl_, 0, sizeof(GraphCtl), s));
+  }
+  if (graph_ && !timing_) {
     while (nsteps - it >= 2) {
       const int first = (it == 0 ? (kStepUseStoredF | kStepDrift | kStepKickB) : (kStepKickA | kStepKickB | kStepDrift)) |
                         (rule_ == 1 ? kStepVmax : 0);
@@ -1339,8 +1350,7 @@ int Engine::step_nvt(int64_t nsteps, const std::vector<double>& dt, const std::v
     if (sys_[k].active) sys_[k].dt = dt[k];
   }
   CKR(upload_params());
-  CKR(ensure_lists(s));
-  CKR(ensure_forces(s));
+  CKR(have_states());
   CK(cudaMemcpyAsync(d_thermo_, th.data(), sizeof(Thermo) * (size_t)ns, cudaMemcpyHostToDevice, s));
   unsigned long long* ke = d_loop_ + 1 + 3 * (size_t)ns;
   CK(cudaMemsetAsync(ke, 0, sizeof(unsigned long long) * 4 * (size_t)ns, s));
@@ -1352,16 +1362,18 @@ int Engine::step_nvt(int64_t nsteps, const std::vector<double>& dt, const std::v
   };
   int64_t it = 0;
   bool opened = false;
+  // (in the loop the launch builds the lists and evaluates the forces that are due)
   while (it < nsteps && graph_ && !timing_ && loop_plan() > 0) {
     int64_t done = 0;
     bool finished = false;
     const int rc = run_loop(std::min<int64_t>(nsteps - it, 1 << 30), true, false, &done, &finished, s, true, !opened,
                             it + std::min<int64_t>(nsteps - it, 1 << 30) < nsteps ? 2 : 1);
-    opened = true;
     it += done;
     if (rc != kOK) return rc;
     for (SysHost& h : sys_)
       if (h.active) h.steps += done, h.f_valid = finished;
+    if (!finished && done == 0) continue;  // a list of the first state overflowed (grown now)
+    opened = true;
     if (!finished) {  // a list overflowed after the last drift: the rest of that step
       CKR(launch_step(0.5, 0.0, kStepStoreF, s));
       for (SysHost& h : sys_)
@@ -1370,7 +1382,11 @@ int Engine::step_nvt(int64_t nsteps, const std::vector<double>& dt, const std::v
       CKR(thermostat(it < nsteps ? 2 : 1));
     }
   }
-  if (it < nsteps && !opened) CKR(thermostat(1));
+  if (it < nsteps) {
+    CKR(ensure_lists(s));
+    CKR(ensure_forces(s));
+    if (!opened) CKR(thermostat(1));
+  }
   for (; it < nsteps; ++it) {
     CKR(step(1, dt, s));
     // the end of this step and the start of the next are consecutive half steps

@@ -172,6 +172,8 @@ class Engine {
   int grow_list_arena(int64_t min_extra_units);
   void update_extent();
   int rebuild(std::vector<int> which, cudaStream_t s);
+  int have_states() const;    // kErrState if an active system has none
+  bool forces_valid() const;  // the stored forces are those of the current positions
   int ensure_lists(cudaStream_t s);
   int ensure_forces(cudaStream_t s);
   int launch_step(double ka, double kb, int flags, cudaStream_t s);

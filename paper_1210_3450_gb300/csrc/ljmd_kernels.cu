@@ -147,6 +147,27 @@ __global__ void k_from_caller(DevArrays a, int cur, const double* __restrict__ x
   }
 }
 
+// Positions (wrapped into [0, L)) and velocities in one pass; x or v may be NULL.
+__global__ void k_state_to_caller(DevArrays a, int cur, double* __restrict__ x, double* __restrict__ v, int sys) {
+  const SysParams& P = a.params[sys];
+  const int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (l >= P.n) return;
+  const int64_t s = P.p_off + l;
+  const int64_t i = a.id[s];
+  if (x) {
+    const double4_32a q = a.x[cur][s];  // positions drift outside [0, L) between list builds
+    x[3 * i + 0] = wrap_fast(q.x, P.L);
+    x[3 * i + 1] = wrap_fast(q.y, P.L);
+    x[3 * i + 2] = wrap_fast(q.z, P.L);
+  }
+  if (v) {
+    const double4_32a q = a.v[s];
+    v[3 * i + 0] = q.x;
+    v[3 * i + 1] = q.y;
+    v[3 * i + 2] = q.z;
+  }
+}
+
 // which: 0 = positions (wrapped into [0, L)), 1 = velocities, 2 = stored forces,
 // 4 = positions as held (not wrapped), 5 = positions at the last list build
 __global__ void k_to_caller(DevArrays a, int cur, int which, double* __restrict__ out, int sys) {
@@ -2408,8 +2429,7 @@ __device__ __forceinline__ void loop_worklists(const DevArrays& a, const LoopArg
     a.chunk_pref[r] = ci - chunks;
     g.reb_count[k] += 1;
     const_cast<int32_t*>(a.rebuild)[k] = 1;
-    a.status[k].overflow = 0;
-    a.status[k].max_count = 0;
+    a.status[k] = SysStatus{0, 0, 0, 0};
   } else if (k >= 0) {
     const_cast<int32_t*>(a.rebuild)[k] = 0;
   }
@@ -2606,8 +2626,10 @@ __global__ void __launch_bounds__(kLoopBlock, T == 4 ? (kFP32 ? 4 : 3) : (kFP32 
     }
   };
 
-  for (int k = threadIdx.x; k < g.nsys; k += kLoopBlock) sh.margin[k] = a.margin[k];
-  load_state();
+  for (int k = threadIdx.x; k < g.nsys; k += kLoopBlock) {
+    sh.margin[k] = a.margin[k];
+    sh.need[k] = (int)((g.rebuild0 >> k) & 1u);
+  }
   const int target_steps = a.ctl->target;
   unsigned arrivals = 0;
   int done = 0, abort = 0;
@@ -2662,13 +2684,53 @@ __global__ void __launch_bounds__(kLoopBlock, T == 4 ? (kFP32 ? 4 : 3) : (kFP32 
     if (comp && sh.scale[sys] != 1.0) v *= sh.scale[sys];
     return true;
   };
-  double fnow = 0.0;  // Nose-Hoover steps: the force at the current positions
-  if (kNvt) {
-    if (comp) fnow = ((const double*)&a.f[slot])[c];
-    if (g.open) alive = thermostat(1);
-  }
+  double fnow = 0.0;             // Nose-Hoover steps: the force at the current positions
+  bool begun = false;            // the state is loaded
+  bool pass = g.rebuild0 != 0u;  // a rebuild pass is due (the systems of sh.need)
+  if (!pass) load_state();
 
-  while (alive && done < target_steps) {
+  while (true) {
+    if (pass) {
+      const bool mine = on && sh.need[sys];
+      if (begun && mine && comp) {
+        ((double*)&a.x[cur][slot])[c] = x;
+        ((double*)&a.v[slot])[c] = v;
+      }
+      if (blockIdx.x == 0 && wv == 0) loop_worklists(a, g, sh.need);
+      if (!(alive = grid_barrier(g.bar, arrivals, sh, a.ctl))) break;
+      cell_count_pass<true>(a, cur);
+      if (!(alive = grid_barrier(g.bar, arrivals, sh, a.ctl))) break;
+      cell_starts_pass(a, a.ctl->nreb, sh.ws);
+      if (!(alive = grid_barrier(g.bar, arrivals, sh, a.ctl))) break;
+      scatter_pass<true>(a, cur);
+      if (!(alive = grid_barrier(g.bar, arrivals, sh, a.ctl))) break;
+      cell_rank_pass<true>(a, cur);
+      if (!(alive = grid_barrier(g.bar, arrivals, sh, a.ctl))) break;
+      build_lists_wide(a, cur, T == 32 ? 8 : T == 16 ? 16 : 32, wide);
+      if (!(alive = grid_barrier(g.bar, arrivals, sh, a.ctl))) break;
+      if ((int)threadIdx.x < g.nsys && sh.need[threadIdx.x]) sh.margin[threadIdx.x] = a.margin[threadIdx.x];
+      if (mine || !begun) load_state();
+      abort = *(volatile int*)&a.ctl->abort;
+      __syncthreads();
+      if (abort) break;  // a list overflowed: the host grows it (uniform over the grid)
+    }
+    if constexpr (kNvt) {
+      if (begun) {  // the step's closing half kick and the thermostat half steps
+        if (on) {
+          fnow = force();
+          if (comp) v = fma(h, fnow, v);
+        }
+        if (!(alive = thermostat(done < target_steps ? 2 : g.halves_end))) break;
+      } else {
+        if (on) {
+          if (!g.stored) fnow = force();
+          else if (comp) fnow = ((const double*)&a.f[slot])[c];
+        }
+        if (g.open && !(alive = thermostat(1))) break;
+      }
+    }
+    begun = true;
+    if (done >= target_steps) break;
     unsigned long long d2 = 0ull;
     // block 0 clears the maximum of the next step: its last readers passed a barrier
     if (blockIdx.x == 0 && (int)threadIdx.x < g.nsys) g.disp[((done + 1) % 3) * g.nsys + threadIdx.x] = 0ull;
@@ -2767,37 +2829,7 @@ __global__ void __launch_bounds__(kLoopBlock, T == 4 ? (kFP32 ? 4 : 3) : (kFP32 
     cur ^= 1;
     ++done;
     if (__syncthreads_or(stop)) { abort = 2; break; }
-    if (__syncthreads_or(need)) {  // rebuild pass
-      const bool mine = on && sh.need[sys];
-      if (mine && comp) {
-        ((double*)&a.x[cur][slot])[c] = x;
-        ((double*)&a.v[slot])[c] = v;
-      }
-      if (blockIdx.x == 0 && wv == 0) loop_worklists(a, g, sh.need);
-      if (!(alive = grid_barrier(g.bar, arrivals, sh, a.ctl))) break;
-      cell_count_pass<true>(a, cur);
-      if (!(alive = grid_barrier(g.bar, arrivals, sh, a.ctl))) break;
-      cell_starts_pass(a, a.ctl->nreb, sh.ws);
-      if (!(alive = grid_barrier(g.bar, arrivals, sh, a.ctl))) break;
-      scatter_pass<true>(a, cur);
-      if (!(alive = grid_barrier(g.bar, arrivals, sh, a.ctl))) break;
-      cell_rank_pass<true>(a, cur);
-      if (!(alive = grid_barrier(g.bar, arrivals, sh, a.ctl))) break;
-      build_lists_wide(a, cur, T == 32 ? 8 : T == 16 ? 16 : 32, wide);
-      if (!(alive = grid_barrier(g.bar, arrivals, sh, a.ctl))) break;
-      if ((int)threadIdx.x < g.nsys && sh.need[threadIdx.x]) sh.margin[threadIdx.x] = a.margin[threadIdx.x];
-      if (mine) load_state();
-      abort = *(volatile int*)&a.ctl->abort;
-      __syncthreads();
-      if (abort) break;  // a list overflowed: the host grows it (uniform over the grid)
-    }
-    if constexpr (kNvt) {  // the step's closing half kick and the thermostat half steps
-      if (on) {
-        fnow = force();
-        if (comp) v = fma(h, fnow, v);
-      }
-      if (!(alive = thermostat(done < target_steps ? 2 : g.halves_end))) break;
-    }
+    pass = __syncthreads_or(need) != 0;
   }
 
   double F = 0.0;
@@ -2806,7 +2838,7 @@ __global__ void __launch_bounds__(kLoopBlock, T == 4 ? (kFP32 ? 4 : 3) : (kFP32 
     F = force();
     if (comp) v = fma(h, F, v);
   }
-  if (comp) {
+  if (comp && (alive || begun)) {
     ((double*)&a.x[cur][slot])[c] = x;
     ((double*)&a.v[slot])[c] = v;
     if (!kFP32) ((int*)&a.xq[cur][slot])[c] = to_fixed(x, qscale);
@@ -2856,6 +2888,11 @@ void launch_from_caller(const DevArrays& a, int cur, const double* x, const doub
                         int64_t ntiles_sys, cudaStream_t s) {
   const int64_t n = ntiles_sys * kTile;
   k_from_caller<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(a, cur, x, v, sys);
+}
+
+void launch_state_to_caller(const DevArrays& a, int cur, double* x, double* v, int64_t sys_n, int sys, cudaStream_t s) {
+  if (sys_n <= 0 || (!x && !v)) return;
+  k_state_to_caller<<<(unsigned)((sys_n + 255) / 256), 256, 0, s>>>(a, cur, x, v, sys);
 }
 
 void launch_to_caller(const DevArrays& a, int cur, int which, double* out, int64_t sys_n, int sys,

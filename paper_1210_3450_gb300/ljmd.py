@@ -11,6 +11,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+import sys
 
 import numpy as np
 
@@ -188,7 +189,8 @@ def _stream_ptr(stream) -> int | None:
 
 
 def _dev_ptr(t, n: int) -> int:
-    if not (t.is_cuda and t.is_contiguous() and str(t.dtype) == "torch.float64" and t.numel() == 3 * n):
+    # (torch is loaded if there is a tensor; comparing the dtype's text takes longer than the call)
+    if not (t.is_cuda and t.is_contiguous() and t.dtype is sys.modules["torch"].float64 and t.numel() == 3 * n):
         raise ValueError("expected a contiguous CUDA float64 tensor with N*3 elements")
     return int(t.data_ptr())
 

@@ -86,3 +86,24 @@ def test_nvt_equals_host_loop(ljmd, n, rho, rc, precision):
     for p, q in zip(out[0][:4], out[1][:4]):
         np.testing.assert_array_equal(p, q)
     assert out[0][4] == out[1][4]
+
+
+@pytest.mark.parametrize("precision", [0, 1], ids=["fp64", "fp32"])
+@pytest.mark.parametrize("nvt", [False, True], ids=["nve", "nvt"])
+def test_first_lists_overflow(ljmd, precision, nvt):
+    """A dense block in a wide box: the first list build of the launch outgrows the
+    capacity expected from the density, is grown by the host and taken up again."""
+    n = 1372
+    x, box = li.perturbed_fcc(n, 0.9, 0.05, 5)
+    x, box = x + 0.1, 2.0 * box
+    v = li.maxwell_boltzmann(n, 0.7, 6)
+    out = []
+    for graph in (0, 1):
+        with ljmd.LJSystem(box, n, 2.5, 0.3, precision) as s:
+            s.set_tuning(graph=graph)
+            s.set_state(x, v)
+            ze = s.step_nvt(12, 0.004, 0.7, 3.0 * n * 0.05) if nvt else s.step(12, 0.004)
+            out.append((*s.get_state(), s.forces(), ze, s.stats()))
+    for p, q in zip(out[0][:3], out[1][:3]):
+        np.testing.assert_array_equal(p, q)
+    assert out[0][3:] == out[1][3:]
