@@ -32,7 +32,10 @@ sys.path.insert(0, ROOT)
 
 METRIC = "particle-steps/s (FP32-force vs FP64) + roofline %; p50/p99 batched MD latency"
 UNIT = "particle-steps/s"
-FP64_PEAK_TFLOPS = 1.25  # GB300 nominal dense FP64 (vector and tensor), recipe table
+# Integer multipliers: one 32 x 32 -> 64-bit warp product per 4 cycles of a scheduler
+# (152 SMs x 4 schedulers x 8 lanes a cycle x 2.07 GHz), in 1e12 products per second.
+INT_PRODUCT_PEAK_T = 10.07
+PAIR_PRODUCTS = 32  # of a pair inside rc in the FP64 form (ljmd_fixed.cuh)
 
 # Compulsory bytes per particle-step of the fused FP32 force + integration kernel
 # (k_step_fp32), by name; the list adds 4 bytes per listed partner.
@@ -81,7 +84,7 @@ def workload_config():
 # ------------------------------------------------------------------ helpers
 
 # the device code of the profiled kernels (host code cannot change their traffic)
-KERNEL_SOURCES = ("ljmd_kernels.cu", "ljmd_dev.cuh", "ljmd_math.cuh")
+KERNEL_SOURCES = ("ljmd_kernels.cu", "ljmd_dev.cuh", "ljmd_fixed.cuh", "ljmd_math.cuh")
 
 
 def kernel_source_hash() -> str:
@@ -345,27 +348,27 @@ def run_ours(args):
             "frac_dram": round(traffic / (k_ms / 1e3) / 1e9 / hbm_peak, 4) if traffic else None,
             "avg_launch_ms": round(k_ms, 4),
             "avg_launch_ms_source": "CUDA events around each launch (host-driven pass of the same run)"}
-    # FP64 step kernel: FP64-pipe bound; flops as the method needs them: the
-    # separation and r^2 of every listed pair (10, an FMA counted as 2) and the
-    # force of every pair inside rc (16)
+    # FP64 step kernel: its pairs run on the integer multipliers (64-bit fixed point).
+    # Per pair inside rc 32 products of 32 x 32 -> 64 bits (or their high halves): 6 for
+    # r^2, 4 for its reciprocal, 10 for the force factor, 12 for the three sums.
     t64 = r64["timing"]
     k64 = t64["step_ms"] / max(t64["step_launches"], 1)
     lp64 = r64["listed"] / n
     in64 = r64["inside"] / n
+    ach64 = PAIR_PRODUCTS * in64 * n / (k64 / 1e3) / 1e12
     flops_pp = 10.0 * lp64 + 16.0 * in64
-    ach64 = flops_pp * n / (k64 / 1e3) / 1e12
-    roof64 = {"bound": "alu", "kernel": "k_step_fp64 (classified, queued FP64 pair force + velocity Verlet)",
-              "achieved": round(ach64, 4), "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-              "frac": round(ach64 / FP64_PEAK_TFLOPS, 4),
+    roof64 = {"bound": "alu", "kernel": "k_step_fp64 (classified, queued 64-bit fixed-point pairs + velocity Verlet)",
+              "achieved": round(ach64, 4), "peak": INT_PRODUCT_PEAK_T, "unit": "T 32x32->64-bit products/s",
+              "frac": round(ach64 / INT_PRODUCT_PEAK_T, 4),
               "traffic": profiled_traffic("k_step_fp64", n),
-              "peak_source": "nominal GB300 FP64 (1.25 TFLOP/s, recipe table)",
-              "algorithmic_flops_per_particle_step": round(flops_pp, 1),
-              "flop_count": "10 per listed pair (separation, r^2) + 16 per pair inside rc (force, accumulation)",
+              "peak_source": "one warp product per 4 cycles of a scheduler (measured 4.2): 152 SMs x 4 x 8 lanes x 2.07 GHz",
+              "products_per_pair_inside": PAIR_PRODUCTS,
+              "fp64_equivalent_tflops": round(flops_pp * n / (k64 / 1e3) / 1e12, 4),
+              "fp64_equivalent_flops_per_particle_step": round(flops_pp, 1),
+              "fp64_equivalent_flop_count": "10 per listed pair (separation, r^2) + 16 per pair inside rc (force, accumulation)",
               "avg_launch_ms": round(k64, 4)}
     if rates:
-        meas = 2.0 * rates["fp64_dfma_per_s"] / 1e12
-        roof64.update(peak_measured=round(meas, 4), frac_measured=round(ach64 / meas, 4),
-                      peak_measured_source="md_probe_fma_rate: DFMA chains on every SM, this run")
+        roof64["fp64_pipe_measured_tflops"] = round(2.0 * rates["fp64_dfma_per_s"] / 1e12, 4)
     line = {
         "metric": METRIC, "value": round(value, 1), "unit": UNIT, "n_gpus": world,
         "steps": args.steps, "warmup": args.warmup, "ms_per_step": round(ms32 / args.steps, 5),

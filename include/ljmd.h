@@ -259,7 +259,7 @@ MD_API int md_forces_noalloc(const double* x_dev, int64_t N, double box_L, doubl
 
 /* Measurement utility, not part of the paper's method: the fused multiply-add
  * throughput of one arithmetic pipe of the current device, the denominator of the
- * FP64 force kernel's roofline (that kernel is bound by the FP64 pipe, not HBM).
+ * rooflines of the kernels whose arithmetic runs on that pipe.
  *   kind       0: FP64 (DFMA), 1: FP32 (FFMA)
  *   iters      iterations of eight independent chains per thread (64 warps per SM);
  *              about 1e5 (FP64) or 5e6 (FP32) run for a few hundred milliseconds
@@ -280,7 +280,9 @@ MD_API int md_probe_fma_rate(int kind, int64_t iters, double* fma_per_s);
  *                        4 warp-cooperative (candidates shared by the lanes of a
  *                        row, staged in shared memory); 5 as 0, each row's
  *                        candidates for the whole warp first copied into shared
- *                        memory with coalesced loads
+ *                        memory with coalesced loads (full-list arenas of up to about
+ *                        42,000 particles instead take one candidate per lane, a block
+ *                        for each run of slots)
  *   MD_TUNE_STEP_HINT    1: L1 eviction hints on the FP32 step kernel's loads (list
  *                        words not kept in L1, partner positions kept)
  *   MD_TUNE_GRAPH        1: md_step runs its steps in CUDA-graph launches (a loop node of
@@ -292,10 +294,9 @@ MD_API int md_probe_fma_rate(int kind, int64_t iters, double* fma_per_s);
  *                        decides after every step. Results are identical. Timing (md_set_timing)
  *                        uses the host-driven loop.
  *   MD_TUNE_FP64_QUEUE   1: the FP64 force loops classify each listed pair on the
- *                        fixed-point shadow positions first and run the FP64
- *                        arithmetic only for the pairs that may be inside rc, taken
- *                        from a per-thread queue in list order, so that warps run
- *                        it with full lanes; 0: one plain loop over the list.
+ *                        fixed-point shadow positions first and compute only the
+ *                        pairs that may be inside rc, taken from a per-thread queue in
+ *                        list order, so that warps run them with full lanes; 0: one plain loop over the list.
  *                        Results are identical bit for bit.
  * Defaults 128 / 2 / 128 / 5 / 1 / 1 / 1. The autotuner (paper_1210_3450_gb300.autotune) times the
  * choices on the caller's own systems and sets the fastest. */

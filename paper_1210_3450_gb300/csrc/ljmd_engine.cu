@@ -298,6 +298,7 @@ void Engine::free_all() {
   drop_graphs();
   dfree(d_ctl_); dfree(d_loop_); dfree(d_reb_count_); hfree(h_ctl_); hfree(h_reb_count_);
   d_ = DevArrays{};
+  fixed_off_ = false;
   stage_n_ = 0;
 }
 
@@ -414,24 +415,47 @@ int Engine::alloc_arrays() {
   CK(cudaMallocHost((void**)&h_ctl_, sizeof(GraphCtl)));
   CK(cudaMallocHost((void**)&h_reb_count_, sizeof(int32_t) * ns));
   ++struct_ver_;
-  CKR(ensure_fixed());
   return upload_params();
 }
 
-// The FP64 form's positions in pair units (its full lists only).
-int Engine::ensure_fixed() {
-  if (precision_ != 0 || half_ || d_.xl[0]) return kOK;
-  CKR(dmalloc(&d_.xl[0], 2 * caps_.slots));  // (every slot is written by a rebuild before it is read)
-  d_.xl[1] = d_.xl[0] + caps_.slots;
+// The FP64 form's positions in pair units, allocated for the first lists of that form
+// (every slot is written by a rebuild before it is read). Without memory for them its
+// pairs take the FP64 pipe until the form changes.
+void Engine::ensure_fixed() {
+  if (precision_ != 0 || half_ || d_.xl[0] || fixed_off_) return;
   ++struct_ver_;
-  return kOK;
+  if (dmalloc(&d_.xl[0], 2 * caps_.slots) != kOK) {
+    set_error("");
+    fixed_off_ = true;
+    return;
+  }
+  d_.xl[1] = d_.xl[0] + caps_.slots;
+}
+
+void Engine::drop_fixed(bool off) {
+  dfree(d_.xl[0]);
+  d_.xl[1] = nullptr;
+  fixed_off_ = off;
+  ++struct_ver_;
+}
+
+// An allocation that the positions in pair units give way to.
+template <class T>
+int Engine::dmalloc_first(T** p, int64_t count) {
+  int r = dmalloc(p, count);
+  if (r == kErrOOM && d_.xl[0]) {
+    drop_fixed(true);
+    r = dmalloc(p, count);
+    if (r == kOK) set_error("");
+  }
+  return r;
 }
 
 int Engine::stage(int64_t n, double** out) {
   if (n > stage_n_) {
     dfree(d_stage_);
     stage_n_ = 0;
-    CKR(dmalloc(&d_stage_, 6 * n));
+    CKR(dmalloc_first(&d_stage_, 6 * n));
     stage_n_ = n;
   }
   *out = d_stage_;
@@ -452,7 +476,7 @@ int Engine::grow_list_arena(int64_t min_extra_units) {
   const int64_t old_units = list_alloc_.cap();
   const int64_t new_units = std::max(old_units + old_units / 2, old_units + min_extra_units);
   uint32_t* nb = nullptr;
-  CKR(dmalloc(&nb, new_units * 4 * kTile));
+  CKR(dmalloc_first(&nb, new_units * 4 * kTile));
   CK(cudaMemcpy(nb, d_.nbr, sizeof(uint32_t) * old_units * 4 * kTile, cudaMemcpyDeviceToDevice));
   dfree(d_.nbr);
   d_.nbr = nb;
@@ -662,7 +686,7 @@ int Engine::set_precision(int mode) {
   if (mode != precision_) {
     precision_ = mode;
     ++struct_ver_;
-    CKR(ensure_fixed());
+    drop_fixed(false);  // every list is rebuilt before the next use
     CKR(upload_params());
     for (SysHost& h : sys_) {
       h.f_valid = false;
@@ -690,7 +714,7 @@ int Engine::set_list_kind(int kind) {
   if ((kind == 1) != half_) {
     half_ = kind == 1;
     ++struct_ver_;
-    CKR(ensure_fixed());
+    drop_fixed(false);  // every list is rebuilt before the next use
     for (SysHost& h : sys_) {
       h.f_valid = false;
       if (h.has_state) h.force_rebuild = true;
@@ -778,6 +802,7 @@ int Engine::read_checks(cudaStream_t s) {
 // Full rebuild (bin, stable counting sort, gather, list) of the given systems.
 int Engine::rebuild(std::vector<int> which, cudaStream_t s) {
   if (which.empty()) return kOK;
+  ensure_fixed();
   std::sort(which.begin(), which.end(),
             [&](int p, int q) { return order_rank_[(size_t)p] < order_rank_[(size_t)q]; });
   for (int attempt = 0; attempt < 4; ++attempt) {
@@ -1128,6 +1153,7 @@ int Engine::after_steps(int64_t done, cudaStream_t s) {
 // Threads per particle of the persistent loop: full lists, at most kLoopMaxSys systems,
 // and for the FP64 form the fixed-point range of every system.
 int Engine::loop_plan() {
+  ensure_fixed();
   if (loop_ver_ == struct_ver_) return loop_lanes_;
   loop_ver_ = struct_ver_;
   loop_lanes_ = 0;

@@ -147,7 +147,8 @@ class Engine {
   int set_active(int k, bool on);
   // Launch shapes: key 0 = step-kernel threads per block (64/128/256), 1 = FP32
   // partner groups per iteration (1/2), 2 = list-build threads per block, 3 =
-  // list-build variant, 4 = FP32 load hints, 5 = graph-captured step loop (0/1).
+  // list-build variant, 4 = FP32 load hints, 5 = steps in device-side loops (0/1),
+  // 6 = queued FP64 pairs (0/1).
   int set_tuning(int key, int value);
   int get_tuning(int key) const;
   // Per-kernel-class device times (CUDA events on the launching stream).
@@ -164,7 +165,10 @@ class Engine {
 
  private:
   int alloc_arrays();
-  int ensure_fixed();
+  void ensure_fixed();
+  void drop_fixed(bool off);
+  template <class T>
+  int dmalloc_first(T** p, int64_t count);
   void free_all();
   int upload_params(int only = -1);
   int upload_order();
@@ -240,6 +244,7 @@ class Engine {
   int precision_ = 0;
   int rule_ = 0;
   bool half_ = false;
+  bool fixed_off_ = false;  // no memory for the positions in pair units
   int cur_ = 0;
   ArenaCaps caps_{0, 0, 0, 0};
   bool list_growable_ = false;  // exact-size arenas grow their list storage on demand

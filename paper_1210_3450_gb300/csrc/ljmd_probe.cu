@@ -1,7 +1,6 @@
 // Pipe-rate probe: the FP64 and FP32 fused multiply-add throughput of the current
-// GPU, measured rather than taken from a data sheet, for the denominators of the
-// FP64 force kernel's roofline (its bound is the FP64 pipe, not HBM). Not part of
-// the paper's method.
+// GPU, measured rather than taken from a data sheet, as denominators for kernels
+// whose arithmetic runs on those pipes. Not part of the paper's method.
 //
 // Every thread runs eight independent multiply-add chains (enough to keep the pipe
 // busy between dependent instructions) for a run-time number of iterations, so

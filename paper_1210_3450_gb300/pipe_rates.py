@@ -3,9 +3,9 @@ SM clock sampled while the probe runs; JSON on stdout.
 
     python -m paper_1210_3450_gb300.pipe_rates [--repeats 3]
 
-These are the measured denominators of the FP64 force kernel's roofline (it is
-bound by the FP64 pipe); the nominal GB300 FP64 rate (1.25 TFLOP/s) is reported
-beside them.
+These are the measured denominators for arithmetic on those pipes (the FP64 form's
+integration and its pairs outside the fixed-point range); the nominal GB300 FP64 rate
+(1.25 TFLOP/s) is reported beside them.
 """
 from __future__ import annotations
 

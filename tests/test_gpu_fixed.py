@@ -90,3 +90,31 @@ def test_energy_and_virial_at_the_edges(name, half, precision):
     assert abs(got["pe"] - ref["pe"]) <= 1e-12 * scale[0]
     assert abs(got["virial"] - ref["virial"]) <= 1e-12 * scale[1]
     assert abs(got["ke"] - ref["ke"]) <= 1e-12 * ref["ke"]
+
+
+def test_leaving_and_entering_the_fixed_point_form():
+    """Positions in pair units are held only by the FP64 form's full lists: changing the
+    precision or the list kind and back gives the same forces and steps bit for bit."""
+    from paper_1210_3450_gb300 import MD_FP64, LJSystem
+    from paper_1210_3450_gb300.ljmd import MD_LIST_FULL, MD_LIST_HALF
+    x, box = li.perturbed_fcc(864, 0.8442, 0.1, 5)
+    v = li.maxwell_boltzmann(864, 0.7, 6)
+
+    def run(s):
+        s.set_state(x, v)
+        f = s.forces()
+        s.step(20, 0.005)
+        return (f,) + tuple(s.get_state())
+
+    with LJSystem(box, 864, 2.5, 0.3, MD_FP64) as s:
+        ref = run(s)
+        s.set_precision(1)
+        run(s)
+        s.set_precision(MD_FP64)
+        again = run(s)
+        s.set_pair_list(MD_LIST_HALF)
+        run(s)
+        s.set_pair_list(MD_LIST_FULL)
+        for got in (again, run(s)):
+            for p, q in zip(ref, got):
+                np.testing.assert_array_equal(p, q)
