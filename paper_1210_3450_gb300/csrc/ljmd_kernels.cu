@@ -2024,9 +2024,12 @@ __global__ void __launch_bounds__(kBlock) k_integrate_half(DevArrays a, int cur,
 // fixed point (ljmd_fixed.cuh; sums exact, over the tile as well) where the cutoff
 // allows it, else and for close pairs on the FP64 pipe. With all pairs on that pipe and
 // each taken twice the kernel ran at its rate: 455 us at 262,143 particles.
+// 28 warps per SM (72 registers): a call takes 390 us at 864,000 particles, against 403 at
+// 24 and 426 at 32 warps. Splitting each particle's pairs evenly instead (by slot parity):
+// 398, since whole warps no longer skip the lower half of their lists.
 // xl: positions in pair units.
-__global__ void __launch_bounds__(kBlock) k_pe_virial(DevArrays a, int cur, int with_pairs,
-                                                      const int32_t* __restrict__ select, const longlong4_32a* xl) {
+__global__ void __launch_bounds__(kBlock, 7) k_pe_virial(DevArrays a, int cur, int with_pairs,
+                                                         const int32_t* __restrict__ select, const longlong4_32a* xl) {
   __shared__ uint32_t qbuf[kQueue64][kBlock];
   TileCtx t;
   if (!tile_ref(a, t)) return;              // uniform over the warp
