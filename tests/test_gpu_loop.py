@@ -107,3 +107,19 @@ def test_first_lists_overflow(ljmd, precision, nvt):
     for p, q in zip(out[0][:3], out[1][:3]):
         np.testing.assert_array_equal(p, q)
     assert out[0][3:] == out[1][3:]
+
+
+@pytest.mark.parametrize("precision", [0, 1], ids=["fp64", "fp32"])
+def test_several_threads(ljmd, precision):
+    """Systems stepped by threads of their own at the same time, each on its stream: every
+    one as it runs alone, bit for bit."""
+    from concurrent.futures import ThreadPoolExecutor
+    args = [(n, rho, 2.5, 0.1, 0.9, precision, 1, (30, 7, 30), 0.005)
+            for n, rho in ((1000, 0.8442), (9729, 0.6), (29185, 0.8), (29185, 0.75))]
+    alone = [_run(ljmd, *a) for a in args]
+    with ThreadPoolExecutor(len(args)) as pool:
+        together = list(pool.map(lambda a: _run(ljmd, *a), args))
+    for a, b in zip(alone, together):
+        for p, q in zip(a[:3], b[:3]):
+            np.testing.assert_array_equal(p, q)
+        assert a[3] == b[3]
