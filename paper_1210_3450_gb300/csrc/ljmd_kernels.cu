@@ -1748,11 +1748,16 @@ __device__ __forceinline__ void queued_pairs(const DevArrays& a, const TileCtx& 
       const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
       k += 4;
       if (k < cnt) w = __ldg(lp4 + (int64_t)(k >> 2) * kTile);  // the next group's load in flight
+      int4 q4[4];  // all four in flight before the first test: 3 % of the step
+      if (!kUpper) {
+#pragma unroll
+        for (int m = 0; m < 4; ++m) q4[m] = qs[partner_slot(a, t.sys, ws[m], P.n, self)];
+      }
 #pragma unroll
       for (int m = 0; m < 4; ++m) {
         const uint32_t j = partner_slot(a, t.sys, ws[m], P.n, self);
         if (kUpper && j <= self) continue;
-        const int4 qj = qs[j];
+        const int4 qj = kUpper ? qs[j] : q4[m];
         const float ax = (float)wrapped_diff(qj.x, qi.x);
         const float ay = (float)wrapped_diff(qj.y, qi.y);
         const float az = (float)wrapped_diff(qj.z, qi.z);
