@@ -3235,7 +3235,17 @@ void launch_step_fp32(const DevArrays& a, int cur, double ka, double kb, int fla
 namespace {
 template <bool kFP32, int T, bool kNvt>
 cudaError_t loop_setup_k(size_t bytes, int* blocks_per_sm) {
-  cudaError_t e = cudaFuncSetAttribute(k_loop<kFP32, T, kNvt>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  // The limit belongs to the kernel, not to a launch: always the largest one, so that
+  // threads with other sizes do not lower it under each other's launches.
+  int dev = 0, optin = 0;
+  cudaFuncAttributes fa{};
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_loop<kFP32, T, kNvt>);
+  if (e != cudaSuccess) return e;
+  const int most = optin - (int)fa.sharedSizeBytes;
+  if (bytes > (size_t)most) return cudaErrorInvalidValue;
+  e = cudaFuncSetAttribute(k_loop<kFP32, T, kNvt>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
   if (e == cudaSuccess)
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_loop<kFP32, T, kNvt>, kLoopBlock, bytes);
   return e;
