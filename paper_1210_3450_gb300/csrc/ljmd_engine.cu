@@ -1154,17 +1154,21 @@ int Engine::after_steps(int64_t done, cudaStream_t s) {
 // and for the FP64 form the fixed-point range of every system.
 int Engine::loop_plan() {
   ensure_fixed();
-  if (loop_ver_ == struct_ver_) return loop_lanes_;
-  loop_ver_ = struct_ver_;
-  loop_lanes_ = 0;
   if (half_ || precision_ > 1 || nsys() > kLoopMaxSys) return 0;
+  // A list's capacity can grow without a change of struct_ver_ (within the arena's free
+  // words), so the plan is made for both.
   int kmax = 0;
-  for (const SysHost& h : sys_) {
-    if (!h.used) continue;
-    kmax = std::max(kmax, h.kmax);
-    if (precision_ == 0 && (h.spec.rc > kFixMaxRc || h.kmax > kFixMaxList)) return 0;
+  for (const SysHost& h : sys_)
+    if (h.used) kmax = std::max(kmax, h.kmax);
+  if (loop_ver_ == struct_ver_ && loop_kmax_ == kmax) return loop_lanes_;
+  loop_ver_ = struct_ver_;
+  loop_kmax_ = kmax;
+  loop_lanes_ = 0;
+  if (precision_ == 0) {
+    if (!d_.xl[0] || kmax > kFixMaxList) return 0;
+    for (const SysHost& h : sys_)
+      if (h.used && h.spec.rc > kFixMaxRc) return 0;
   }
-  if (precision_ == 0 && !d_.xl[0]) return 0;
   loop_lanes_ = loop_lanes(precision_ == 1, ntiles_, kmax, &loop_stride_);
   return loop_lanes_;
 }

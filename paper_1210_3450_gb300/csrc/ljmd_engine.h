@@ -235,7 +235,8 @@ class Engine {
   unsigned long long* d_loop_ = nullptr;  // persistent loop: barrier word, 3 maxima and 12 energy limbs per system
   Thermo* d_thermo_ = nullptr;            // thermostats (nsys) of md_step_nvt
   int loop_lanes_ = 0, loop_stride_ = 0;
-  int64_t loop_ver_ = -1;                 // struct_ver_ the plan was made for
+  int64_t loop_ver_ = -1;                 // struct_ver_ the plan was made for ...
+  int loop_kmax_ = -1;                    // ... and the longest list capacity
   GraphCtl* h_ctl_ = nullptr;
   int32_t* d_reb_count_ = nullptr;
   int32_t* h_reb_count_ = nullptr;

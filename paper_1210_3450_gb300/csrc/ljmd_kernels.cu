@@ -2517,6 +2517,7 @@ __global__ void __launch_bounds__(kLoopBlock, T == 4 ? (kFP32 ? 4 : 3) : (kFP32 
     }
     const int most = __reduce_max_sync(kFull, cnt);
     niter = (most + CH * T - 1) / (CH * T);
+    if (!check_ok(a, sys < 0 ? 0 : sys, niter * CH * T <= g.stride, kChkCount)) niter = g.stride / (CH * T);
     const uint32_t* lp = a.nbr + (on ? list_word(P.l_off, local / kTile, P.kmax, local % kTile, 0) : 0);
     for (int k = sub; k < niter * CH * T; k += T) {
       uint32_t e = (uint32_t)local;
