@@ -75,6 +75,7 @@ struct SysParams {
   int32_t rule;      // list validity: 0 displacement (2 d_max >= skin), 1 velocity bound (DUTC)
   int32_t half;      // 1: half list (each pair once, in its lower slot's list; Newton's third law)
   int32_t fixed;     // 1: the cutoff is in the range of the 64-bit fixed-point pair arithmetic (rc <= kFixMaxRc)
+  int32_t wide;      // 1: listed pairs may come apart farther than its separations reach (fix_wide)
 };
 
 // Per-system status words written by kernels and read by the host.

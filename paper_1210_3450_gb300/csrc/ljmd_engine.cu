@@ -599,6 +599,7 @@ int Engine::upload_params(int only) {
     }
     P.Lfix = fix_host(h.spec.L);
     P.fixed = h.spec.rc <= kFixMaxRc ? 1 : 0;
+    P.wide = fix_wide(h.spec.rc, h.spec.skin) ? 1 : 0;
     if (P.fixed) {
       P.rc2fix = (long long)std::llrint(std::ldexp(P.rc2, 56));
       P.c2fix = (long long)std::llrint(std::ldexp(h.c2 / 3.0, 56)) + kFixBias;
@@ -1151,7 +1152,8 @@ int Engine::after_steps(int64_t done, cudaStream_t s) {
 }
 
 // Threads per particle of the persistent loop: full lists, at most kLoopMaxSys systems,
-// and for the FP64 form the fixed-point range of every system.
+// and for the FP64 form the fixed-point range of every system, for all its listed pairs
+// (the loop does not test them on the shadows first).
 int Engine::loop_plan() {
   ensure_fixed();
   if (half_ || precision_ > 1 || nsys() > kLoopMaxSys) return 0;
@@ -1167,7 +1169,7 @@ int Engine::loop_plan() {
   if (precision_ == 0) {
     if (!d_.xl[0] || kmax > kFixMaxList) return 0;
     for (const SysHost& h : sys_)
-      if (h.used && h.spec.rc > kFixMaxRc) return 0;
+      if (h.used && (h.spec.rc > kFixMaxRc || fix_wide(h.spec.rc, h.spec.skin))) return 0;
   }
   loop_lanes_ = loop_lanes(precision_ == 1, ntiles_, kmax, &loop_stride_);
   return loop_lanes_;

@@ -22,6 +22,10 @@
 //   force sums / 24       2^-84   (96 bits; 468 pairs of the largest force, 4.37,
 //                         reach their range)
 // Pairs closer than sqrt(0.84) and lists longer than kFixMaxList take the FP64 pipe.
+// Separations of kFixMaxSep and more may come out of the wrapped differences as shorter
+// ones (and r^2 of 128 and more as a negative number), so a loop that hands every listed
+// pair on, and not only those that passed a test on the shadows, must know that no listed
+// pair comes that far apart.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -33,6 +37,7 @@ namespace ljmd {
 constexpr int kFixMaxList = 448;                                // longest list summed in 96 bits
 constexpr unsigned kFixR2Min = 14092862u;                      // 0.84 in units of 2^-24 (r^2's high word)
 constexpr double kFixMaxRc = 3.99;                              // r^2 < 16
+constexpr double kFixMaxSep = 7.9;                              // separations below 8, r^2 < 128
 
 // A number split into a signed high and a signed low half (the low half rounded to
 // nearest): products of halves are signed 32 x 32 -> 64. fix_split takes the number
@@ -328,6 +333,10 @@ static __device__ __forceinline__ bool fix_pair(const longlong4_32a& qi, const l
   }
   return !far;
 }
+
+// Whether pairs listed within rc + skin may come kFixMaxSep apart before the list is built
+// anew (either rule rebuilds once two particles may have moved `skin` against each other).
+static inline bool fix_wide(double rc, double skin) { return !(rc + 2.0 * skin <= kFixMaxSep); }
 
 // x >= 2^-8 in position units (host; exact).
 static inline long long fix_host(double x) {

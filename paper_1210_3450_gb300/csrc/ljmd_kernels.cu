@@ -1888,8 +1888,15 @@ __global__ void __launch_bounds__(BLOCK, MODE == 0 ? 1024 / BLOCK : 1) k_step_fp
                           [&](const longlong4_32a& q, uint32_t e) { pf.pair(q, e); });
     } else {
       const uint32_t* lp = a.nbr + list_word(P.l_off, t.tl, P.kmax, lane, 0);
+      const bool shadows = MODE == 0 && pf.fixed && P.wide;
       for (int k = 0; k < cnt; ++k) {
         const uint32_t e = __ldg(lp + (int64_t)(k >> 2) * (4 * kTile) + (k & 3));
+        if (shadows) {  // the queue's test: pairs surely outside rc, which may be out of range, are left out
+          const int4 qi = a.xq[cur][t.s], qj = a.xq[cur][P.p_off + pf.slot(e)];
+          const float ax = (float)wrapped_diff(qj.x, qi.x), ay = (float)wrapped_diff(qj.y, qi.y),
+                      az = (float)wrapped_diff(qj.z, qi.z);
+          if (!(fmaf(az, az, fmaf(ay, ay, ax * ax)) < P.rc2q_hi)) continue;
+        }
         pf.pair(pf.load(e), e);
       }
     }
