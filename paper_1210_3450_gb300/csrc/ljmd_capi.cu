@@ -303,6 +303,12 @@ int md_debug_set_list_word(md_ctx* c, int64_t slot, int32_t entry, uint32_t word
   return c->eng.debug_set_list_word(0, slot, entry, word, c->stream);
 }
 
+int md_debug_loop_polls(md_ctx* c, int64_t polls) {
+  int r = check_ctx(c);
+  if (r) return r;
+  return c->eng.debug_loop_polls(polls);
+}
+
 int md_get_list(md_ctx* c, int64_t* start, int32_t* partners) {
   int r = check_ctx(c);
   if (r) return r;

@@ -129,6 +129,7 @@ struct LoopArgs {
   int finish;    // 1: after the last step, forces (stored) and the closing half kick
   int stride;    // list words per particle in shared memory
   int lanes;     // threads per particle
+  int polls;     // of a grid barrier before the launch gives up
   int32_t* rebuild_ids;
   int32_t* reb_pref;
   int32_t* reb_count;

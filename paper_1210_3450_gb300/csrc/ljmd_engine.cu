@@ -1151,6 +1151,19 @@ int Engine::after_steps(int64_t done, cudaStream_t s) {
   return kOK;
 }
 
+// After a launch that ended anywhere in its steps: the positions, velocities and lists of
+// the systems that took part may be those of different steps, so they have no state until
+// a new one is set. The cell counters, which every binning leaves at zero, may be in use.
+int Engine::lose_states(cudaStream_t s) {
+  for (SysHost& h : sys_) {
+    if (!h.used || !h.active) continue;
+    h.has_state = h.f_valid = false;
+    h.force_rebuild = true;
+    CK(cudaMemsetAsync(d_.ccount + h.c_off, 0, sizeof(int32_t) * (h.ncell + 1), s));
+  }
+  return sync_check(s);
+}
+
 // Threads per particle of the persistent loop: full lists, at most kLoopMaxSys systems,
 // and for the FP64 form the fixed-point range of every system, for all its listed pairs
 // (the loop does not test them on the shadows first).
@@ -1199,6 +1212,7 @@ int Engine::run_loop(int64_t nsteps, bool stored, bool steady, int64_t* done, bo
   g.finish = 1;
   g.stride = loop_stride_;
   g.lanes = loop_lanes_;
+  g.polls = loop_polls_;
   g.rebuild_ids = d_rebuild_ + nsys();
   g.reb_pref = d_rebuild_ + 2 * nsys();
   g.reb_count = d_reb_count_;
@@ -1222,7 +1236,8 @@ int Engine::run_loop(int64_t nsteps, bool stored, bool steady, int64_t* done, bo
   CKR(sync_check(s));
   n_launch_ += 1;
   if (h_ctl_->abort == 3) {
-    set_error("a grid barrier of the step loop gave up");
+    CKR(lose_states(s));
+    set_error("a grid barrier of the step loop gave up: the states are lost");
     return kErrTimeout;
   }
   *done = h_ctl_->done;
@@ -1538,6 +1553,12 @@ int Engine::debug_set_list_word(int k, int64_t slot, int m, uint32_t word, cudaS
   const int64_t w = list_word(h.l_off, (int)(slot / kTile), h.kmax, (int)(slot % kTile), m);
   CK(cudaMemcpyAsync(d_.nbr + w, &word, sizeof(uint32_t), cudaMemcpyHostToDevice, s));
   return sync_check(s);
+}
+
+int Engine::debug_loop_polls(int64_t polls) {
+  if (polls < 0 || polls > 1 << 30) { set_error("polls out of range"); return kErrArg; }
+  loop_polls_ = (int)polls;
+  return kOK;
 }
 
 int Engine::get_list(int k, int64_t* start, int32_t* partners, cudaStream_t s) {

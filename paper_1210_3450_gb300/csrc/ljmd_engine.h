@@ -142,6 +142,7 @@ class Engine {
   int list_size(int k, int64_t* total, cudaStream_t s);
   // Checked build only: overwrite list entry m of sorted slot `slot` (a test of the checks).
   int debug_set_list_word(int k, int64_t slot, int m, uint32_t word, cudaStream_t s);
+  int debug_loop_polls(int64_t polls);
   int get_list(int k, int64_t* start, int32_t* partners, cudaStream_t s);
 
   int set_active(int k, bool on);
@@ -200,6 +201,7 @@ class Engine {
   int run_loop(int64_t nsteps, bool stored, bool steady, int64_t* done, bool* finished, cudaStream_t s,
                bool nvt = false, bool open = false, int halves_end = 1);
   int after_steps(int64_t done, cudaStream_t s);
+  int lose_states(cudaStream_t s);
   int sync_check(cudaStream_t s);
   bool any_active() const;  // some system takes part in launches
   int read_checks(cudaStream_t s);  // checked build: MD_ERR_CHECK if a device check failed
@@ -235,6 +237,7 @@ class Engine {
   unsigned long long* d_loop_ = nullptr;  // persistent loop: barrier word, 3 maxima and 12 energy limbs per system
   Thermo* d_thermo_ = nullptr;            // thermostats (nsys) of md_step_nvt
   int loop_lanes_ = 0, loop_stride_ = 0;
+  int loop_polls_ = 1 << 21;              // of a grid barrier before it gives up (about a second)
   int64_t loop_ver_ = -1;                 // struct_ver_ the plan was made for ...
   int loop_kmax_ = -1;                    // ... and the longest list capacity
   GraphCtl* h_ctl_ = nullptr;

@@ -2380,7 +2380,6 @@ namespace {
 
 constexpr int kLoopBlock = 256;
 constexpr int kLoopWarps = kLoopBlock / 32;
-constexpr int kBarrierPolls = 1 << 21;  // about a second, then the launch gives up
 
 __host__ __device__ constexpr int loop_chunk(int T) { return T >= 32 ? 3 : 4; }  // pairs per thread between exchanges
 // FP32 exchange buffer of one particle (words; the 4 extra ones keep the particles of a
@@ -2408,20 +2407,22 @@ struct LoopShared {
 };
 
 // Every block of the (cooperative) launch arrives before any passes. False if the wait
-// ran out; `target` counts this block's barriers in arrivals.
-__device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned& target, LoopShared& sh, GraphCtl* ctl) {
+// ran out; `target` counts this block's barriers in arrivals. A block that gave up arrives
+// no more, so no other block gets past its next barrier: the phases behind a barrier only
+// ever run on complete ones before it.
+__device__ __forceinline__ bool grid_barrier(const LoopArgs& g, unsigned& target, LoopShared& sh, GraphCtl* ctl) {
   __syncthreads();
   if (threadIdx.x == 0) {
     target += gridDim.x;
     __threadfence();  // the block's writes (ordered before it by the barrier above)
-    atomicAdd(bar, 1u);
+    atomicAdd(g.bar, 1u);
     int polls = 0;
     unsigned v;
     do {
-      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
-    } while ((int)(v - target) < 0 && ++polls < kBarrierPolls);
-    sh.flag = polls < kBarrierPolls;
-    if (polls >= kBarrierPolls) atomicMax(&ctl->abort, 3);
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(g.bar) : "memory");
+    } while ((int)(v - target) < 0 && ++polls < g.polls);
+    sh.flag = polls < g.polls;
+    if (polls >= g.polls) atomicMax(&ctl->abort, 3);
   }
   __syncthreads();
   return sh.flag != 0;
@@ -2698,7 +2699,7 @@ __global__ void __launch_bounds__(kLoopBlock, T == 4 ? (kFP32 ? 4 : 3) : (kFP32 
         add_limbs(ke + 4 * k, m);
       }
     }
-    if (!grid_barrier(g.bar, arrivals, sh, a.ctl)) return false;
+    if (!grid_barrier(g, arrivals, sh, a.ctl)) return false;
     if (dactive) {
       const unsigned long long* ke = g.ke + ((turn % 3) * g.nsys + threadIdx.x) * 4;
       sh.scale[threadIdx.x] = thermo_halves(thermo, limbs_ke(__ldcg(ke), __ldcg(ke + 1), __ldcg(ke + 2), __ldcg(ke + 3)), halves);
@@ -2721,17 +2722,17 @@ __global__ void __launch_bounds__(kLoopBlock, T == 4 ? (kFP32 ? 4 : 3) : (kFP32 
         ((double*)&a.v[slot])[c] = v;
       }
       if (blockIdx.x == 0 && wv == 0) loop_worklists(a, g, sh.need);
-      if (!(alive = grid_barrier(g.bar, arrivals, sh, a.ctl))) break;
+      if (!(alive = grid_barrier(g, arrivals, sh, a.ctl))) break;
       cell_count_pass<true>(a, cur);
-      if (!(alive = grid_barrier(g.bar, arrivals, sh, a.ctl))) break;
+      if (!(alive = grid_barrier(g, arrivals, sh, a.ctl))) break;
       cell_starts_pass(a, a.ctl->nreb, sh.ws);
-      if (!(alive = grid_barrier(g.bar, arrivals, sh, a.ctl))) break;
+      if (!(alive = grid_barrier(g, arrivals, sh, a.ctl))) break;
       scatter_pass<true>(a, cur);
-      if (!(alive = grid_barrier(g.bar, arrivals, sh, a.ctl))) break;
+      if (!(alive = grid_barrier(g, arrivals, sh, a.ctl))) break;
       cell_rank_pass<true>(a, cur);
-      if (!(alive = grid_barrier(g.bar, arrivals, sh, a.ctl))) break;
+      if (!(alive = grid_barrier(g, arrivals, sh, a.ctl))) break;
       build_lists_wide(a, cur, T == 32 ? 8 : T == 16 ? 16 : 32, wide);
-      if (!(alive = grid_barrier(g.bar, arrivals, sh, a.ctl))) break;
+      if (!(alive = grid_barrier(g, arrivals, sh, a.ctl))) break;
       if ((int)threadIdx.x < g.nsys && sh.need[threadIdx.x]) sh.margin[threadIdx.x] = a.margin[threadIdx.x];
       if (mine || !begun) load_state();
       abort = *(volatile int*)&a.ctl->abort;
@@ -2830,7 +2831,7 @@ __global__ void __launch_bounds__(kLoopBlock, T == 4 ? (kFP32 ? 4 : 3) : (kFP32 
         atomicMax(&g.disp[(done % 3) * g.nsys + k], m);
       }
     }
-    if (!grid_barrier(g.bar, arrivals, sh, a.ctl)) { alive = false; break; }
+    if (!grid_barrier(g, arrivals, sh, a.ctl)) { alive = false; break; }
     // the list-validity decision (k_decide's)
     bool need = false, stop = false;
     if ((int)threadIdx.x < g.nsys) {

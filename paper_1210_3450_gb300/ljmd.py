@@ -91,6 +91,7 @@ SIGNATURES = {
     "md_batch_get_checkpoint": (C.c_int, [_P, C.c_int, _PD, _PD, _PD, _PD]),
     "md_batch_set_checkpoint": (C.c_int, [_P, C.c_int, _PD, _PD, _PD, C.c_double]),
     "md_debug_set_list_word": (C.c_int, [_P, C.c_int64, C.c_int32, C.c_uint32]),
+    "md_debug_loop_polls": (C.c_int, [_P, C.c_int64]),
     "md_get_list": (C.c_int, [_P, _PI64, _PI32]),
     "md_pair_stats": (C.c_int, [_P, _PI64, _PI64]),
     "md_bubbles": (C.c_int, [_P, C.c_double, C.c_double, _PI32, C.POINTER(C.c_uint8), _PI64, _PI64, C.c_int64]),
@@ -327,6 +328,10 @@ class LJSystem:
     def debug_set_list_word(self, slot: int, entry: int, word: int):
         """Checked build only: overwrite one raw list word (a test of the device checks)."""
         _check(_lib.md_debug_set_list_word(self._h, int(slot), int(entry), int(word) & 0xFFFFFFFF))
+
+    def debug_loop_polls(self, polls: int):
+        """Poll limit of the one-launch step loop's waits (a test of its giving up)."""
+        _check(_lib.md_debug_loop_polls(self._h, int(polls)))
 
     def list_size(self) -> int:
         t = C.c_int64()
