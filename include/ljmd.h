@@ -208,7 +208,9 @@ MD_API int md_debug_set_list_word(md_ctx* ctx, int64_t slot, int32_t entry, uint
 /* For tests of a failing step loop: the waits of the one-launch step loop of small arenas
  * (see MD_TUNE_GRAPH) give up after `polls` polls (>= 0) instead of after about a second.
  * A call whose wait gave up returns MD_ERR_TIMEOUT, and the systems that took part have
- * no state until one is set. Errors: MD_ERR_ARG. */
+ * no state until one is set. polls = -1: the launch itself counts as refused by the driver
+ * (as where a part of the device cannot hold all its blocks at once), and the call takes
+ * its steps in graph launches. Errors: MD_ERR_ARG. */
 MD_API int md_debug_loop_polls(md_ctx* ctx, int64_t polls);
 
 /* Current full list in caller numbering: start[N+1] (int64) and partners[total] (int32)

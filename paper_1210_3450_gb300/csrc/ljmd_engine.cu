@@ -1225,10 +1225,14 @@ int Engine::run_loop(int64_t nsteps, bool stored, bool steady, int64_t* done, bo
     g.halves_end = halves_end;
     g.finish = 0;
   }
-  const cudaError_t e = launch_loop(a, g, s);
+  const cudaError_t e = loop_polls_ < 0 ? cudaErrorCooperativeLaunchTooLarge : launch_loop(a, g, s);
   if (e != cudaSuccess) {
-    set_error(std::string("persistent step loop: ") + cudaGetErrorString(e));
-    return kErrCuda;
+    // refused (a stream that has only a part of the device may not hold all blocks at
+    // once): no step is taken here, the caller goes on without the loop, and an error that
+    // is not the loop's own comes up there
+    cudaGetLastError();
+    loop_lanes_ = 0;
+    return kOK;
   }
   CK(cudaMemcpyAsync(h_ctl_, d_ctl_, sizeof(GraphCtl), cudaMemcpyDeviceToHost, s));
   CK(cudaMemcpyAsync(h_reb_count_, d_reb_count_, sizeof(int32_t) * nsys(), cudaMemcpyDeviceToHost, s));
@@ -1556,8 +1560,9 @@ int Engine::debug_set_list_word(int k, int64_t slot, int m, uint32_t word, cudaS
 }
 
 int Engine::debug_loop_polls(int64_t polls) {
-  if (polls < 0 || polls > 1 << 30) { set_error("polls out of range"); return kErrArg; }
+  if (polls < -1 || polls > 1 << 30) { set_error("polls out of range"); return kErrArg; }
   loop_polls_ = (int)polls;
+  loop_ver_ = -1;  // (a refused launch is tried again)
   return kOK;
 }
 

@@ -330,7 +330,8 @@ class LJSystem:
         _check(_lib.md_debug_set_list_word(self._h, int(slot), int(entry), int(word) & 0xFFFFFFFF))
 
     def debug_loop_polls(self, polls: int):
-        """Poll limit of the one-launch step loop's waits (a test of its giving up)."""
+        """Poll limit of the one-launch step loop's waits, -1: the launch counts as
+        refused (a test of its giving up and of its fallback)."""
         _check(_lib.md_debug_loop_polls(self._h, int(polls)))
 
     def list_size(self) -> int:

@@ -50,9 +50,29 @@ def test_state_is_lost_and_can_be_set_again(ljmd, precision, nvt, polls):
             np.testing.assert_array_equal(p, q)
 
 
+@pytest.mark.parametrize("nvt", [False, True], ids=["nve", "nvt"])
+@pytest.mark.parametrize("precision", [0, 1], ids=["fp64", "fp32"])
+def test_refused_launch(ljmd, precision, nvt):
+    """A refused launch: the call takes its steps as without the loop, and so does the next."""
+    n = 2000
+    x, box = li.perturbed_fcc(n, 0.8442, 0.1, 23)
+    v = li.maxwell_boltzmann(n, 0.9, 24)
+    out = []
+    for polls in (1 << 21, -1):
+        with ljmd.LJSystem(box, n, 2.5, 0.3, precision) as s:
+            s.debug_loop_polls(polls)
+            s.set_state(x, v)
+            ze = []
+            for steps in (11, 1, 4):
+                ze += s.step_nvt(steps, 0.005, 0.9, 3.0 * n * 0.05) if nvt else [s.step(steps, 0.005)]
+            out.append((*s.get_state(), s.forces(), np.array(ze if nvt else [0.0]), np.array(list(s.stats().values()))))
+    for p, q in zip(*out):
+        np.testing.assert_array_equal(p, q)
+
+
 def test_limit_is_checked(ljmd):
     with ljmd.LJSystem(20.0, 100, 2.5, 0.3) as s:
-        for bad in (-1, 1 << 31):
+        for bad in (-2, 1 << 31):
             with pytest.raises(ljmd.MDError) as e:
                 s.debug_loop_polls(bad)
             assert e.value.code == ljmd.MD_ERR_ARG
