@@ -1405,6 +1405,23 @@ int Engine::step_nvt(int64_t nsteps, const std::vector<double>& dt, const std::v
   CK(cudaMemcpyAsync(d_thermo_, th.data(), sizeof(Thermo) * (size_t)ns, cudaMemcpyHostToDevice, s));
   unsigned long long* ke = d_loop_ + 1 + 3 * (size_t)ns;
   CK(cudaMemsetAsync(ke, 0, sizeof(unsigned long long) * 4 * (size_t)ns, s));
+  const int rc = nvt_steps(nsteps, dt, ke, s);
+  if (rc == kErrTimeout) return rc;  // the states are lost
+  // after an error in a step as well: the thermostats have moved with the particles
+  const std::string why = last_error_cstr();
+  CK(cudaMemcpyAsync(th.data(), d_thermo_, sizeof(Thermo) * (size_t)ns, cudaMemcpyDeviceToHost, s));
+  CKR(sync_check(s));
+  for (int k = 0; k < ns; ++k) {
+    if (!sys_[k].active) continue;
+    zeta[k] = th[(size_t)k].zeta;
+    eta[k] = th[(size_t)k].eta;
+  }
+  set_error(why);
+  return rc;
+}
+
+int Engine::nvt_steps(int64_t nsteps, const std::vector<double>& dt, unsigned long long* ke, cudaStream_t s) {
+  const int ns = nsys();
   auto thermostat = [&](int halves) -> int {
     launch_thermostat(arrays(), ns, d_thermo_, halves, ke, d_obs_, s);
     CKL();
@@ -1443,13 +1460,6 @@ int Engine::step_nvt(int64_t nsteps, const std::vector<double>& dt, const std::v
     // the end of this step and the start of the next are consecutive half steps
     CK(cudaMemsetAsync(ke, 0, sizeof(unsigned long long) * 4 * (size_t)ns, s));
     CKR(thermostat(it + 1 < nsteps ? 2 : 1));
-  }
-  CK(cudaMemcpyAsync(th.data(), d_thermo_, sizeof(Thermo) * (size_t)ns, cudaMemcpyDeviceToHost, s));
-  CKR(sync_check(s));
-  for (int k = 0; k < ns; ++k) {
-    if (!sys_[k].active) continue;
-    zeta[k] = th[(size_t)k].zeta;
-    eta[k] = th[(size_t)k].eta;
   }
   return kOK;
 }

@@ -202,6 +202,7 @@ class Engine {
                bool nvt = false, bool open = false, int halves_end = 1);
   int after_steps(int64_t done, cudaStream_t s);
   int lose_states(cudaStream_t s);
+  int nvt_steps(int64_t nsteps, const std::vector<double>& dt, unsigned long long* ke, cudaStream_t s);
   int sync_check(cudaStream_t s);
   bool any_active() const;  // some system takes part in launches
   int read_checks(cudaStream_t s);  // checked build: MD_ERR_CHECK if a device check failed

@@ -52,3 +52,27 @@ def test_nvt_batch_equals_alone(ljmd):
             np.testing.assert_array_equal(xb, xs)
             np.testing.assert_array_equal(vb, vs)
             assert z[k] == zk and e[k] == ek
+
+
+def test_thermostat_after_an_error(ljmd):
+    """A step that ends with MD_ERR_NONFINITE gives back the thermostat that the velocities
+    have moved with: the opening half step, with and without the loop."""
+    import ctypes as C
+    n, dt, T, Q, z0, e0 = 500, 0.005, 0.9, 70.0, 0.25, -1.0
+    x, box = li.perturbed_fcc(n, 0.8, 0.05, 805)
+    x[7, 1] = np.nan
+    v = li.maxwell_boltzmann(n, 1.3, 806)
+    ke = 0.5 * (v * v).sum()
+    gT = 3.0 * (n - 1) * T
+    zeta = z0 + 0.25 * dt * (2.0 * ke - gT) / Q
+    eta = e0 + 0.5 * dt * zeta
+    zeta += 0.25 * dt * (2.0 * ke * np.exp(-dt * zeta) - gT) / Q
+    for graph in (0, 1):
+        with ljmd.LJSystem(box, n, 2.5, 0.3) as s:
+            s.set_tuning(graph=graph)
+            s.set_state(x, v)
+            z, e = C.c_double(z0), C.c_double(e0)
+            rc = ljmd.load_library().md_step_nvt(s._h, 50, dt, T, Q, C.byref(z), C.byref(e))
+            assert rc == ljmd.MD_ERR_NONFINITE
+            assert b"non-finite" in ljmd.load_library().md_last_error()
+            assert abs(z.value - zeta) < 1e-12 and abs(e.value - eta) < 1e-12
