@@ -137,13 +137,15 @@ struct LoopArgs {
   unsigned* bar;             // grid barrier's arrival count (zeroed before the launch)
   // Nose-Hoover steps (thermo != NULL): the launch starts with a thermostat half step if
   // `open` is set, then takes `halves_end` half steps after its last step (two after each
-  // other one); ke: 3 x 4 limbs of the kinetic-energy sums per system, taken in turn
-  // (zeroed before the launch)
+  // other one); ke: 3 x kKeWords words of the kinetic-energy sums per system, taken in
+  // turn (zeroed before the launch)
   Thermo* thermo;
   unsigned long long* ke;
   int open, halves_end;
 };
 constexpr int kLoopMaxSys = 32;
+constexpr int kKeWords = 9;                  // of a kinetic-energy sum: 8 limbs, squares out of range
+constexpr int kLoopWords = 3 + 3 * kKeWords; // per system: the maxima and sums above
 
 struct DevArrays {
   double4_32a* x[2];      // positions (w unused), ping-pong by step parity
@@ -265,8 +267,8 @@ void launch_step_fp32(const DevArrays& a, int cur, double ka, double kb, int fla
 // select: per-system flags (NULL = every active system)
 void launch_pe_virial(const DevArrays& a, int cur, int with_pairs, const int32_t* select, cudaStream_t s);
 void launch_scale_v(const DevArrays& a, const double* scale, cudaStream_t s);
-// `halves` thermostat half steps of every active system: kinetic energies (4 limbs per
-// system in ke, zero before and after), factors into scale, velocities scaled.
+// `halves` thermostat half steps of every active system: kinetic energies (kKeWords
+// per system in ke, zero before and after), factors into scale, velocities scaled.
 void launch_thermostat(const DevArrays& a, int nsys, Thermo* thermo, int halves, unsigned long long* ke, double* scale,
                        cudaStream_t s);
 void launch_pair_stats(const DevArrays& a, int cur, unsigned long long* out2, cudaStream_t s);

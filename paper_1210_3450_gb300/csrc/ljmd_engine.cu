@@ -407,9 +407,9 @@ int Engine::alloc_arrays() {
   CK(cudaMallocHost((void**)&h_rebuild_, sizeof(int32_t) * (4 * ns + 2)));
   CK(cudaMallocHost((void**)&h_obs_, sizeof(double) * 3 * ns));
   CKR(dmalloc(&d_ctl_, 1));
-  // barrier word, maxima and energy limbs; behind them the thermostats
-  CKR(dmalloc(&d_loop_, 1 + 15 * (int64_t)ns + (int64_t)ns * (int64_t)(sizeof(Thermo) / sizeof(unsigned long long))));
-  d_thermo_ = (Thermo*)(d_loop_ + 1 + 15 * (size_t)ns);
+  // barrier word, maxima and energy sums; behind them the thermostats
+  CKR(dmalloc(&d_loop_, 1 + kLoopWords * (int64_t)ns + (int64_t)ns * (int64_t)(sizeof(Thermo) / sizeof(unsigned long long))));
+  d_thermo_ = (Thermo*)(d_loop_ + 1 + kLoopWords * (size_t)ns);
   CKR(dmalloc(&d_reb_count_, ns));
   CK(cudaMemset(d_ctl_, 0, sizeof(GraphCtl)));
   CK(cudaMallocHost((void**)&h_ctl_, sizeof(GraphCtl)));
@@ -1197,7 +1197,7 @@ int Engine::run_loop(int64_t nsteps, bool stored, bool steady, int64_t* done, bo
   *h_ctl_ = c;
   CK(cudaMemcpyAsync(d_ctl_, h_ctl_, sizeof(GraphCtl), cudaMemcpyHostToDevice, s));
   CK(cudaMemsetAsync(d_reb_count_, 0, sizeof(int32_t) * nsys(), s));
-  CK(cudaMemsetAsync(d_loop_, 0, sizeof(unsigned long long) * (1 + 15 * (size_t)nsys()), s));
+  CK(cudaMemsetAsync(d_loop_, 0, sizeof(unsigned long long) * (1 + kLoopWords * (size_t)nsys()), s));
   DevArrays a = arrays();
   a.ctl = d_ctl_;
   LoopArgs g{};
@@ -1404,7 +1404,7 @@ int Engine::step_nvt(int64_t nsteps, const std::vector<double>& dt, const std::v
   CKR(have_states());
   CK(cudaMemcpyAsync(d_thermo_, th.data(), sizeof(Thermo) * (size_t)ns, cudaMemcpyHostToDevice, s));
   unsigned long long* ke = d_loop_ + 1 + 3 * (size_t)ns;
-  CK(cudaMemsetAsync(ke, 0, sizeof(unsigned long long) * 4 * (size_t)ns, s));
+  CK(cudaMemsetAsync(ke, 0, sizeof(unsigned long long) * kKeWords * (size_t)ns, s));
   const int rc = nvt_steps(nsteps, dt, ke, s);
   if (rc == kErrTimeout) return rc;  // the states are lost
   // after an error in a step as well: the thermostats have moved with the particles
@@ -1446,7 +1446,7 @@ int Engine::nvt_steps(int64_t nsteps, const std::vector<double>& dt, unsigned lo
       CKR(launch_step(0.5, 0.0, kStepStoreF, s));
       for (SysHost& h : sys_)
         if (h.active) h.f_valid = true;
-      CK(cudaMemsetAsync(ke, 0, sizeof(unsigned long long) * 4 * (size_t)ns, s));
+      CK(cudaMemsetAsync(ke, 0, sizeof(unsigned long long) * kKeWords * (size_t)ns, s));
       CKR(thermostat(it < nsteps ? 2 : 1));
     }
   }
@@ -1458,7 +1458,7 @@ int Engine::nvt_steps(int64_t nsteps, const std::vector<double>& dt, unsigned lo
   for (; it < nsteps; ++it) {
     CKR(step(1, dt, s));
     // the end of this step and the start of the next are consecutive half steps
-    CK(cudaMemsetAsync(ke, 0, sizeof(unsigned long long) * 4 * (size_t)ns, s));
+    CK(cudaMemsetAsync(ke, 0, sizeof(unsigned long long) * kKeWords * (size_t)ns, s));
     CKR(thermostat(it + 1 < nsteps ? 2 : 1));
   }
   return kOK;

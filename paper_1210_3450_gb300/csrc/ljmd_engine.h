@@ -235,7 +235,7 @@ class Engine {
   int64_t gver_[2] = {-1, -1};
   cudaStream_t cap_[2] = {nullptr, nullptr};
   GraphCtl* d_ctl_ = nullptr;
-  unsigned long long* d_loop_ = nullptr;  // persistent loop: barrier word, 3 maxima and 12 energy limbs per system
+  unsigned long long* d_loop_ = nullptr;  // persistent loop: barrier word, kLoopWords per system
   Thermo* d_thermo_ = nullptr;            // thermostats (nsys) of md_step_nvt
   int loop_lanes_ = 0, loop_stride_ = 0;
   int loop_polls_ = 1 << 21;              // of a grid barrier before it gives up (about a second)

@@ -199,20 +199,6 @@ static __device__ __forceinline__ unsigned long long fix_sqr(unsigned long long 
 // Exact sum of 64-bit non-negative terms in 128 bits.
 struct FixAcc {
   unsigned long long lo = 0ull, hi = 0ull;
-  // Adds an FP64 number >= 0 in units of 2^-64 (bits below the unit are dropped;
-  // 2^63 and more, and what is not finite, count as 2^62).
-  __device__ __forceinline__ void add_fp64(double v) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-    const int sh = (int)((b >> 52) & 0x7FF) - (1075 - 64);
-    const unsigned long long m = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);
-    unsigned long long l, h;
-    if (sh > 74) { l = 0ull; h = 1ull << 62; }
-    else if (sh >= 64) { l = 0ull; h = m << (sh - 64); }
-    else if (sh > 0) { l = m << sh; h = m >> (64 - sh); }
-    else { l = sh > -64 ? m >> -sh : 0ull; h = 0ull; }
-    lo += l;
-    hi += h + (lo < l ? 1ull : 0ull);
-  }
   __device__ __forceinline__ void add(unsigned long long v) {
     lo += v;
     hi += lo < v ? 1ull : 0ull;
@@ -233,6 +219,61 @@ struct FixAcc {
     const unsigned long long r = (m >> 11) + ((m >> 10) & 1ull);  // 53 bits; may round up to 2^53
     const int ex = 1023 + 52 + 11 + 64 - z - unit;
     return __longlong_as_double((long long)(((unsigned long long)(ex - 1) << 52) + r));
+  }
+};
+
+// Exact sum of FP64 squares in 256 bits, units of 2^-160: squares of 2^-108 and more (a
+// velocity component of 5e-17) keep all their bits, and 2^28 of the largest stay in range.
+// Squares of 2^64 and more, and what is not finite, are only kept as the largest of them,
+// which then stands for the sum.
+struct SquareSum {
+  unsigned long long w[4] = {0ull, 0ull, 0ull, 0ull};
+  unsigned long long over = 0ull;
+  static constexpr unsigned long long kOver = (1023ull + 64ull) << 52;  // 2^64
+  __device__ __forceinline__ void add_words(unsigned long long a, unsigned long long b, unsigned long long c,
+                                            unsigned long long d) {
+    asm("add.cc.u64 %0, %0, %4;\n\t"
+        "addc.cc.u64 %1, %1, %5;\n\t"
+        "addc.cc.u64 %2, %2, %6;\n\t"
+        "addc.u64 %3, %3, %7;"
+        : "+l"(w[0]), "+l"(w[1]), "+l"(w[2]), "+l"(w[3])
+        : "l"(a), "l"(b), "l"(c), "l"(d));
+  }
+  __device__ __forceinline__ void add(double v) {  // v: a square
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull;
+    if (b >= kOver) {
+      over = b > over ? b : over;
+      return;
+    }
+    const int sh = (int)(b >> 52) - (1075 - 160);
+    const unsigned long long m = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);
+    const int k = sh >> 6, r = sh & 63;
+    unsigned long long lo = m << r, hi = r ? m >> (64 - r) : 0ull;
+    if (sh < 0) {
+      lo = sh > -64 ? m >> -sh : 0ull;
+      hi = 0ull;
+    }
+    add_words(k <= 0 ? lo : 0ull, k == 1 ? lo : (k == 0 ? hi : 0ull), k == 2 ? lo : (k == 1 ? hi : 0ull),
+              k == 2 ? hi : 0ull);
+  }
+  // Adds the sum of the lane o away (all 32 lanes of the warp call it).
+  __device__ __forceinline__ void join(int o) {
+    unsigned long long y[4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) y[m] = __shfl_xor_sync(0xffffffffu, w[m], o);
+    const unsigned long long v = __shfl_xor_sync(0xffffffffu, over, o);
+    add_words(y[0], y[1], y[2], y[3]);
+    over = v > over ? v : over;
+  }
+  // Half the sum as FP64 (rounded to nearest).
+  __device__ __forceinline__ double half() const {
+    if (over) return 0.5 * __longlong_as_double((long long)over);
+    int k = 3;
+    while (k > 0 && w[k] == 0ull) --k;
+    FixAcc s;
+    s.hi = w[k];
+    s.lo = k > 0 ? w[k - 1] : 0ull;
+    return s.value(161 + 64 - 64 * k);
   }
 };
 

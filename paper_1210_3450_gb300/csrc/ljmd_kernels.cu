@@ -2266,26 +2266,31 @@ __global__ void __launch_bounds__(256) k_obs_final(const int32_t* __restrict__ w
 // ------------------------------------------ Nose-Hoover thermostat (Sec. 4.1)
 
 // The kinetic energy of the thermostat is an exact sum of the squared velocity components
-// (FP64 squares in units of 2^-64, added as integers in four 32-bit limbs), so every way
-// of running the steps, alone or in a batch, gives the same bits whatever the order.
+// (SquareSum; in global memory eight 32-bit limbs and the word of the squares out of
+// range), so every way of running the steps, alone or in a batch, gives the same bits
+// whatever the order.
 namespace {
 
-__device__ __forceinline__ void add_limbs(unsigned long long* ke, const FixAcc& s) {
-  if (s.lo & 0xffffffffull) atomicAdd(ke + 0, s.lo & 0xffffffffull);
-  if (s.lo >> 32) atomicAdd(ke + 1, s.lo >> 32);
-  if (s.hi & 0xffffffffull) atomicAdd(ke + 2, s.hi & 0xffffffffull);
-  if (s.hi >> 32) atomicAdd(ke + 3, s.hi >> 32);
+__device__ __forceinline__ void add_limbs(unsigned long long* ke, const SquareSum& s) {
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    if (s.w[m] & 0xffffffffull) atomicAdd(ke + 2 * m, s.w[m] & 0xffffffffull);
+    if (s.w[m] >> 32) atomicAdd(ke + 2 * m + 1, s.w[m] >> 32);
+  }
+  if (s.over) atomicMax(ke + 8, s.over);
 }
 // Kinetic energy from the limbs.
-__device__ __forceinline__ double limbs_ke(unsigned long long a, unsigned long long b, unsigned long long c,
-                                           unsigned long long d) {
-  b += a >> 32;
-  c += b >> 32;
-  d += c >> 32;
-  FixAcc s;
-  s.lo = (b << 32) | (a & 0xffffffffull);
-  s.hi = (d << 32) | (c & 0xffffffffull);
-  return s.value(65);  // half the sum of the squares
+__device__ __forceinline__ double limbs_ke(const unsigned long long* ke) {
+  SquareSum s;
+  unsigned long long carry = 0ull;
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    const unsigned long long a = __ldcg(ke + 2 * m) + carry, b = __ldcg(ke + 2 * m + 1) + (a >> 32);
+    s.w[m] = (b << 32) | (a & 0xffffffffull);
+    carry = b >> 32;
+  }
+  s.over = __ldcg(ke + 8);
+  return s.half();
 }
 
 // `halves` consecutive thermostat half steps from one kinetic energy: each is
@@ -2312,14 +2317,14 @@ __device__ __forceinline__ double thermo_halves(Thermo& t, double ke, int halves
 __global__ void __launch_bounds__(256) k_ke_limbs(DevArrays a, unsigned long long* ke) {
   const int lane = threadIdx.x & 31;
   const int nw = (int)((gridDim.x * blockDim.x) >> 5);
-  FixAcc s;
+  SquareSum s;
   int last = -1;
   auto flush = [&]() {
     if (last < 0) return;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s.join(o);
-    if (lane == 0) add_limbs(ke + 4 * last, s);
-    s = FixAcc();
+    if (lane == 0) add_limbs(ke + kKeWords * last, s);
+    s = SquareSum();
   };
   // each warp a run of consecutive tiles (few changes of system)
   const int per = (a.ntiles + nw - 1) / nw;
@@ -2336,9 +2341,9 @@ __global__ void __launch_bounds__(256) k_ke_limbs(DevArrays a, unsigned long lon
     const int local = (w - P.t_off) * kTile + lane;
     if (local < P.n) {
       const double4_32a v = a.v[P.p_off + local];
-      s.add_fp64(__dmul_rn(v.x, v.x));
-      s.add_fp64(__dmul_rn(v.y, v.y));
-      s.add_fp64(__dmul_rn(v.z, v.z));
+      s.add(__dmul_rn(v.x, v.x));
+      s.add(__dmul_rn(v.y, v.y));
+      s.add(__dmul_rn(v.z, v.z));
     }
   }
   flush();
@@ -2350,11 +2355,11 @@ __global__ void k_thermostat(DevArrays a, int nsys, Thermo* thermo, int halves, 
   double f = 1.0;
   if (a.params[k].active) {
     Thermo t = thermo[k];
-    f = thermo_halves(t, limbs_ke(ke[4 * k], ke[4 * k + 1], ke[4 * k + 2], ke[4 * k + 3]), halves);
+    f = thermo_halves(t, limbs_ke(ke + kKeWords * k), halves);
     thermo[k] = t;
   }
   scale[k] = f;
-  for (int m = 0; m < 4; ++m) ke[4 * k + m] = 0ull;
+  for (int m = 0; m < kKeWords; ++m) ke[kKeWords * k + m] = 0ull;
 }
 
 // ------------------------------------ persistent step loop of small arenas
@@ -2400,7 +2405,7 @@ struct LoopShared {
   int sys[kLoopWarps];
   double margin[kLoopMaxSys];
   double scale[kLoopMaxSys];
-  FixAcc ke[kLoopWarps];
+  SquareSum ke[kLoopWarps];
   int need[kLoopMaxSys];
   int ws[kScanBlock / 32];
   int flag;  // barrier: 0 gave up
@@ -2676,10 +2681,10 @@ __global__ void __launch_bounds__(kLoopBlock, T == 4 ? (kFP32 ? 4 : 3) : (kFP32 
   // False if the barrier gave up.
   int turn = 0;
   [[maybe_unused]] auto thermostat = [&](int halves) -> bool {
-    if (blockIdx.x == 0 && (int)threadIdx.x < 4 * g.nsys)  // the next turn's sums: their last readers passed a barrier
-      g.ke[((turn + 1) % 3) * 4 * g.nsys + threadIdx.x] = 0ull;
-    FixAcc s;
-    if (comp) s.add_fp64(__dmul_rn(v, v));
+    if (blockIdx.x == 0)  // the next turn's sums: their last readers passed a barrier
+      for (int m = threadIdx.x; m < kKeWords * g.nsys; m += kLoopBlock) g.ke[((turn + 1) % 3) * kKeWords * g.nsys + m] = 0ull;
+    SquareSum s;
+    if (comp) s.add(__dmul_rn(v, v));
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s.join(o);
     if (lane == 0) {
@@ -2689,20 +2694,20 @@ __global__ void __launch_bounds__(kLoopBlock, T == 4 ? (kFP32 ? 4 : 3) : (kFP32 
     __syncthreads();
     if (wv == 0) {
       const int k = sh.sys[lane & (kLoopWarps - 1)];
-      FixAcc m = sh.ke[lane & (kLoopWarps - 1)];
-      unsigned long long* ke = g.ke + (turn % 3) * 4 * g.nsys;
+      SquareSum m = sh.ke[lane & (kLoopWarps - 1)];
+      unsigned long long* ke = g.ke + (turn % 3) * kKeWords * g.nsys;
       if (__all_sync(kFull, k == sh.sys[0])) {
 #pragma unroll
         for (int o = kLoopWarps / 2; o > 0; o >>= 1) m.join(o);
-        if (lane == 0 && k >= 0) add_limbs(ke + 4 * k, m);
+        if (lane == 0 && k >= 0) add_limbs(ke + kKeWords * k, m);
       } else if (lane < kLoopWarps && k >= 0) {
-        add_limbs(ke + 4 * k, m);
+        add_limbs(ke + kKeWords * k, m);
       }
     }
     if (!grid_barrier(g, arrivals, sh, a.ctl)) return false;
     if (dactive) {
-      const unsigned long long* ke = g.ke + ((turn % 3) * g.nsys + threadIdx.x) * 4;
-      sh.scale[threadIdx.x] = thermo_halves(thermo, limbs_ke(__ldcg(ke), __ldcg(ke + 1), __ldcg(ke + 2), __ldcg(ke + 3)), halves);
+      const unsigned long long* ke = g.ke + ((turn % 3) * g.nsys + threadIdx.x) * kKeWords;
+      sh.scale[threadIdx.x] = thermo_halves(thermo, limbs_ke(ke), halves);
     }
     ++turn;
     __syncthreads();

@@ -76,3 +76,30 @@ def test_thermostat_after_an_error(ljmd):
             assert rc == ljmd.MD_ERR_NONFINITE
             assert b"non-finite" in ljmd.load_library().md_last_error()
             assert abs(z.value - zeta) < 1e-12 and abs(e.value - eta) < 1e-12
+
+
+@pytest.mark.parametrize("graph", [0, 1])
+@pytest.mark.parametrize("precision", [0, 1], ids=["fp64", "fp32"])
+@pytest.mark.parametrize("speed", [1e-12, 1e-9, 1e-6, 1e-3, 1.0, 1e4, 1e9])
+def test_kinetic_energy_at_any_scale(ljmd, speed, precision, graph):
+    """Particles out of each other's reach: the thermostat variables after one step are
+    those of the kinetic energy alone, whatever its scale. Their FP64 chain of a few
+    operations and the sum of 375 squares leave a relative 1e-13."""
+    n, box = 125, 60.0
+    k = np.arange(n)
+    x = np.stack([k % 5, k // 5 % 5, k // 25], 1) * 12.0 + 1.0
+    v = speed * li.maxwell_boltzmann(n, 1.0, 807)
+    dt, Q = min(0.005, 1e-3 / speed), n * speed ** 2 * 0.01
+    ke, zeta, eta = 0.5 * (v * v).sum(), 0.0, 0.0
+    for _ in range(2):
+        zeta += 0.25 * dt * 2.0 * ke / Q
+        eta += 0.5 * dt * zeta
+        ke *= np.exp(-0.5 * dt * zeta) ** 2
+        zeta += 0.25 * dt * 2.0 * ke / Q
+    with ljmd.LJSystem(box, n, 2.5, 0.3, precision) as s:
+        s.set_tuning(graph=graph)
+        s.set_state(x, v)
+        z, e = s.step_nvt(1, dt, 0.0, Q)
+        vs = s.get_state()[1]
+    assert abs(z - zeta) <= 1e-13 * zeta and abs(e - eta) <= 1e-13 * eta
+    assert abs(0.5 * (vs * vs).sum() - ke) <= 1e-13 * ke
