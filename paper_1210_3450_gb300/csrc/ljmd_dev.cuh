@@ -155,7 +155,8 @@ struct DevArrays {
   double4_32a* f;         // stored forces (double); half list: the own-list sums of the step
   double4_32a* facc;      // half list: forces added by the partners' threads (atomics), zeroed on use
   int4* xq[2];        // fixed-point shadow positions (uint32 per axis, wraps at L)
-  longlong4_32a* xl[2];  // FP64 form: positions in fixed-point pair units (2^-60, modulo 2^64)
+  longlong4_32a* xl[2];  // FP64 form with full lists (else NULL): positions in fixed-point pair units (2^-60,
+                         // modulo 2^64), in the memory of facc and vtmp
   int32_t* id;        // caller index of each slot, -1 for padding
   int32_t* cell;      // cell of each slot (valid after binning)
   int32_t* ncnt;      // list length of each slot

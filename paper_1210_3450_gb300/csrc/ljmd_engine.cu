@@ -288,7 +288,6 @@ int footprint(const SysSpec& s, SysFootprint* f, SysHost* h) {
 
 void Engine::free_all() {
   for (int b = 0; b < 2; ++b) { dfree(d_.x[b]); dfree(d_.xq[b]); }
-  dfree(d_.xl[0]);
   dfree(d_.v); dfree(d_.xref); dfree(d_.xqref); dfree(d_.f); dfree(d_.facc); dfree(d_.id); dfree(d_.cell); dfree(d_.ncnt);
   dfree(d_.nbr); dfree(d_.tile_obs); dfree(d_.skey); dfree(d_.xf); dfree(d_.vtmp); dfree(d_.idtmp);
   dfree(d_.celltmp); dfree(d_.perm); dfree(d_.sid); dfree(d_.ccount); dfree(d_.cstart); dfree(d_.chunk_sum);
@@ -298,7 +297,6 @@ void Engine::free_all() {
   drop_graphs();
   dfree(d_ctl_); dfree(d_loop_); dfree(d_reb_count_); hfree(h_ctl_); hfree(h_reb_count_);
   d_ = DevArrays{};
-  fixed_off_ = false;
   stage_n_ = 0;
 }
 
@@ -418,44 +416,11 @@ int Engine::alloc_arrays() {
   return upload_params();
 }
 
-// The FP64 form's positions in pair units, allocated for the first lists of that form
-// (every slot is written by a rebuild before it is read). Without memory for them its
-// pairs take the FP64 pipe until the form changes.
-void Engine::ensure_fixed() {
-  if (precision_ != 0 || half_ || d_.xl[0] || fixed_off_) return;
-  ++struct_ver_;
-  if (dmalloc(&d_.xl[0], 2 * caps_.slots) != kOK) {
-    set_error("");
-    fixed_off_ = true;
-    return;
-  }
-  d_.xl[1] = d_.xl[0] + caps_.slots;
-}
-
-void Engine::drop_fixed(bool off) {
-  dfree(d_.xl[0]);
-  d_.xl[1] = nullptr;
-  fixed_off_ = off;
-  ++struct_ver_;
-}
-
-// An allocation that the positions in pair units give way to.
-template <class T>
-int Engine::dmalloc_first(T** p, int64_t count) {
-  int r = dmalloc(p, count);
-  if (r == kErrOOM && d_.xl[0]) {
-    drop_fixed(true);
-    r = dmalloc(p, count);
-    if (r == kOK) set_error("");
-  }
-  return r;
-}
-
 int Engine::stage(int64_t n, double** out) {
   if (n > stage_n_) {
     dfree(d_stage_);
     stage_n_ = 0;
-    CKR(dmalloc_first(&d_stage_, 6 * n));
+    CKR(dmalloc(&d_stage_, 6 * n));
     stage_n_ = n;
   }
   *out = d_stage_;
@@ -476,7 +441,7 @@ int Engine::grow_list_arena(int64_t min_extra_units) {
   const int64_t old_units = list_alloc_.cap();
   const int64_t new_units = std::max(old_units + old_units / 2, old_units + min_extra_units);
   uint32_t* nb = nullptr;
-  CKR(dmalloc_first(&nb, new_units * 4 * kTile));
+  CKR(dmalloc(&nb, new_units * 4 * kTile));
   CK(cudaMemcpy(nb, d_.nbr, sizeof(uint32_t) * old_units * 4 * kTile, cudaMemcpyDeviceToDevice));
   dfree(d_.nbr);
   d_.nbr = nb;
@@ -664,7 +629,15 @@ int Engine::upload_order() {
 
 DevArrays Engine::arrays() const {
   DevArrays a = d_;
-  if (precision_ != 0 || half_) a.xl[0] = a.xl[1] = nullptr;  // not kept up by the other forms
+  // Positions in pair units, kept up by the FP64 form with full lists only, in memory that
+  // this form has no other use for: the half list's scattered forces, and the gathered
+  // velocities of a rebuild, which copies each slot's velocity back before it writes the
+  // slot's position there. Their own 64 bytes per slot went past the memory that an
+  // arena's capacities promise, and made the arithmetic depend on what was free.
+  if (precision_ == 0 && !half_) {
+    a.xl[0] = reinterpret_cast<longlong4_32a*>(d_.facc);
+    a.xl[1] = reinterpret_cast<longlong4_32a*>(d_.vtmp);
+  }
   a.params = d_params_;
   a.status = d_status_;
   a.disp2 = d_disp2_;
@@ -687,8 +660,6 @@ int Engine::set_precision(int mode) {
   if (mode != precision_) {
     precision_ = mode;
     ++struct_ver_;
-    drop_fixed(false);  // every list is rebuilt before the next use
-    CKR(upload_params());
     for (SysHost& h : sys_) {
       h.f_valid = false;
       if (h.has_state) h.force_rebuild = true;  // refresh the fixed-point shadow
@@ -715,7 +686,11 @@ int Engine::set_list_kind(int kind) {
   if ((kind == 1) != half_) {
     half_ = kind == 1;
     ++struct_ver_;
-    drop_fixed(false);  // every list is rebuilt before the next use
+    if (half_) {  // the scattered forces start from zero (positions in pair units were there)
+      CK(cudaDeviceSynchronize());
+      CK(cudaMemset(d_.facc, 0, sizeof(double4_32a) * caps_.slots));
+      CK(cudaDeviceSynchronize());
+    }
     for (SysHost& h : sys_) {
       h.f_valid = false;
       if (h.has_state) h.force_rebuild = true;
@@ -741,8 +716,9 @@ int Engine::set_active(int k, bool on) {
                     cudaMemcpyDeviceToDevice));
       CK(cudaMemcpy(d_.xq[cur_] + h.p_off, d_.xq[h.park] + h.p_off, sizeof(int4) * nslot,
                     cudaMemcpyDeviceToDevice));
-      if (d_.xl[0])
-        CK(cudaMemcpy(d_.xl[cur_] + h.p_off, d_.xl[h.park] + h.p_off, sizeof(longlong4_32a) * nslot,
+      const DevArrays a = arrays();
+      if (a.xl[0])
+        CK(cudaMemcpy(a.xl[cur_] + h.p_off, a.xl[h.park] + h.p_off, sizeof(longlong4_32a) * nslot,
                       cudaMemcpyDeviceToDevice));
     }
     h.park = -1;
@@ -803,7 +779,6 @@ int Engine::read_checks(cudaStream_t s) {
 // Full rebuild (bin, stable counting sort, gather, list) of the given systems.
 int Engine::rebuild(std::vector<int> which, cudaStream_t s) {
   if (which.empty()) return kOK;
-  ensure_fixed();
   std::sort(which.begin(), which.end(),
             [&](int p, int q) { return order_rank_[(size_t)p] < order_rank_[(size_t)q]; });
   for (int attempt = 0; attempt < 4; ++attempt) {
@@ -1168,7 +1143,6 @@ int Engine::lose_states(cudaStream_t s) {
 // and for the FP64 form the fixed-point range of every system, for all its listed pairs
 // (the loop does not test them on the shadows first).
 int Engine::loop_plan() {
-  ensure_fixed();
   if (half_ || precision_ > 1 || nsys() > kLoopMaxSys) return 0;
   // A list's capacity can grow without a change of struct_ver_ (within the arena's free
   // words), so the plan is made for both.
@@ -1180,7 +1154,7 @@ int Engine::loop_plan() {
   loop_kmax_ = kmax;
   loop_lanes_ = 0;
   if (precision_ == 0) {
-    if (!d_.xl[0] || kmax > kFixMaxList) return 0;
+    if (kmax > kFixMaxList) return 0;
     for (const SysHost& h : sys_)
       if (h.used && (h.spec.rc > kFixMaxRc || fix_wide(h.spec.rc, h.spec.skin))) return 0;
   }

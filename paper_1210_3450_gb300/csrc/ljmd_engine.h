@@ -166,10 +166,6 @@ class Engine {
 
  private:
   int alloc_arrays();
-  void ensure_fixed();
-  void drop_fixed(bool off);
-  template <class T>
-  int dmalloc_first(T** p, int64_t count);
   void free_all();
   int upload_params(int only = -1);
   int upload_order();
@@ -249,7 +245,6 @@ class Engine {
   int precision_ = 0;
   int rule_ = 0;
   bool half_ = false;
-  bool fixed_off_ = false;  // no memory for the positions in pair units
   int cur_ = 0;
   ArenaCaps caps_{0, 0, 0, 0};
   bool list_growable_ = false;  // exact-size arenas grow their list storage on demand

@@ -430,9 +430,12 @@ __device__ __forceinline__ longlong4_32a fix4(const double4_32a& x) {
 __device__ __forceinline__ void copy_back_slot(const DevArrays& a, int cur, int64_t s) {
   const double4_32a x = a.xref[s];
   a.x[cur][s] = x;
-  if (a.xl[0]) a.xl[cur][s] = fix4(x);
   a.v[s] = a.vtmp[s];
   a.id[s] = a.idtmp[s];
+  if (a.xl[0]) {
+    asm volatile("" ::: "memory");  // xl[1] is vtmp's memory: not before the load above
+    a.xl[cur][s] = fix4(x);
+  }
   a.cell[s] = a.celltmp[s];
 }
 
@@ -1810,7 +1813,7 @@ struct PairForce {
                                        double* slow_, int stride_)
       : a(a_), t(t_), P(P_), cur(cur_), slow(slow_), stride(stride_) {
     slow[0] = slow[stride] = slow[2 * stride] = 0.0;
-    fixed = MODE == 0 && a.xl[0] && P.fixed && cnt <= kFixMaxList;
+    fixed = MODE == 0 && P.fixed && cnt <= kFixMaxList;
     qi = fixed && t.act ? a.xl[cur][t.s] : longlong4_32a{0, 0, 0, 0};
     qi.x -= kFixBias; qi.y -= kFixBias; qi.z -= kFixBias;  // separations come biased for fix_split
   }
