@@ -268,12 +268,18 @@ struct SquareSum {
   // Half the sum as FP64 (rounded to nearest).
   __device__ __forceinline__ double half() const {
     if (over) return 0.5 * __longlong_as_double((long long)over);
-    int k = 3;
-    while (k > 0 && w[k] == 0ull) --k;
-    FixAcc s;
-    s.hi = w[k];
-    s.lo = k > 0 ? w[k - 1] : 0ull;
-    return s.value(161 + 64 - 64 * k);
+    FixAcc s;  // the top word that is not zero, and the next
+    s.hi = w[3];
+    s.lo = w[2];
+    int unit = 161 - 128;
+#pragma unroll
+    for (int k = 2; k >= 0; --k) {  // (no index known only at run time: the words stay in registers)
+      if (s.hi != 0ull) break;
+      s.hi = w[k];
+      s.lo = k > 0 ? w[k - 1] : 0ull;
+      unit += 64;
+    }
+    return s.value(unit);
   }
 };
 
