@@ -35,7 +35,7 @@ UNIT = "particle-steps/s"
 # Integer multipliers: one 32 x 32 -> 64-bit warp product per 4 cycles of a scheduler
 # (152 SMs x 4 schedulers x 8 lanes a cycle x 2.07 GHz), in 1e12 products per second.
 INT_PRODUCT_PEAK_T = 10.07
-PAIR_PRODUCTS = 32  # of a pair inside rc in the FP64 form (ljmd_fixed.cuh)
+PAIR_PRODUCTS = 38  # of a pair inside rc in the FP64 form (ljmd_fixed.cuh)
 
 # Compulsory bytes per particle-step of the fused FP32 force + integration kernel
 # (k_step_fp32), by name; the list adds 4 bytes per listed partner.
@@ -349,8 +349,8 @@ def run_ours(args):
             "avg_launch_ms": round(k_ms, 4),
             "avg_launch_ms_source": "CUDA events around each launch (host-driven pass of the same run)"}
     # FP64 step kernel: its pairs run on the integer multipliers (64-bit fixed point).
-    # Per pair inside rc 32 products of 32 x 32 -> 64 bits (or their high halves): 6 for
-    # r^2, 4 for its reciprocal, 10 for the force factor, 12 for the three sums.
+    # Per pair inside rc 38 products of 32 x 32 -> 64 bits (or their high halves): 6 for
+    # r^2, 4 for its reciprocal, 13 for the force factor, 15 for the three sums.
     t64 = r64["timing"]
     k64 = t64["step_ms"] / max(t64["step_launches"], 1)
     lp64 = r64["listed"] / n

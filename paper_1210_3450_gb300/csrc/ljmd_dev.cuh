@@ -57,7 +57,8 @@ struct SysParams {
   double skin;       // list margin (validity rule 2 d_max >= skin)
   long long Lfix;    // L in fixed-point pair units (2^-60, modulo 2^64)
   long long rc2fix;  // rc^2 in units of 2^-56
-  long long c2fix;   // c2 / 3 in units of 2^-56, plus kFixBias
+  long long c2fix;   // c2 / 3 in units of 2^-88, biased (FixC2): high 64 bits ...
+  unsigned c2fix_lo; // ... and low 32
   double disp_thr;   // FP32-force form: threshold of the squared fixed-point displacement
   float rlf;         // rc + skin as float
   float csf;         // cell side L / nc as float

@@ -567,7 +567,9 @@ int Engine::upload_params(int only) {
     P.wide = fix_wide(h.spec.rc, h.spec.skin) ? 1 : 0;
     if (P.fixed) {
       P.rc2fix = (long long)std::llrint(std::ldexp(P.rc2, 56));
-      P.c2fix = (long long)std::llrint(std::ldexp(h.c2 / 3.0, 56)) + kFixBias;
+      const FixC2 c = fix_c2(h.c2, P.rc2);
+      P.c2fix = c.hi;
+      P.c2fix_lo = c.lo;
     }
     P.skin = h.spec.skin;
     {

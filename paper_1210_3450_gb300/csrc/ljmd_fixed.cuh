@@ -6,10 +6,10 @@
 // Here a pair's force factor comes from products of 64-bit fixed-point numbers, each
 // formed from 32 x 32 -> 64-bit multiply-adds of its halves, and the sums are kept as
 // 96-bit integers: additions are exact, so a force does not depend on the order in
-// which its pairs are added. Nothing is rounded more coarsely than in FP64: against
-// 128-bit arithmetic the forces of perturbed lattices at densities 0.3 to 0.9, cutoffs
-// 2.5 to 3.9, err by 2e-16 to 1.5e-15 (rms) where the FP64 pipe's err by 1.2e-15 to
-// 2.4e-14.
+// which its pairs are added. No factor is rounded more coarsely than in FP64, at any
+// distance in the range: against 113-bit arithmetic it errs (rms, relative to its 24 r^-8)
+// by 0.2 to 0.9e-16 beyond r = 1.2 and by up to 3.8e-16 below, where the FP64 pipe's errs by
+// 0.8 to 3.4e-16 and by up to 1.1e-15 (cutoffs 2.5 and 3.99).
 //
 // Formats (value = integer x unit):
 //   position, separation  unit 2^-60, modulo 2^64 (16 length units; a separation
@@ -17,8 +17,8 @@
 //                         and an FP64 position of 2^-8 or more is held exactly)
 //   r^2                   2^-56   (r^2 < 16)
 //   y = 1 / r^2           2^-63   (r^2 >= kFixR2Min = 0.84: y < 1.1905)
-//   y^2, y^3, y^4         2^-62, 2^-61, 2^-60
-//   g / 24                2^-56   (|g / 24| < 4.77)
+//   y^2, y^3, y^4         2^-62, 2^-61, 2^-92 (96 bits: y^4 falls to 2^-16 at r = 4)
+//   g / 24                2^-88   (96 bits; |g / 24| < 4.77)
 //   force sums / 24       2^-84   (96 bits; 468 pairs of the largest force, 4.37,
 //                         reach their range)
 // Pairs closer than sqrt(0.84) and lists longer than kFixMaxList take the FP64 pipe.
@@ -46,6 +46,15 @@ constexpr double kFixMaxSep = 7.9;                              // separations b
 constexpr long long kFixBias = 0x80000000ll;
 struct Fix2 {
   int h, l;
+};
+// The same with a third, signed part 2^-32 below.
+struct Fix3 {
+  int h, l, m;
+};
+// c2 / 3 in units of 2^-88 plus the biases of both lower parts.
+struct FixC2 {
+  long long hi;
+  unsigned lo;
 };
 static __device__ __forceinline__ Fix2 fix_split(long long biased) {
   Fix2 s;
@@ -113,18 +122,21 @@ static __device__ __forceinline__ unsigned long long fix_rcp(unsigned long long 
   return y;
 }
 
-// g / 24 = y^4 (1 - 2 y^3) + c2 / 3 (g: the factor 24 r^-8 - 48 r^-14 + 8 c2) plus
-// kFixBias; c2_3b is c2 / 3 in units of 2^-56 plus kFixBias. With y < 1.1905 the cross
-// terms of y y^2 stay below 2^64.
-static __device__ __forceinline__ long long fix_force_factor(unsigned long long y, long long c2_3b) {
-  long long g;
+// g / 24 = y^4 (1 - 2 y^3) + c2 / 3 (g: the factor 24 r^-8 - 48 r^-14 + 8 c2). With
+// y < 1.1905 the cross terms of y y^2 stay below 2^64; y^2 is rounded (the constant holds
+// the mean of the dropped square of the low half as well), and y^4 and the products keep
+// what lies below the second half, without which pairs beyond r = 1.6 would be rounded
+// more coarsely than in FP64 (5e-15 of 24 r^-8 at 2.4, 4.5e-13 at 3.9). The six products
+// more (three here, one per sum) cost 0.09 ms of a pass over 2,048,000 particles (1.01 ms).
+static __device__ __forceinline__ Fix3 fix_force_factor(unsigned long long y, const FixC2& c2) {
+  Fix3 g;
   asm("{\n\t"
       ".reg .u64 c, p;\n\t"
       ".reg .s64 d, t;\n\t"
       ".reg .u32 y0, y1, a0, a1, b0, b1, c0, c1, z;\n\t"
-      ".reg .s32 wh, wl, qh, ql, d0, d1, sg;\n\t"
-      "mov.b64 {y0, y1}, %1;\n\t"
-      "mul.wide.u32 c, y1, y0;\n\t"            // y^2 (unit 2^-62)
+      ".reg .s32 wh, wl, qh, ql, qm, d0, d1, sg;\n\t"
+      "mov.b64 {y0, y1}, %3;\n\t"
+      "mad.wide.u32 c, y1, y0, 0x6AAAAAAA;\n\t"  // y^2 (unit 2^-62)
       "shr.u64 c, c, 31;\n\t"
       "mad.wide.u32 p, y1, y1, c;\n\t"
       "mov.b64 {a0, a1}, p;\n\t"
@@ -135,26 +147,38 @@ static __device__ __forceinline__ long long fix_force_factor(unsigned long long 
       "mov.b64 c, {c1, z};\n\t"
       "mad.wide.u32 c, y1, a1, c;\n\t"
       "mov.b64 {b0, b1}, c;\n\t"
-      "sub.cc.u32 b0, 0x80000000, b0;\n\t"     // 1 - 2 y^3 (unit 2^-60) plus the bias
+      "sub.cc.u32 b0, 0x80000000, b0;\n\t"     // w = 1 - 2 y^3 (unit 2^-60), split
       "subc.u32 wh, 0x10000000, b1;\n\t"
       "add.u32 wl, b0, 0x80000000;\n\t"
-      "mad.wide.u32 c, a1, a0, 0x4000000000000000;\n\t"  // y^4 (unit 2^-60) plus the bias
+      "mul.hi.u32 c0, a0, a0;\n\t"             // q = y^4 (unit 2^-92), split: half the cross
+      "shr.u32 c0, c0, 1;\n\t"                 // terms (unit 2^-91) with both biases
+      "add.u32 c0, c0, 0x40000000;\n\t"
+      "mov.u32 c1, 0x40000000;\n\t"
+      "mov.b64 c, {c0, c1};\n\t"
+      "mad.wide.u32 c, a1, a0, c;\n\t"
+      "mov.b64 {c0, c1}, c;\n\t"
+      "mad.lo.u32 qm, c0, 2, 0x80000000;\n\t"
       "shr.u64 c, c, 31;\n\t"
       "mad.wide.u32 p, a1, a1, c;\n\t"
       "mov.b64 {b0, qh}, p;\n\t"
       "add.u32 ql, b0, 0x80000000;\n\t"
-      "mad.wide.s32 d, wl, qh, 0x80000000;\n\t"  // the product, rounded to unit 2^-56
+      "mul.wide.s32 d, ql, wl;\n\t"            // q w: the parts of 2^-120,
+      "mad.wide.s32 d, qm, wh, d;\n\t"
+      "shr.s64 d, d, 32;\n\t"
+      "mad.wide.s32 d, wl, qh, d;\n\t"         // 2^-88
       "mad.wide.s32 d, wh, ql, d;\n\t"
-      "mad.wide.s32 t, wh, qh, %2;\n\t"
+      "mad.wide.s32 t, wh, qh, %4;\n\t"        // and 2^-56
       "mov.b64 {d0, d1}, d;\n\t"
       "shr.s32 sg, d1, 31;\n\t"
       "mov.b64 {c0, c1}, t;\n\t"
-      "add.cc.u32 c0, c0, d1;\n\t"
-      "addc.u32 c1, c1, sg;\n\t"
-      "mov.b64 %0, {c0, c1};\n\t"
+      "add.cc.u32 d0, d0, %5;\n\t"
+      "addc.cc.u32 c0, c0, d1;\n\t"
+      "addc.u32 %0, c1, sg;\n\t"
+      "add.u32 %1, c0, 0x80000000;\n\t"
+      "add.u32 %2, d0, 0x80000000;\n\t"
       "}"
-      : "=l"(g)
-      : "l"(y), "l"(c2_3b));
+      : "=r"(g.h), "=r"(g.l), "=r"(g.m)
+      : "l"(y), "l"(c2.hi), "r"(c2.lo));
   return g;
 }
 
@@ -283,19 +307,20 @@ struct SquareSum {
   }
 };
 
-// 96-bit sum of products g d (units 2^-84: g 2^-56, d 2^-60).
+// 96-bit sum of products g d (units 2^-84: g 2^-88, d 2^-60).
 struct FixSum {
   unsigned lo = 0u;   // units of 2^-84
   long long hi = 0;   // units of 2^-52
-  __device__ __forceinline__ void add(const Fix2& g, const Fix2& d) {
+  __device__ __forceinline__ void add(const Fix3& g, const Fix2& d) {
     asm("{\n\t"
-        ".reg .s32 m, sg, c0, c1, h0, h1;\n\t"
+        ".reg .s32 sg, c0, c1, h0, h1;\n\t"
         ".reg .s64 c;\n\t"
-        "mul.hi.s32 m, %3, %5;\n\t"
-        "cvt.s64.s32 c, m;\n\t"
-        "mad.wide.s32 c, %2, %5, c;\n\t"
-        "mad.wide.s32 c, %3, %4, c;\n\t"
-        "mad.wide.s32 %1, %2, %4, %1;\n\t"
+        "mul.wide.s32 c, %3, %6;\n\t"      // 2^-116
+        "mad.wide.s32 c, %4, %5, c;\n\t"
+        "shr.s64 c, c, 32;\n\t"
+        "mad.wide.s32 c, %2, %6, c;\n\t"   // 2^-84
+        "mad.wide.s32 c, %3, %5, c;\n\t"
+        "mad.wide.s32 %1, %2, %5, %1;\n\t" // 2^-52
         "mov.b64 {c0, c1}, c;\n\t"
         "shr.s32 sg, c1, 31;\n\t"
         "mov.b64 {h0, h1}, %1;\n\t"
@@ -305,7 +330,7 @@ struct FixSum {
         "mov.b64 %1, {h0, h1};\n\t"
         "}"
         : "+r"(lo), "+l"(hi)
-        : "r"(g.h), "r"(g.l), "r"(d.h), "r"(d.l));
+        : "r"(g.h), "r"(g.l), "r"(g.m), "r"(d.h), "r"(d.l));
   }
   // Adds the sum of the lane o away (all 32 lanes of the warp call it).
   __device__ __forceinline__ void join(int o) {
@@ -363,17 +388,16 @@ static __device__ __forceinline__ unsigned long long fix_separation2(const longl
 }
 
 // One pair: where r < rc, its force is added to the sums (qi, code, L as above; rc2 in
-// units of 2^-56, c2_3b as for fix_force_factor). Returns true, with
-// nothing added, for a pair closer than the range (the FP64 pipe takes it).
+// units of 2^-56, c2 as for fix_force_factor). Returns true, with nothing added, for a pair closer than the range (the FP64 pipe takes it).
 static __device__ __forceinline__ bool fix_pair(const longlong4_32a& qi, const longlong4_32a& qj, unsigned code,
-                                                long long L, long long rc2, long long c2_3b, FixSum& sx, FixSum& sy,
+                                                long long L, long long rc2, const FixC2& c2, FixSum& sx, FixSum& sy,
                                                 FixSum& sz) {
   Fix2 fx, fy, fz;
   fix_separation(qi, qj, code, L, fx, fy, fz);
   const unsigned long long r2 = fix_r2(fx, fy, fz);
   const bool far = (unsigned)(r2 >> 32) >= kFixR2Min;
   if (far & ((long long)(r2 - (unsigned long long)rc2) < 0)) {
-    const Fix2 g = fix_split(fix_force_factor(fix_rcp(r2), c2_3b));
+    const Fix3 g = fix_force_factor(fix_rcp(r2), c2);
     sx.add(g, fx);
     sy.add(g, fy);
     sz.add(g, fz);
@@ -391,6 +415,23 @@ static inline long long fix_host(double x) {
   const unsigned long long m = (unsigned long long)std::ldexp(std::frexp(x, &e), 53);  // x = m 2^(e - 53)
   const int sh = e - 53 + 60;
   return (long long)(sh >= 64 ? 0ull : sh >= 0 ? m << sh : m >> -sh);
+}
+
+// c2 / 3 for fix_force_factor (host; rounded to nearest). Cutoffs below the range of the
+// pairs, whose c2 may not fit, have no pair that takes it.
+static inline FixC2 fix_c2(double c2, double rc2) {
+  __int128 v = 0;
+  if (rc2 > 0.83) {
+    int e = 0;
+    const long long m = (long long)std::ldexp(std::frexp(c2, &e), 53);  // c2 = m 2^(e - 53)
+    const int sh = e - 53 + 88;
+    if (sh >= 0) {
+      v = (__int128)m * ((__int128)1 << sh) + 1;
+      v = (v - (v < 0 ? (v % 3 + 3) % 3 : v % 3)) / 3;  // floor((m 2^sh + 1) / 3)
+    }
+  }
+  v += (__int128)kFixBias + ((__int128)kFixBias << 32);
+  return FixC2{(long long)(v >> 32), (unsigned)v};
 }
 
 }  // namespace ljmd

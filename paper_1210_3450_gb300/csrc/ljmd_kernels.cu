@@ -1846,7 +1846,7 @@ struct PairForce {
   __device__ __forceinline__ void pair(const longlong4_32a& qj, uint32_t e) {
     const unsigned code = e >> kIdxBits;
     if (MODE == 0 && fixed) {
-      if (fix_pair(qi, qj, code, P.Lfix, P.rc2fix, P.c2fix, sx, sy, sz)) fp64_pair(slot(e), code);
+      if (fix_pair(qi, qj, code, P.Lfix, P.rc2fix, FixC2{P.c2fix, P.c2fix_lo}, sx, sy, sz)) fp64_pair(slot(e), code);
     } else {
       fp64_pair(slot(e), code);
     }
@@ -2503,7 +2503,8 @@ __global__ void __launch_bounds__(kLoopBlock, T == 4 ? (kFP32 ? 4 : 3) : (kFP32 
   Word* list = lists + (size_t)part * g.stride;
   float* ex = ex_all + (size_t)part * loop_ex(T);
   const float qu = P.qunit, rc2f = P.rc2f, c2x8 = 8.0f * P.c2f;
-  const long long rc2x = P.rc2fix, c2x = P.c2fix;
+  const long long rc2x = P.rc2fix;
+  const FixC2 c2x{P.c2fix, P.c2fix_lo};
   const double dt = P.dt, h = P.hdt, qscale = P.qscale;
 
   int cur = g.cur;

@@ -48,7 +48,8 @@ struct NaParams {
   double L, inv_cs, rc2, c2x8;
   int n, nc;
   // fixed-point form (k_na_force_fixed)
-  long long Lfix, rc2fix, c2fix;
+  long long Lfix, rc2fix;
+  FixC2 c2fix;
   float rc2q;  // rc^2 (1 + 1e-5) in units of 2^-56
 };
 
@@ -448,7 +449,7 @@ extern "C" int md_forces_noalloc(const double* x_dev, int64_t N, double box_L, d
   if (p.nc > 1 && rc <= kFixMaxRc && box_L / p.nc < 3.99) {
     p.Lfix = fix_host(box_L);
     p.rc2fix = (long long)std::llrint(std::ldexp(p.rc2, 56));
-    p.c2fix = (long long)std::llrint(std::ldexp(p.c2x8 / 24.0, 56)) + kFixBias;
+    p.c2fix = fix_c2(p.c2x8 / 8.0, p.rc2);
     p.rc2q = (float)(std::ldexp(p.rc2, 56) * (1.0 + 1e-5));
     k_na_rank<true><<<blocks, 256, 0, s>>>(base, p, x_dev);
     // threads per particle: enough to fill the GPU
