@@ -182,50 +182,68 @@ static __device__ __forceinline__ Fix3 fix_force_factor(unsigned long long y, co
   return g;
 }
 
-// y^3 (units 2^-61) and the square of a fraction a < 2^31.4 / 2^32 of its range (units
-// 2^-2u of the high words: y^3 in 2^-61 gives y^6 in 2^-58).
-static __device__ __forceinline__ unsigned long long fix_y3(unsigned long long y) {
-  unsigned long long r;
+// A 96-bit number: 64 bits and the 32 below.
+struct Fix96 {
+  unsigned long long hi;
+  unsigned lo;
+};
+// y^3 in units of 2^-93, and the square of an a < 2^31.4 / 2^32 of its range (a in units of
+// 2^-u: units of 2^(32 - 2 u); y^3's high part in 2^-61 gives y^6 in 2^-90).
+static __device__ __forceinline__ Fix96 fix_y3(unsigned long long y) {
+  Fix96 r;
   asm("{\n\t"
       ".reg .u64 c, p;\n\t"
-      ".reg .u32 y0, y1, a0, a1, c0, c1, z;\n\t"
-      "mov.b64 {y0, y1}, %1;\n\t"
-      "mul.wide.u32 c, y1, y0;\n\t"
+      ".reg .u32 y0, y1, a0, a1, c1, z;\n\t"
+      "mov.b64 {y0, y1}, %2;\n\t"
+      "mad.wide.u32 c, y1, y0, 0x6AAAAAAA;\n\t"  // y^2 (unit 2^-62), rounded as in fix_force_factor
       "shr.u64 c, c, 31;\n\t"
       "mad.wide.u32 p, y1, y1, c;\n\t"
       "mov.b64 {a0, a1}, p;\n\t"
-      "mul.wide.u32 c, y1, a0;\n\t"
-      "mad.wide.u32 c, y0, a1, c;\n\t"
-      "mov.b64 {c0, c1}, c;\n\t"
       "mov.u32 z, 0;\n\t"
+      "mul.hi.u32 c1, y0, a0;\n\t"
+      "mov.b64 c, {c1, z};\n\t"
+      "mad.wide.u32 c, y1, a0, c;\n\t"
+      "mad.wide.u32 c, y0, a1, c;\n\t"
+      "mov.b64 {%1, c1}, c;\n\t"
       "mov.b64 c, {c1, z};\n\t"
       "mad.wide.u32 %0, y1, a1, c;\n\t"
       "}"
-      : "=l"(r)
+      : "=l"(r.hi), "=&r"(r.lo)
       : "l"(y));
   return r;
 }
-static __device__ __forceinline__ unsigned long long fix_sqr(unsigned long long a) {
-  unsigned long long r;
+static __device__ __forceinline__ Fix96 fix_sqr(unsigned long long a) {
+  Fix96 r;
   asm("{\n\t"
       ".reg .u64 c;\n\t"
-      ".reg .u32 a0, a1;\n\t"
-      "mov.b64 {a0, a1}, %1;\n\t"
-      "mul.wide.u32 c, a1, a0;\n\t"
+      ".reg .u32 a0, a1, c0, z;\n\t"
+      "mov.b64 {a0, a1}, %2;\n\t"
+      "mov.u32 z, 0;\n\t"
+      "mul.hi.u32 c0, a0, a0;\n\t"
+      "shr.u32 c0, c0, 1;\n\t"
+      "mov.b64 c, {c0, z};\n\t"
+      "mad.wide.u32 c, a1, a0, c;\n\t"  // half the cross terms
+      "mov.b64 {c0, z}, c;\n\t"
+      "shl.b32 %1, c0, 1;\n\t"
       "shr.u64 c, c, 31;\n\t"
       "mad.wide.u32 %0, a1, a1, c;\n\t"
       "}"
-      : "=l"(r)
+      : "=l"(r.hi), "=&r"(r.lo)
       : "l"(a));
   return r;
 }
 
-// Exact sum of 64-bit non-negative terms in 128 bits.
+// Exact sum of 64- or 96-bit non-negative terms in 128 bits.
 struct FixAcc {
   unsigned long long lo = 0ull, hi = 0ull;
   __device__ __forceinline__ void add(unsigned long long v) {
     lo += v;
     hi += lo < v ? 1ull : 0ull;
+  }
+  __device__ __forceinline__ void add(const Fix96& v) {
+    const unsigned long long l = (v.hi << 32) | v.lo;
+    lo += l;
+    hi += (v.hi >> 32) + (lo < l ? 1ull : 0ull);
   }
   // Adds the sum of the lane o away (all 32 lanes of the warp call it).
   __device__ __forceinline__ void join(int o) {

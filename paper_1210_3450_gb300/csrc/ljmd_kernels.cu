@@ -2096,8 +2096,8 @@ __global__ void __launch_bounds__(kBlock, 7) k_pe_virial(DevArrays a, int cur, i
         const unsigned long long r2 = fix_separation2(qi, qj, code, P.Lfix);
         const bool far = (unsigned)(r2 >> 32) >= kFixR2Min;
         if (far & ((long long)(r2 - (unsigned long long)P.rc2fix) < 0)) {
-          const unsigned long long y3 = fix_y3(fix_rcp(r2));
-          a12.add(fix_sqr(y3));
+          const Fix96 y3 = fix_y3(fix_rcp(r2));
+          a12.add(fix_sqr(y3.hi));
           a6.add(y3);
           ar.add(r2);
           ++nin;
@@ -2122,12 +2122,12 @@ __global__ void __launch_bounds__(kBlock, 7) k_pe_virial(DevArrays a, int cur, i
         s6 += __shfl_xor_sync(kFull, s6, o);
         sr += __shfl_xor_sync(kFull, sr, o);
       }
-      s12 += a12.value(58);
-      s6 += a6.value(61);
+      s12 += a12.value(90);
+      s6 += a6.value(93);
       sr += ar.value(56);
     } else {
-      s12 = a12.value(58);
-      s6 = a6.value(61);
+      s12 = a12.value(90);
+      s6 = a6.value(93);
       sr = ar.value(56);
     }
     const double c2 = P.c2;

@@ -88,3 +88,37 @@ def test_dilute_gas(ljmd):
     with ljmd.LJSystem(box, len(x), 3.9, 0.3) as s:
         s.set_state(x, np.zeros_like(x))
         _check(s.forces(), exact)
+
+
+@pytest.mark.parametrize("precision", [0, 1], ids=["fp64", "fp32"])
+@pytest.mark.parametrize("half", [False, True], ids=["full", "half"])
+def test_energy_and_virial_of_weak_pairs(ljmd, half, precision):
+    """125 pairs near the cutoff. With the errors above, r^-12 within 6 x 3.5 + 3 = 24 u and
+    r^-6 within 12.5 u; the sums, their products with the coefficients (8 roundings in c2
+    and c0) and the final sums 3 more."""
+    from paper_1210_3450_gb300.ljmd import MD_LIST_HALF
+    rc, box, m = 3.99, 50.0, 5
+    x = _dimers(rc, box, m)
+    x[125:] = x[:125] + (x[125:] - x[:125]) * (np.linspace(3.5, 3.989, 125) / np.linspace(0.9, rc, 125))[:, None]
+    rq = Q(rc) ** 2
+    c2, c0 = 6 / rq ** 7 - 3 / rq ** 4, 4 / rq ** 3 - 7 / rq ** 6
+    d = x[None, :, :] - x[:, None, :]
+    k = np.round(d / box)
+    near = np.argwhere(np.triu(((d - box * k) ** 2).sum(2) < rc * rc * (1 + 1e-9), 1))
+    pe, w, bound = Q(0), Q(0), np.zeros(2)
+    for i, j in near.tolist():
+        rr = sum((Q(b) - Q(a) - int(q) * Q(box)) ** 2 for a, b, q in zip(x[i].tolist(), x[j].tolist(), k[i, j]))
+        if rr < rq:
+            s = 1 / rr ** 3
+            pe += 4 * (s * s - s) + 4 * (c2 * rr + c0)
+            w += 48 * s * s - 24 * s - 8 * c2 * rr
+            s, k2, k0 = float(s), abs(float(c2 * rr)), abs(float(c0))
+            bound += U * np.array([4 * (27 * s * s + 15.5 * s + 11 * k2 + 11 * k0), 48 * 27 * s * s + 24 * 15.5 * s + 88 * k2])
+    assert len(near) >= 125
+    with ljmd.LJSystem(box, len(x), rc, 0.3, precision) as s:
+        if half:
+            s.set_pair_list(MD_LIST_HALF)
+        s.set_state(x, np.zeros_like(x))
+        o = s.observables()
+    assert abs(float(Q(o["pe"]) - pe)) <= bound[0]
+    assert abs(float(Q(o["virial"]) - w)) <= bound[1]
