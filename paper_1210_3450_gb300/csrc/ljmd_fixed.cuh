@@ -8,8 +8,8 @@
 // 96-bit integers: additions are exact, so a force does not depend on the order in
 // which its pairs are added. No factor is rounded more coarsely than in FP64, at any
 // distance in the range: against 113-bit arithmetic it errs (rms, relative to its 24 r^-8)
-// by 0.2 to 0.9e-16 beyond r = 1.2 and by up to 3.8e-16 below, where the FP64 pipe's errs by
-// 0.8 to 3.4e-16 and by up to 1.1e-15 (cutoffs 2.5 and 3.99).
+// by 0.06 to 0.8e-16 beyond r = 1.2 and by up to 1.3e-16 below, where the FP64 pipe's errs by
+// 0.8 to 3.4e-16 and by up to 1.1e-15 (cutoffs 2.5 and 3.99), with a mean below 2e-17.
 //
 // Formats (value = integer x unit):
 //   position, separation  unit 2^-60, modulo 2^64 (16 length units; a separation
@@ -78,11 +78,13 @@ static __device__ __forceinline__ long long to_fix(double x) {
 // multiplier for 4 cycles, four times a float one, and is what bounds the pair).
 
 // r^2 of a separation (units 2^-56; the products of two low halves are below the unit).
+// The constant is the mean of what is cut off, which with that of fix_rcp would leave every
+// 1 / r^2 too large by 2e-17, and a virial of many pairs by what single ones average out.
 static __device__ __forceinline__ unsigned long long fix_r2(const Fix2& x, const Fix2& y, const Fix2& z) {
   unsigned long long r;
   asm("{\n\t"
       ".reg .s64 s;\n\t"
-      "mul.wide.s32 s, %1, %2;\n\t"
+      "mad.wide.s32 s, %1, %2, 0x60000000;\n\t"
       "mad.wide.s32 s, %3, %4, s;\n\t"
       "mad.wide.s32 s, %5, %6, s;\n\t"
       "shr.s64 s, s, 31;\n\t"
@@ -106,7 +108,8 @@ static __device__ __forceinline__ unsigned long long fix_rcp(unsigned long long 
   const unsigned y0 = __float2uint_rn(yf * 4503599627370496.0f);            // 2^52: unit 2^-28
   const int e0 = (int)(rh * y0 + __umulhi(rl, y0));                         // unit 2^-52
   const unsigned y1 = (y0 << 3) - (unsigned)(__mulhi((int)y0, e0) >> 17);   // unit 2^-31
-  const int e1 = (int)(0u - (rh * y1 + __umulhi(rl, y1)));                  // unit 2^-55
+  const unsigned ry = (unsigned)(((unsigned long long)rl * y1 + 0x80000000ull) >> 32);
+  const int e1 = (int)(0u - (rh * y1 + ry));                                // unit 2^-55
   unsigned long long y;                                                     // y1 + y1 e1
   asm("{\n\t"
       ".reg .s64 c;\n\t"

@@ -122,3 +122,30 @@ def test_energy_and_virial_of_weak_pairs(ljmd, half, precision):
         o = s.observables()
     assert abs(float(Q(o["pe"]) - pe)) <= bound[0]
     assert abs(float(Q(o["virial"]) - w)) <= bound[1]
+
+
+def test_virial_of_many_pairs_has_no_bias(ljmd):
+    """The virial of 64,000 close pairs against integers of 200 bits: independent rounding
+    errors of the pairs, each of the worst case above, add up to less than 4 times the
+    square root of their number (1.6 % of the sum of the worst cases)."""
+    m, box, rc = 40, 240.0, 2.5
+    g = np.random.Generator(np.random.PCG64(23))
+    k = np.arange(m ** 3)
+    c = np.stack([k % m, k // m % m, k // m ** 2], 1) * 6.0 + 1.5 + g.uniform(0, 0.5, (m ** 3, 3))
+    u = g.standard_normal((m ** 3, 3))
+    u /= np.linalg.norm(u, axis=1, keepdims=True)
+    x = np.concatenate([c, c + u * g.uniform(1.0, 1.2, m ** 3)[:, None]])
+    one = 1 << 60  # positions of 2^-8 and more are whole numbers of 2^-60
+    q = np.array([[int(v * 2.0 ** 45) << 15 if v >= 128 else int(v * one) for v in p] for p in x.tolist()], dtype=object)
+    d = q[m ** 3:] - q[:m ** 3]
+    rr = (d * d).sum(1)                                      # 2^-120
+    y = np.array([(1 << 320) // v for v in rr.tolist()], dtype=object)  # 2^-200
+    s = np.array([v * v * v >> 400 for v in y.tolist()], dtype=object)  # 2^-200
+    s6, s12 = sum(s.tolist()), sum(v * v >> 200 for v in s.tolist())
+    rq = Q(rc) ** 2
+    w = Q(48 * s12 - 24 * s6, 1 << 200) - 8 * (6 / rq ** 7 - 3 / rq ** 4) * Q(sum(rr.tolist()), 1 << 120)
+    worst = U * (48 * 27 * float(Q(s12, 1 << 200)) + 24 * 15.5 * float(Q(s6, 1 << 200)))
+    with ljmd.LJSystem(box, len(x), rc, 0.3) as h:
+        h.set_state(x, np.zeros_like(x))
+        got = h.observables()["virial"]
+    assert abs(float(Q(got) - w)) <= 4.0 / m ** 1.5 * worst
