@@ -50,7 +50,7 @@ struct NaParams {
   // fixed-point form (k_na_force_fixed)
   long long Lfix, rc2fix;
   FixC2 c2fix;
-  float rc2q;  // rc^2 (1 + 1e-5) in units of 2^-56
+  float rc2q;  // (rc + 2^-24)^2 (1 + 1e-5) in units of 2^-56
 };
 
 struct NaScratch {
@@ -223,7 +223,7 @@ __global__ void k_na_force(unsigned char* base, NaParams p, const double* __rest
 // FP64 and ran the force body for whichever lane was inside: 1,150 us at 65,536
 // particles, 600 us at 500 (two blocks of threads). Here the particles are taken in cell
 // order, the candidates of a row of cells are tested on the high words of their
-// positions (unit 2^-28) in float against rc^2 (1 + 1e-5), and each thread queues its
+// positions (unit 2^-28) in float against rc^2 and a margin, and each thread queues its
 // maybe-inside ones and works them off behind the tests. The sums are exact integers,
 // the pairs closer than the fixed-point range are added in a fixed order.
 constexpr int kNaBlock = 128;
@@ -450,7 +450,10 @@ extern "C" int md_forces_noalloc(const double* x_dev, int64_t N, double box_L, d
     p.Lfix = fix_host(box_L);
     p.rc2fix = (long long)std::llrint(std::ldexp(p.rc2, 56));
     p.c2fix = fix_c2(p.c2x8 / 8.0, p.rc2);
-    p.rc2q = (float)(std::ldexp(p.rc2, 56) * (1.0 + 1e-5));
+    // the high words' separations err by less than 3 units of 2^-28 per axis (2e-8 in all),
+    // which counts for cutoffs below 0.004; their float r^2 by a few parts in 1e7
+    const double rq = rc + 5.9604644775390625e-08;
+    p.rc2q = (float)(std::ldexp(rq * rq, 56) * (1.0 + 1e-5));
     k_na_rank<true><<<blocks, 256, 0, s>>>(base, p, x_dev);
     // threads per particle: enough to fill the GPU
     if (N <= 2432) launch_na_force_fixed<32>(base, p, x_dev, f_dev, s);

@@ -44,3 +44,26 @@ def test_position_not_finite(ljmd, oracle, value):
     f = _forces(ljmd, x, box, 2.5)
     assert np.isfinite(np.delete(f, 7, 0)).all()
     assert np.abs(np.delete(f, 7, 0) - ref).max() <= 1e-12 * np.sqrt((ref ** 2).sum(1).mean())
+
+
+@pytest.mark.parametrize("rc", [1e-2, 1e-4, 1e-6, 1e-7, 1e-9])
+def test_short_cutoffs(ljmd, rc):
+    """Pairs at 0.3 to 0.999 of cutoffs near and below the resolution of the candidate test:
+    each force within 1e-12 of its terms in numpy's FP64 (a few tens of roundings)."""
+    m = 6
+    g = np.random.Generator(np.random.PCG64(41))
+    k = np.arange(m ** 3)
+    c = np.stack([k % m, k // m % m, k // m ** 2], 1) / m + 0.05 + g.uniform(0, 0.05, (m ** 3, 3))
+    u = g.standard_normal((m ** 3, 3))
+    u /= np.linalg.norm(u, axis=1, keepdims=True)
+    x = np.concatenate([c, c + u * (rc * np.linspace(0.3, 0.999, m ** 3))[:, None]])
+    d = x[m ** 3:] - x[:m ** 3]
+    y = 1.0 / (d * d).sum(1)
+    yc = rc ** -2.0
+    inside = y > yc
+    assert inside.sum() > 0.9 * m ** 3
+    f = ((24 * y ** 4 - 48 * y ** 7 + 8 * (6 * yc ** 7 - 3 * yc ** 4)) * inside)[:, None] * d
+    size = (24 * y ** 4 + 48 * y ** 7 + 8 * (6 * yc ** 7 + 3 * yc ** 4)) / np.sqrt(y)
+    got = _forces(ljmd, x, 1.0, rc)
+    for a, b in ((got[:m ** 3], f), (got[m ** 3:], -f)):
+        assert (np.abs(a - b).max(1) <= 1e-12 * size).all()
