@@ -1300,7 +1300,8 @@ __device__ __forceinline__ int build_span(const DevArrays& a, int cur, int sys, 
             code = (dx > hl ? 2u : (dx < -hl ? 1u : 0u)) | (dy > hl ? 8u : (dy < -hl ? 4u : 0u)) |
                    (dz > hl ? 32u : (dz < -hl ? 16u : 0u));
             in = true;
-            if (!(r2 < lo2q) || close < 1e-4f * hl) {  // the exact FP64 test
+            // the exact FP64 test (also for a position that is not finite, whose shadow is 0)
+            if (!(r2 < lo2q) || close < 1e-4f * hl || !(dx + dy + dz < 1e30f)) {
               const double4_32a xi = xs[i], xj = xs[j];
               const unsigned r = exact_inside(xi.x, xi.y, xi.z, xj.x, xj.y, xj.z, 0xffu, Pp->L, Pp->rl2);
               in = (r & 0x100u) != 0u;

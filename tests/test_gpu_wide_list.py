@@ -31,3 +31,26 @@ def test_same_list_words(n, rho, rc, half):
             got.append(s.get_list())
     np.testing.assert_array_equal(got[0][0], got[1][0])
     np.testing.assert_array_equal(got[0][1], got[1][1])
+
+
+@pytest.mark.parametrize("value", [np.nan, np.inf])
+@pytest.mark.parametrize("precision", [0, 1], ids=["fp64", "fp32"])
+def test_position_not_finite_in_one_cell(precision, value):
+    """A one-cell box in which a position is not finite: the particle has no partners, as in
+    the other builds, and the other forces are those without it."""
+    from paper_1210_3450_gb300 import LJSystem
+    n = 60
+    x, box = li.perturbed_fcc(n, 0.3, 0.05, 5)
+    x = np.mod(x - x[3] + 0.4, box)  # a partner in reach of the origin
+    x[7, 1] = value
+    got = []
+    for keep in (np.arange(n), np.delete(np.arange(n), 7)):
+        with LJSystem(box, len(keep), 1.9, 0.3, precision) as s:
+            s.set_state(x[keep], np.zeros((len(keep), 3)))
+            start, partners = s.get_list()
+            got.append(s.forces())
+        if len(keep) == n:
+            assert start[8] == start[7] and not (partners == 7).any()
+    assert box < 3 * 2.2
+    rms = np.sqrt((got[1] ** 2).sum(1).mean())
+    assert np.abs(np.delete(got[0], 7, 0) - got[1]).max() <= (1e-12 if precision == 0 else 1e-5) * rms
