@@ -337,6 +337,7 @@ int Engine::init_arena(const ArenaCaps& caps, int precision) {
   h_tile_sys_.assign((size_t)(caps_.slots / kTile), -1);
   ntiles_ = 0;
   cur_ = 0;
+  n_fixed_ = 0;
   return alloc_arrays();
 }
 
@@ -489,6 +490,7 @@ int Engine::add_system(const SysSpec& s, int* id) {
   h.c_off = c0;
   h.l_off = l0 * 4 * kTile;
   sys_[k] = h;
+  n_fixed_ += s.rc <= kFixMaxRc ? 1 : 0;
   // cell counters of the new range must start at zero
   CK(cudaMemset(d_.ccount + h.c_off, 0, sizeof(int32_t) * (h.ncell + 1)));
   CKR(upload_tiles(k, k));
@@ -505,6 +507,7 @@ int Engine::remove_system(int k) {
   slot_alloc_.release(h.t_off, h.ntiles);
   cell_alloc_.release(h.c_off, h.ncell + 1);
   list_alloc_.release(h.l_off / (4 * kTile), (int64_t)h.ntiles * h.kmax / 4);
+  n_fixed_ -= h.spec.rc <= kFixMaxRc ? 1 : 0;
   h = SysHost{};
   update_extent();
   return upload_params(k);
@@ -631,12 +634,13 @@ int Engine::upload_order() {
 
 DevArrays Engine::arrays() const {
   DevArrays a = d_;
-  // Positions in pair units, kept up by the FP64 form with full lists only, in memory that
+  // Positions in pair units, kept up by the FP64 form with full lists only (and systems in
+  // their range), in memory that
   // this form has no other use for: the half list's scattered forces, and the gathered
   // velocities of a rebuild, which copies each slot's velocity back before it writes the
   // slot's position there. Their own 64 bytes per slot went past the memory that an
   // arena's capacities promise, and made the arithmetic depend on what was free.
-  if (precision_ == 0 && !half_) {
+  if (precision_ == 0 && !half_ && n_fixed_ > 0) {
     a.xl[0] = reinterpret_cast<longlong4_32a*>(d_.facc);
     a.xl[1] = reinterpret_cast<longlong4_32a*>(d_.vtmp);
   }

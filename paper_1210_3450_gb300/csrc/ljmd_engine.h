@@ -245,6 +245,7 @@ class Engine {
   int precision_ = 0;
   int rule_ = 0;
   bool half_ = false;
+  int n_fixed_ = 0;  // systems in the range of the fixed-point pairs
   int cur_ = 0;
   ArenaCaps caps_{0, 0, 0, 0};
   bool list_growable_ = false;  // exact-size arenas grow their list storage on demand
