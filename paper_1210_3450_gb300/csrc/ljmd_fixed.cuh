@@ -21,7 +21,9 @@
 //   g / 24                2^-88   (96 bits; |g / 24| < 4.77)
 //   force sums / 24       2^-84   (96 bits; 468 pairs of the largest force, 4.37,
 //                         reach their range)
-// Pairs closer than sqrt(0.84) and lists longer than kFixMaxList take the FP64 pipe.
+// Pairs closer than sqrt(0.84) take the FP64 pipe, for lists longer than kFixMaxList those
+// closer than 1 (beyond it a force / 24 is below 1.081: 1,895 pairs reach the sums' range),
+// for lists longer than kFixMaxLong all (fix_limit).
 // Separations of kFixMaxSep and more may come out of the wrapped differences as shorter
 // ones (and r^2 of 128 and more as a negative number), so a loop that hands every listed
 // pair on, and not only those that passed a test on the shadows, must know that no listed
@@ -34,7 +36,8 @@
 
 namespace ljmd {
 
-constexpr int kFixMaxList = 448;                                // longest list summed in 96 bits
+constexpr int kFixMaxList = 448;                                // longest list summed in 96 bits ...
+constexpr int kFixMaxLong = 1880;                               // ... without pairs closer than 1
 constexpr unsigned kFixR2Min = 14092862u;                      // 0.84 in units of 2^-24 (r^2's high word)
 constexpr double kFixMaxRc = 3.99;                              // r^2 < 16
 constexpr double kFixMaxSep = 7.9;                              // separations below 8, r^2 < 128
@@ -408,15 +411,21 @@ static __device__ __forceinline__ unsigned long long fix_separation2(const longl
   return fix_r2(fx, fy, fz);
 }
 
+// The squared distance (its high word) from which a particle's pairs are taken in fixed
+// point.
+static __device__ __forceinline__ unsigned fix_limit(int listed) {
+  return listed <= kFixMaxList ? kFixR2Min : listed <= kFixMaxLong ? 1u << 24 : ~0u;
+}
+
 // One pair: where r < rc, its force is added to the sums (qi, code, L as above; rc2 in
 // units of 2^-56, c2 as for fix_force_factor). Returns true, with nothing added, for a pair closer than the range (the FP64 pipe takes it).
 static __device__ __forceinline__ bool fix_pair(const longlong4_32a& qi, const longlong4_32a& qj, unsigned code,
                                                 long long L, long long rc2, const FixC2& c2, FixSum& sx, FixSum& sy,
-                                                FixSum& sz) {
+                                                FixSum& sz, unsigned limit = kFixR2Min) {
   Fix2 fx, fy, fz;
   fix_separation(qi, qj, code, L, fx, fy, fz);
   const unsigned long long r2 = fix_r2(fx, fy, fz);
-  const bool far = (unsigned)(r2 >> 32) >= kFixR2Min;
+  const bool far = (unsigned)(r2 >> 32) >= limit;
   if (far & ((long long)(r2 - (unsigned long long)rc2) < 0)) {
     const Fix3 g = fix_force_factor(fix_rcp(r2), c2);
     sx.add(g, fx);

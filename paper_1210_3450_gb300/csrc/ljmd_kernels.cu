@@ -1806,7 +1806,7 @@ struct PipeForce {
   const int n;
   long long rc2b;
   double x = 0.0, y = 0.0, z = 0.0;
-  static constexpr bool fixed = false;
+  static constexpr unsigned limit = ~0u;
 
   __device__ __forceinline__ PipeForce(const DevArrays& a_, const TileCtx& t_, const SysParams& P, int cur)
       : a(a_), t(t_), xs(a_.x[cur] + P.p_off), xi(t_.act ? xs[t_.local] : make_double4_32a(0.0, 0.0, 0.0, 0.0)), L(P.L),
@@ -1836,16 +1836,21 @@ struct PipeForce {
   }
 };
 
-// The same in fixed point (ljmd_fixed.cuh) where the system's cutoff and the particle's
-// list length allow it; other particles' pairs and those closer than its range take the
-// FP64 pipe, in the same order as above.
+// The same in fixed point (ljmd_fixed.cuh) where the system's cutoff, the particle's list
+// length and the pair's distance allow it; the other pairs take the FP64 pipe, in the same
+// order as above. kAny: for warps in which some particle has more than 448 listed pairs (with
+// all of those on the FP64 pipe, beside shorter lists in the same warps, a step of 2,000
+// particles at density 1.5, rc 3.9, took 1.3 times as long as without fixed point; 0.8 now) or
+// a system out of the cutoff's range. As a run-time limit for every warp it cost 5 % of the
+// step.
+template <bool kAny>
 struct PairForce {
   const DevArrays& a;
   const TileCtx& t;
   const SysParams& P;
   int cur;
   longlong4_32a qi;
-  bool fixed;
+  unsigned limit;  // kAny; else kFixR2Min
   FixSum sx, sy, sz;
   double* slow;  // the FP64 pairs' sums, one column of a shared array per thread
   int stride;
@@ -1854,8 +1859,8 @@ struct PairForce {
                                        double* slow_, int stride_)
       : a(a_), t(t_), P(P_), cur(cur_), slow(slow_), stride(stride_) {
     slow[0] = slow[stride] = slow[2 * stride] = 0.0;
-    fixed = P.fixed && cnt <= kFixMaxList;
-    qi = fixed && t.act ? a.xl[cur][t.s] : longlong4_32a{0, 0, 0, 0};
+    limit = !kAny ? kFixR2Min : P.fixed ? fix_limit(cnt) : ~0u;
+    qi = t.act ? a.xl[cur][t.s] : longlong4_32a{0, 0, 0, 0};
     qi.x -= kFixBias; qi.y -= kFixBias; qi.z -= kFixBias;  // separations come biased for fix_split
   }
   __device__ __forceinline__ void fp64_pair(uint32_t j, unsigned code) {
@@ -1881,25 +1886,19 @@ struct PairForce {
     return partner_slot(a, t.sys, e, P.n, (uint32_t)t.local);
   }
   __device__ __forceinline__ longlong4_32a load(uint32_t e) const {
-    if (fixed) return a.xl[cur][P.p_off + slot(e)];
-    return longlong4_32a{0, 0, 0, 0};
+    return a.xl[cur][P.p_off + slot(e)];
   }
   __device__ __forceinline__ void pair(const longlong4_32a& qj, uint32_t e) {
     const unsigned code = e >> kIdxBits;
-    if (fixed) {
-      if (fix_pair(qi, qj, code, P.Lfix, P.rc2fix, FixC2{P.c2fix, P.c2fix_lo}, sx, sy, sz)) fp64_pair(slot(e), code);
-    } else {
+    if (fix_pair(qi, qj, code, P.Lfix, P.rc2fix, FixC2{P.c2fix, P.c2fix_lo}, sx, sy, sz, kAny ? limit : kFixR2Min))
       fp64_pair(slot(e), code);
-    }
   }
   // The sums as FP64 (the FP64 pairs' share added where there is one).
   __device__ __forceinline__ void result(double& x, double& y, double& z) const {
     x = slow[0]; y = slow[stride]; z = slow[2 * stride];
-    if (fixed) {
-      const bool some = x != 0.0 || y != 0.0 || z != 0.0;
-      const double fx = sx.value24(), fy = sy.value24(), fz = sz.value24();
-      x = some ? fx + x : fx; y = some ? fy + y : fy; z = some ? fz + z : fz;
-    }
+    const bool some = x != 0.0 || y != 0.0 || z != 0.0;
+    const double fx = sx.value24(), fy = sy.value24(), fz = sz.value24();
+    x = some ? fx + x : fx; y = some ? fy + y : fy; z = some ? fz + z : fz;
   }
 };
 
@@ -1934,7 +1933,7 @@ __global__ void __launch_bounds__(BLOCK, FIXED ? 1024 / BLOCK : 1) k_step_fp64(D
                                    [&](const auto& q, uint32_t e) { pf.pair(q, e); });
       } else {
         const uint32_t* lp = a.nbr + list_word(P.l_off, t.tl, P.kmax, lane, 0);
-        const bool shadows = pf.fixed && P.wide;
+        const bool shadows = pf.limit != ~0u && P.wide;
         for (int k = 0; k < cnt; ++k) {
           const uint32_t e = __ldg(lp + (int64_t)(k >> 2) * (4 * kTile) + (k & 3));
           if (shadows) {  // the queue's test: pairs surely outside rc, which may be out of range, are left out
@@ -1948,8 +1947,13 @@ __global__ void __launch_bounds__(BLOCK, FIXED ? 1024 / BLOCK : 1) k_step_fp64(D
       }
       pf.result(Fx, Fy, Fz);
     };
-    if constexpr (FIXED) sum(PairForce(a, t, P, cur, cnt, &slow[0][threadIdx.x], BLOCK));
-    else sum(PipeForce<MODE>(a, t, P, cur));
+    if constexpr (!FIXED) {
+      sum(PipeForce<MODE>(a, t, P, cur));
+    } else if (P.fixed && __reduce_max_sync(kFull, cnt) <= kFixMaxList) {  // uniform over the warp
+      sum(PairForce<false>(a, t, P, cur, cnt, &slow[0][threadIdx.x], BLOCK));
+    } else {
+      sum(PairForce<true>(a, t, P, cur, cnt, &slow[0][threadIdx.x], BLOCK));
+    }
   }
   unsigned long long d2b = 0ull;
   if (t.act) d2b = integrate<false>(a, P, t, cur, a.x[cur][t.s], Fx, Fy, Fz, ka, kb, flags);

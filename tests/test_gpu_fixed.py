@@ -118,3 +118,29 @@ def test_leaving_and_entering_the_fixed_point_form():
         for got in (again, run(s)):
             for p, q in zip(ref, got):
                 np.testing.assert_array_equal(p, q)
+
+
+@pytest.mark.parametrize("rho,amp", [(1.5, 0.02), (6.6, 0.01)])
+def test_lists_beyond_the_sums(rho, amp):
+    """Lists around 448 and 1,880 partners, where the range of the fixed-point pairs is cut
+    back, in the same warps as shorter ones: every force within 1e-12 of the rms force of its
+    own kind of list, both force loops equal."""
+    from paper_1210_3450_gb300 import MD_FP64, LJSystem
+    x, box = li.perturbed_fcc(6000, rho, amp, 8)
+    keep = (x[:, 0] < 0.6 * box) | (np.arange(len(x)) % 3 == 0)
+    x = np.ascontiguousarray(x[keep])
+    ref = oracle.forces_brute(x, box, 3.9)
+    size = np.sqrt((ref ** 2).sum(1))
+    got = []
+    with LJSystem(box, len(x), 3.9, 0.3, MD_FP64) as s:
+        for queue in (1, 0):
+            s.set_tuning(fp64_queue=queue)
+            s.set_state(x, np.zeros_like(x))
+            got.append(s.forces())
+        cnt = np.diff(s.get_list()[0])
+    limit = 448 if rho < 2 else 1880
+    assert cnt.min() <= limit < cnt.max()
+    np.testing.assert_array_equal(got[0], got[1])
+    for part in (cnt <= limit, cnt > limit):
+        rms = np.sqrt((size[part] ** 2).mean())
+        assert np.abs(got[0] - ref)[part].max() <= 1e-12 * rms
