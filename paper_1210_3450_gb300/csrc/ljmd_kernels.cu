@@ -1905,10 +1905,10 @@ struct PairForce {
 // FIXED: an arena with systems in the range of the fixed-point pairs; the instance without
 // keeps its sums and the particle in registers (a step of 100,000 particles at rc 4.5 takes
 // 1.33 ms with it and 1.43 with the other). QUEUE false: the plain loop over the list.
-// 32 warps per SM (64 registers): 1.01 ms per pair pass at 2,048,000 particles against
-// 1.06 at 28 and 1.08 at 24.
+// 28 warps per SM (72 registers, no spills): 20 steps of 2,048,000 particles take 23.9 ms
+// against 24.2 at 32 and at 24 warps, of 100,000 2.06 against 2.13 and 2.00.
 template <int BLOCK, int MODE, bool QUEUE, bool FIXED>
-__global__ void __launch_bounds__(BLOCK, FIXED ? 1024 / BLOCK : 1) k_step_fp64(DevArrays a, int cur, double ka, double kb, int flags) {
+__global__ void __launch_bounds__(BLOCK, FIXED ? 896 / BLOCK : 1) k_step_fp64(DevArrays a, int cur, double ka, double kb, int flags) {
   __shared__ uint32_t qbuf[QUEUE ? kQueue64 : 1][BLOCK];  // entry q of thread t at [q][t]: no bank conflicts
   __shared__ double slow[FIXED ? 3 : 1][BLOCK];
   if (a.ctl) {  // graph-captured loop (uniform over the grid)
