@@ -252,9 +252,17 @@ void launch_build_list(const DevArrays& a, int cur, const Tuning& tu, cudaStream
 void launch_decide(const DevArrays& a, int nsys, int fp32, int vflag, int32_t* rebuild, int32_t* rebuild_ids,
                    int32_t* reb_pref, int32_t* reb_count, cudaGraphConditionalHandle h_if,
                    cudaGraphConditionalHandle h_loop, int last, cudaStream_t s);
-// Persistent step loop of small arenas: threads per particle for the given launch (0: the
-// arena does not fit; kmax: the longest list capacity) and the shared list stride.
-int loop_lanes(int fp32, int ntiles, int kmax, int* stride);
+// Persistent step loop of small arenas: the launches of an arena, the most threads per
+// particle first (kmax: the longest list capacity).
+struct LoopPlan {
+  int lanes;      // threads per particle
+  int stride;     // list words per particle in shared memory
+  int blocks;     // of the launch
+  int resident;   // blocks that are resident at once (0: the arena does not fit)
+  int alone;      // the same for a launch that has the device for itself
+};
+constexpr int kLoopPlans = 4;
+void loop_plans(int fp32, int ntiles, int kmax, LoopPlan* plans);
 // One cooperative launch that takes ctl->target steps, rebuilds included (see k_loop).
 cudaError_t launch_loop(const DevArrays& a, const LoopArgs& g, cudaStream_t s);
 // mode 0: FP64 reciprocal; 1..4: approximate reciprocal of Sec. 3.3 (8 bits,

@@ -3,6 +3,8 @@
 // the paper (rebuild when twice the largest displacement since the last build
 // reaches the skin) and the rebuild sequence (bin, sort, gather, list build).
 #include <algorithm>
+#include <atomic>
+#include <chrono>
 #include <cmath>
 #include <cstring>
 #include <string>
@@ -1145,6 +1147,55 @@ int Engine::lose_states(cudaStream_t s) {
   return sync_check(s);
 }
 
+// The step calls under way on each device, of all handles: a grid of the persistent loop
+// waits until all its blocks are resident, so calls that step at the same time (threads
+// with handles of their own) each take their share of the device, or the graph loop if
+// none of its launches fits in that. With a whole device for each, they ran one after the
+// other: 8 threads of 4,000 particles (FP32 forces, 200 steps each) took 14.8 ms, with
+// graph launches 5.6, with shares 3.5. The most calls of the last 10 ms count, so that the
+// first of several that start together again does not take the whole device (6.9 ms).
+// Results do not depend on the launch.
+class StepCall {
+ public:
+  explicit StepCall(bool on) {
+    int dev = -1;
+    if (!on || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices) return;
+    dev_ = dev;
+    const int n = ++calls_[dev];
+    if (n > 1 && n >= peak(dev)) peak_[dev] = now() << 16 | n;
+  }
+  ~StepCall() {
+    if (dev_ >= 0) --calls_[dev_];
+  }
+  StepCall(const StepCall&) = delete;
+  StepCall& operator=(const StepCall&) = delete;
+  static int count() {
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices) return 1;
+    return std::max(calls_[dev].load(), peak(dev));
+  }
+
+ private:
+  static constexpr int kDevices = 64;
+  static std::atomic<int> calls_[kDevices];
+  static std::atomic<int64_t> peak_[kDevices];  // time (us) and number of the most calls
+  int dev_ = -1;
+  static int64_t now() {
+    using namespace std::chrono;
+    return duration_cast<microseconds>(steady_clock::now().time_since_epoch()).count();
+  }
+  static int peak(int dev) {
+    const int64_t p = peak_[dev].load();
+    return now() - (p >> 16) < 10000 ? (int)(p & 0xffff) : 0;
+  }
+};
+std::atomic<int> StepCall::calls_[StepCall::kDevices];
+std::atomic<int64_t> StepCall::peak_[StepCall::kDevices];
+
+// Steps of one launch of the persistent loop: a long call gives its share of the device back
+// now and then (a launch more per 2,000 steps costs 0.2 % of 1,000 particles' steps).
+constexpr int64_t kLoopSteps = 2000;
+
 // Threads per particle of the persistent loop: full lists, at most kLoopMaxSys systems,
 // and for the FP64 form the fixed-point range of every system, for all its listed pairs
 // (the loop does not test them on the shadows first).
@@ -1155,17 +1206,29 @@ int Engine::loop_plan() {
   int kmax = 0;
   for (const SysHost& h : sys_)
     if (h.used) kmax = std::max(kmax, h.kmax);
-  if (loop_ver_ == struct_ver_ && loop_kmax_ == kmax) return loop_lanes_;
-  loop_ver_ = struct_ver_;
-  loop_kmax_ = kmax;
-  loop_lanes_ = 0;
-  if (precision_ == 0) {
-    if (kmax > kFixMaxList) return 0;
+  if (loop_ver_ != struct_ver_ || loop_kmax_ != kmax) {
+    loop_ver_ = struct_ver_;
+    loop_kmax_ = kmax;
+    loop_refused_ = precision_ == 0 && kmax > kFixMaxList;
     for (const SysHost& h : sys_)
-      if (h.used && (h.spec.rc > kFixMaxRc || fix_wide(h.spec.rc, h.spec.skin))) return 0;
+      if (precision_ == 0 && h.used && (h.spec.rc > kFixMaxRc || fix_wide(h.spec.rc, h.spec.skin))) loop_refused_ = true;
+    if (!loop_refused_) loop_plans(precision_ == 1, ntiles_, kmax, loop_plans_);
   }
-  loop_lanes_ = loop_lanes(precision_ == 1, ntiles_, kmax, &loop_stride_);
-  return loop_lanes_;
+  if (loop_refused_) return 0;
+  const int calls = StepCall::count();
+  auto take = [&](bool share) {
+    for (const LoopPlan& p : loop_plans_)
+      if (p.blocks > 0 && (share ? (int64_t)p.blocks * calls <= p.resident : p.blocks <= p.alone)) {
+        loop_ = p;
+        return p.lanes;
+      }
+    return 0;
+  };
+  if (calls <= 1) return take(false);
+  const int lanes = take(true);
+  // two of the FP64 form one after the other rather than two graph loops (two threads of
+  // 16,000 particles, 200 steps: 9.8 against 12.5 ms; four: 20.6 against 15.0)
+  return lanes == 0 && calls == 2 && precision_ == 0 ? take(false) : lanes;
 }
 
 int Engine::run_loop(int64_t nsteps, bool stored, bool steady, int64_t* done, bool* finished, cudaStream_t s,
@@ -1190,8 +1253,8 @@ int Engine::run_loop(int64_t nsteps, bool stored, bool steady, int64_t* done, bo
   g.stored = stored && g.rebuild0 == 0u && forces_valid() ? 1 : 0;
   g.steady = steady ? 1 : 0;
   g.finish = 1;
-  g.stride = loop_stride_;
-  g.lanes = loop_lanes_;
+  g.stride = loop_.stride;
+  g.lanes = loop_.lanes;
   g.polls = loop_polls_;
   g.rebuild_ids = d_rebuild_ + nsys();
   g.reb_pref = d_rebuild_ + 2 * nsys();
@@ -1211,7 +1274,7 @@ int Engine::run_loop(int64_t nsteps, bool stored, bool steady, int64_t* done, bo
     // once): no step is taken here, the caller goes on without the loop, and an error that
     // is not the loop's own comes up there
     cudaGetLastError();
-    loop_lanes_ = 0;
+    loop_refused_ = true;
     return kOK;
   }
   CK(cudaMemcpyAsync(h_ctl_, d_ctl_, sizeof(GraphCtl), cudaMemcpyDeviceToHost, s));
@@ -1239,39 +1302,47 @@ int Engine::step(int64_t nsteps, const std::vector<double>& dt, cudaStream_t s) 
   }
   if (nsteps == 0 || !any_active()) return kOK;  // an empty or fully paused arena: nothing to do
   CKR(upload_params());
+  const StepCall call(!nvt_);  // (a Nose-Hoover call counts itself)
   int64_t it = 0;
-  bool finished = false;
+  bool open = false;  // the closing half kick of the last step is still due
   if (graph_ && !timing_ && loop_plan() > 0) {
     CKR(have_states());  // (the launch builds the lists and evaluates the forces that are due)
     while (it < nsteps && loop_plan() > 0) {
       int64_t done = 0;
-      const int rc = run_loop(std::min<int64_t>(nsteps - it, 1 << 30), it == 0, it > 0, &done, &finished, s);
+      bool finished = false;
+      const int rc = run_loop(std::min(nsteps - it, kLoopSteps), !open, open, &done, &finished, s);
       it += done;
       if (rc != kOK) return rc;
+      open = !finished && (open || done > 0);
+      if (finished)
+        for (SysHost& h : sys_)
+          if (h.active) h.f_valid = true;
     }
   }
-  if (!finished) {
+  if (it < nsteps || open) {
     CKR(ensure_lists(s));
-    if (it == 0) CKR(ensure_forces(s));
+    if (!open) CKR(ensure_forces(s));
     CK(cudaMemsetAsync(d_ctl_, 0, sizeof(GraphCtl), s));
   }
   if (graph_ && !timing_) {
     while (nsteps - it >= 2) {
-      const int first = (it == 0 ? (kStepUseStoredF | kStepDrift | kStepKickB) : (kStepKickA | kStepKickB | kStepDrift)) |
+      const int first = (!open ? (kStepUseStoredF | kStepDrift | kStepKickB) : (kStepKickA | kStepKickB | kStepDrift)) |
                         (rule_ == 1 ? kStepVmax : 0);
       int64_t done = 0;
       const int rc = run_graph(std::min<int64_t>(nsteps - it, 1 << 30) & ~int64_t(1), first, &done, s);
       it += done;
+      open = open || done > 0;
       if (rc != kOK) return rc;
     }
   }
   for (; it < nsteps; ++it) {
-    if (it == 0) CKR(launch_step(0.0, 0.5, kStepUseStoredF | kStepDrift, s));
+    if (!open) CKR(launch_step(0.0, 0.5, kStepUseStoredF | kStepDrift, s));
     else CKR(launch_step(0.5, 0.5, kStepDrift, s));
+    open = true;
     cur_ ^= 1;
     CKR(post_drift(s));
   }
-  if (!finished) {  // the closing half kick of the last step
+  if (open) {
     CKR(launch_step(0.5, 0.0, kStepStoreF, s));
     CKR(sync_check(s));
   }
@@ -1385,7 +1456,10 @@ int Engine::step_nvt(int64_t nsteps, const std::vector<double>& dt, const std::v
   CK(cudaMemcpyAsync(d_thermo_, th.data(), sizeof(Thermo) * (size_t)ns, cudaMemcpyHostToDevice, s));
   unsigned long long* ke = d_loop_ + 1 + 3 * (size_t)ns;
   CK(cudaMemsetAsync(ke, 0, sizeof(unsigned long long) * kKeWords * (size_t)ns, s));
+  const StepCall call(true);
+  nvt_ = true;
   const int rc = nvt_steps(nsteps, dt, ke, s);
+  nvt_ = false;
   if (rc == kErrTimeout) return rc;  // the states are lost
   // after an error in a step as well: the thermostats have moved with the particles
   const std::string why = last_error_cstr();
@@ -1414,8 +1488,8 @@ int Engine::nvt_steps(int64_t nsteps, const std::vector<double>& dt, unsigned lo
   while (it < nsteps && graph_ && !timing_ && loop_plan() > 0) {
     int64_t done = 0;
     bool finished = false;
-    const int rc = run_loop(std::min<int64_t>(nsteps - it, 1 << 30), true, false, &done, &finished, s, true, !opened,
-                            it + std::min<int64_t>(nsteps - it, 1 << 30) < nsteps ? 2 : 1);
+    const int rc = run_loop(std::min(nsteps - it, kLoopSteps), true, false, &done, &finished, s, true, !opened,
+                            nsteps - it > kLoopSteps ? 2 : 1);
     it += done;
     if (rc != kOK) return rc;
     for (SysHost& h : sys_)

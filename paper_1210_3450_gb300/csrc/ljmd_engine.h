@@ -190,8 +190,9 @@ class Engine {
   void drop_graphs();
   int run_graph(int64_t nsteps, int first_flags, int64_t* done, cudaStream_t s);
   // Persistent step loop of small arenas (tuning key 5 as well): all steps of a call in
-  // one cooperative launch, the closing force evaluation included. loop_plan returns its
-  // threads per particle, 0 where the arena does not take it.
+  // one cooperative launch (kLoopSteps at most), the closing force evaluation included.
+  // loop_plan chooses the launch (loop_) and returns its threads per particle, 0 where the
+  // arena does not take it.
   int loop_plan();
   // nvt: Nose-Hoover steps (d_thermo_), with an opening half step if `open` is set.
   int run_loop(int64_t nsteps, bool stored, bool steady, int64_t* done, bool* finished, cudaStream_t s,
@@ -233,7 +234,9 @@ class Engine {
   GraphCtl* d_ctl_ = nullptr;
   unsigned long long* d_loop_ = nullptr;  // persistent loop: barrier word, kLoopWords per system
   Thermo* d_thermo_ = nullptr;            // thermostats (nsys) of md_step_nvt
-  int loop_lanes_ = 0, loop_stride_ = 0;
+  LoopPlan loop_plans_[kLoopPlans] = {};
+  bool loop_refused_ = false;             // the driver refused a launch
+  LoopPlan loop_{};                       // the launch that loop_plan chose
   int loop_polls_ = 1 << 21;              // of a grid barrier before it gives up (about a second)
   int64_t loop_ver_ = -1;                 // struct_ver_ the plan was made for ...
   int loop_kmax_ = -1;                    // ... and the longest list capacity
@@ -245,6 +248,7 @@ class Engine {
   int precision_ = 0;
   int rule_ = 0;
   bool half_ = false;
+  bool nvt_ = false;  // within step_nvt
   int n_fixed_ = 0;  // systems in the range of the fixed-point pairs
   int cur_ = 0;
   ArenaCaps caps_{0, 0, 0, 0};

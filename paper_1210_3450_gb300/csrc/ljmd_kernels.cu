@@ -3352,28 +3352,28 @@ const void* loop_kernel(int T) {
 unsigned loop_blocks(int ntiles, int T) { return (unsigned)(((int64_t)ntiles * kTile * T + kLoopBlock - 1) / kLoopBlock); }
 }  // namespace
 
-// The most threads per particle whose blocks are all resident at once: 32 and 16 up to
-// two blocks per SM (2,432 and 4,864 particles), 8 and 4 up to what fits (three or four
-// blocks of the FP32 form, 38,912 particles; three of the FP64 form, 29,184).
-int loop_lanes(int fp32, int ntiles, int kmax, int* stride) {
+// A launch takes the most threads per particle whose blocks are all resident at once: alone
+// on the device 32 and 16 up to two blocks per SM (2,432 and 4,864 particles), 8 and 4 up
+// to what fits (three or four blocks of the FP32 form, 38,912 particles; three of the FP64
+// form, 29,184).
+void loop_plans(int fp32, int ntiles, int kmax, LoopPlan* plans) {
   int dev = 0, sms = 0;
-  if (ntiles <= 0 || (int64_t)ntiles * kTile > 65535 /* LoopWord */ || cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
-  for (int T : {32, 16, 8, 4}) {
+  const bool fits = ntiles > 0 && (int64_t)ntiles * kTile <= 65535 /* LoopWord */ && cudaGetDevice(&dev) == cudaSuccess &&
+                    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess;
+  for (int m = 0; m < kLoopPlans; ++m) {
+    const int T = 32 >> m;
+    LoopPlan& p = plans[m];
+    p = LoopPlan{T, 0, 0, 0, 0};
+    if (!fits) continue;
     size_t bytes = 0;
     int bps = 0;
-    const cudaError_t e = fp32 ? loop_setup<true>(T, kmax, stride, &bytes, &bps) : loop_setup<false>(T, kmax, stride, &bytes, &bps);
-    if (e != cudaSuccess) {
-      cudaGetLastError();
-      continue;
-    }
-    if (T >= 16) bps = std::min(bps, 2);
-    if (loop_blocks(ntiles, T) <= (unsigned)(sms * bps)) return T;
+    const cudaError_t e = fp32 ? loop_setup<true>(T, kmax, &p.stride, &bytes, &bps) : loop_setup<false>(T, kmax, &p.stride, &bytes, &bps);
+    if (e != cudaSuccess) continue;
+    p.blocks = (int)loop_blocks(ntiles, T);
+    p.resident = sms * bps;
+    p.alone = T >= 16 ? sms * std::min(bps, 2) : p.resident;
   }
-  return 0;
+  cudaGetLastError();
 }
 
 cudaError_t launch_loop(const DevArrays& a, const LoopArgs& g, cudaStream_t s) {

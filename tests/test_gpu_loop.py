@@ -123,3 +123,49 @@ def test_several_threads(ljmd, precision):
         for p, q in zip(a[:3], b[:3]):
             np.testing.assert_array_equal(p, q)
         assert a[3] == b[3]
+
+
+@pytest.mark.parametrize("precision", [0, 1], ids=["fp64", "fp32"])
+@pytest.mark.parametrize("nvt", [False, True], ids=["nve", "nvt"])
+def test_more_steps_than_a_launch(ljmd, precision, nvt):
+    """A call of more steps than the loop takes in one launch, an odd number of launches."""
+    n, steps = 108, 4003
+    x, box = li.perturbed_fcc(n, 0.3, 0.1, 3)
+    v = li.maxwell_boltzmann(n, 1.0, 4)
+    out = []
+    for graph in (0, 1):
+        with ljmd.LJSystem(box, n, 2.5, 0.3, precision) as s:
+            s.set_tuning(graph=graph)
+            s.set_state(x, v)
+            ze = s.step_nvt(steps, 0.002, 1.0, 3.0 * n * 0.05) if nvt else s.step(steps, 0.002)
+            out.append((*s.get_state(), s.forces(), np.array(ze if nvt else [0.0]), np.array(list(s.stats().values()))))
+    for p, q in zip(*out):
+        np.testing.assert_array_equal(p, q)
+
+
+def test_several_threads_share_the_device(ljmd):
+    """Handles stepped at the same time take smaller launches or graph launches: the same
+    results, NVE and Nose-Hoover, over several calls."""
+    from concurrent.futures import ThreadPoolExecutor
+    cases = [(1000 + 700 * (k % 5), k % 2, k % 3 == 0) for k in range(10)]
+
+    def run(case):
+        n, precision, nvt = case
+        x, box = li.perturbed_fcc(n, 0.8, 0.1, n)
+        v = li.maxwell_boltzmann(n, 0.9, n + 1)
+        with ljmd.LJSystem(box, n, 2.5, 0.3, precision) as s:
+            s.set_state(x, v)
+            ze = [0.0, 0.0]
+            for steps in (40, 1, 33, 80):
+                if nvt:
+                    ze = s.step_nvt(steps, 0.004, 0.9, 3.0 * n * 0.05, *ze)
+                else:
+                    s.step(steps, 0.004)
+            return (*s.get_state(), s.forces(), np.array(ze))
+
+    alone = [run(c) for c in cases]
+    with ThreadPoolExecutor(len(cases)) as pool:
+        together = list(pool.map(run, cases))
+    for a, b in zip(alone, together):
+        for p, q in zip(a, b):
+            np.testing.assert_array_equal(p, q)
