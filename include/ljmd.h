@@ -144,7 +144,8 @@ MD_API int md_get_state(md_ctx* ctx, double* x, double* v);
 MD_API int md_get_state_dev(md_ctx* ctx, double* x_dev, double* v_dev, void* stream);
 
 /* Advance nsteps velocity-Verlet steps of size dt (nsteps >= 0). Blocks until done.
- * Errors: MD_ERR_STATE (no state), MD_ERR_NONFINITE, MD_ERR_LIST_OVERFLOW, MD_ERR_CUDA. */
+ * Errors: MD_ERR_STATE (no state), MD_ERR_NONFINITE, MD_ERR_LIST_OVERFLOW, MD_ERR_TIMEOUT (the
+ * state is lost: set one anew), MD_ERR_CUDA. */
 MD_API int md_step(md_ctx* ctx, int64_t nsteps, double dt);
 
 /* Same, ordered on the given stream (the call still waits for the per-step list
@@ -155,7 +156,9 @@ MD_API int md_step_async(md_ctx* ctx, int64_t nsteps, double dt, void* stream);
  * step, one velocity-Verlet step (md_step) and a thermostat half step, the reversible
  * splitting: zeta += dt/4 G, eta += dt/2 zeta, v *= exp(-dt/2 zeta), zeta += dt/4 G'
  * with G = (2 KE - 3 (N - 1) T) / Q. zeta and eta (thermostat velocity and position)
- * are read and updated; KE + PE + Q zeta^2 / 2 + 3 (N - 1) T eta is conserved. */
+ * are read and updated, after an error in a step as well (to the thermostat that the
+ * velocities have moved with; not after MD_ERR_TIMEOUT); KE + PE + Q zeta^2 / 2 +
+ * 3 (N - 1) T eta is conserved. KE is an exact sum of the squared velocity components. */
 MD_API int md_step_nvt(md_ctx* ctx, int64_t nsteps, double dt, double T, double Q, double* zeta,
                        double* eta);
 
@@ -288,18 +291,20 @@ MD_API int md_probe_fma_rate(int kind, int64_t iters, double* fma_per_s);
  *                        4 warp-cooperative (candidates shared by the lanes of a
  *                        row, staged in shared memory); 5 as 0, each row's
  *                        candidates for the whole warp first copied into shared
- *                        memory with coalesced loads (full-list arenas of up to about
- *                        42,000 particles instead take one candidate per lane, a block
- *                        for each run of slots)
+ *                        memory with coalesced loads (arenas of up to about 42,000
+ *                        particles instead take one candidate per lane, a block for
+ *                        each run of slots)
  *   MD_TUNE_STEP_HINT    1: L1 eviction hints on the FP32 step kernel's loads (list
  *                        words not kept in L1, partner positions kept)
  *   MD_TUNE_GRAPH        1: md_step runs its steps in CUDA-graph launches (a loop node of
  *                        two steps, each followed by a device-side list-validity
  *                        decision and a conditional rebuild pass), reading the
  *                        control words once per launch; small full-list arenas (up to
- *                        32 systems of at most about 30,000 particles together) run all
- *                        steps of a call in one cooperative launch instead; 0: the host
- *                        decides after every step. Results are identical. Timing (md_set_timing)
+ *                        32 systems of at most about 30,000 particles together; FP64
+ *                        with rc <= 3.99 and rc + 2 skin <= 7.9) run the steps of a call
+ *                        in cooperative launches of up to 2,000 instead, each a share of
+ *                        the device where several handles step at the same time; 0: the
+ *                        host decides after every step. Results are identical. Timing (md_set_timing)
  *                        uses the host-driven loop.
  *   MD_TUNE_FP64_QUEUE   1: the FP64 force loops classify each listed pair on the
  *                        fixed-point shadow positions first and compute only the

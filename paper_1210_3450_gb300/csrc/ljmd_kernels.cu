@@ -1704,17 +1704,17 @@ __device__ __forceinline__ double force_factor(double r2, double c2x8) {
 
 // FP64 form. On GB300 a warp's FP64 instruction holds the FP64 pipe for 64 cycles, so
 // with the 17 FP64 instructions of a pair the loop ran at that pipe's rate (3.7 ms per
-// step at 2,048,000 particles, pipe 89 % busy; 1.05 now). Two things take the load off it:
+// step at 2,048,000 particles, pipe 89 % busy; 1.10 now). Two things take the load off it:
 //   The pair arithmetic runs in 64-bit fixed point on the integer multipliers
-//   (ljmd_fixed.cuh: about 245 cycles per pair and warp against 1,140): 1.01 ms per
-//   pair pass, with smaller errors than the FP64 pipe's.
+//   (ljmd_fixed.cuh: 38 products of 4 cycles each, against 1,090 cycles), with smaller
+//   errors than the FP64 pipe's.
 //   Pairs outside rc are left out before it. Each thread classifies its listed
 //   partners on their fixed-point shadow positions (integer separations, float r^2)
 //   against rc^2 (1 + 1e-5), a bound that no pair inside rc can exceed (each shadow
 //   coordinate errs by at most half a unit of L / 2^32, and the float r^2 by a few
 //   parts in 1e7), and queues the list words of the pairs that may be inside in shared
 //   memory; the pairs then run in rounds in which every thread with partners left
-//   takes the next one of its own queue (1.10 ms without the queue).
+//   takes the next one of its own queue (1.26 ms per step without the queue).
 // The FP64 pipe still takes the pairs out of the fixed-point range, cutoffs above
 // kFixMaxRc and the approximate-reciprocal modes: 3 DADD for the separation and 3
 // operations for r^2, the exact test r^2 < rc^2 (bit patterns, r^2 >= 0), the
@@ -2094,9 +2094,10 @@ __global__ void __launch_bounds__(kBlock) k_integrate_half(DevArrays a, int cur,
 // fixed point (ljmd_fixed.cuh; sums exact, over the tile as well) where the cutoff
 // allows it, else and for close pairs on the FP64 pipe. With all pairs on that pipe and
 // each taken twice the kernel ran at its rate: 455 us at 262,143 particles.
-// 28 warps per SM (72 registers): a call takes 390 us at 864,000 particles, against 403 at
-// 24 and 426 at 32 warps. Splitting each particle's pairs evenly instead (by slot parity):
-// 398, since whole warps no longer skip the lower half of their lists.
+// 28 warps per SM (72 registers): a call takes 419 us at 864,000 particles, against 426 at
+// 24 and 443 at 32 warps. Splitting each particle's pairs evenly instead (by slot parity)
+// was 2 % slower, since whole warps no longer skip the lower half of their lists. The bits
+// below the second half of r^-6 and r^-12 cost 8 % (390 us without them).
 // xl: positions in pair units.
 __global__ void __launch_bounds__(kBlock, 7) k_pe_virial(DevArrays a, int cur, int with_pairs,
                                                          const int32_t* __restrict__ select, const longlong4_32a* xl) {
@@ -2426,8 +2427,9 @@ __global__ void k_thermostat(DevArrays a, int nsys, Thermo* thermo, int halves, 
 // (step, decision, conditional rebuild node, and five kernels per rebuild) it took 28 to
 // 33 us at 1000 to 32,000 particles with FP32 forces and 70 to 77 with FP64 ones, of which
 // the pair arithmetic is about 1 to 8. Here one cooperative launch takes all steps of a
-// call: 6.8, 9.9, 17 and 24 us at 1000, 4000, 16,000 and 32,000 particles (FP32 forces,
-// rebuilds included), 7.8, 11.5 and 26 us at 1000, 4000 and 16,000 (FP64). Without its
+// call: 8.0, 10.4, 18 and 25 us at 1000, 4000, 16,000 and 32,000 particles (FP32 forces; 200
+// steps from a lattice, its lists and rebuilds included), 9.0, 12.4 and 27 us at 1000, 4000
+// and 16,000 (FP64). Without its
 // rebuilds a step of 4000 particles takes 5.0 us: forces 2.2, update 0.9, barrier 1.5,
 // decision 0.4; a rebuild 40 us. Several threads share a particle, whose
 // position, velocity and list stay in registers and shared memory between rebuilds; a

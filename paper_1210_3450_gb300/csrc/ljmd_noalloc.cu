@@ -231,7 +231,8 @@ constexpr int kNaQueue = 32;
 // Candidates that a thread loads at a time (one at a time waits for L2: 140 us a call at
 // 65,536 particles, 4 threads each; two 116, three 109, four 104. With more threads a row
 // gives each fewer: 4,000 particles, 8 threads each, 50.8 us, three 41.1, four 42.6;
-// 500 particles, 32 threads each, 36.4, 34.8, 36.9).
+// 500 particles, 32 threads each, 36.4, 34.8, 36.9; with a factor of two parts, with the
+// present one 3 % more).
 __host__ __device__ constexpr int na_loads(int T) { return T <= 4 ? 4 : 3; }
 
 template <int T>
