@@ -636,12 +636,12 @@ int Engine::upload_order() {
 
 DevArrays Engine::arrays() const {
   DevArrays a = d_;
-  // Positions in pair units, kept up by the FP64 form with full lists only (and systems in
-  // their range), in memory that
-  // this form has no other use for: the half list's scattered forces, and the gathered
-  // velocities of a rebuild, which copies each slot's velocity back before it writes the
-  // slot's position there. Their own 64 bytes per slot went past the memory that an
-  // arena's capacities promise, and made the arithmetic depend on what was free.
+  // Positions in pair units, kept up by the FP64 form with full lists and systems in their
+  // range, in memory that this form has no other use for: the half list's scattered
+  // forces, and the gathered velocities of a rebuild, which copies each slot's velocity
+  // back before it writes the slot's position there. (64 bytes per slot of their own went
+  // past the memory that an arena's capacities promise, and made the arithmetic depend on
+  // what was free.)
   if (precision_ == 0 && !half_ && n_fixed_ > 0) {
     a.xl[0] = reinterpret_cast<longlong4_32a*>(d_.facc);
     a.xl[1] = reinterpret_cast<longlong4_32a*>(d_.vtmp);

@@ -16,7 +16,7 @@ def _state_lost(ljmd, s):
         assert e.value.code == ljmd.MD_ERR_STATE
 
 
-@pytest.mark.parametrize("polls", [0, 1, 16])
+@pytest.mark.parametrize("polls", [0, 1, 4])
 @pytest.mark.parametrize("nvt", [False, True], ids=["nve", "nvt"])
 @pytest.mark.parametrize("precision", [0, 1], ids=["fp64", "fp32"])
 def test_state_is_lost_and_can_be_set_again(ljmd, precision, nvt, polls):
